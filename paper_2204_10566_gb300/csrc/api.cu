@@ -54,6 +54,10 @@ struct lbm_ctx {
     int32_t *d_tiles = nullptr;      // tile records of the tile fluid kernel
     int2 *d_items = nullptr;         // pairs of fast tiles of the FP16S pair kernel
     int2 *d_rest = nullptr;          // chunks of the other tiles (the chunk kernel beside it)
+    int32_t *d_units = nullptr;      // unit records of the staged FP16S kernel
+    int32_t *d_units_wall = nullptr; // the same without the cells with interpolated walls
+    int64_t n_units_wall = 0;
+    int stage_blocks = 0;            // grid of the staged kernel
     double *d_partials = nullptr;
     double *d_health = nullptr;
     uint32_t *d_status = nullptr;
@@ -141,6 +145,9 @@ void release_wall_q(lbm_ctx *c) {
     dev_free(c, c->d_wnodes, (size_t)c->n_wnodes * 16);
     if (c->d_chunks_wall) dev_free(c, c->d_chunks_wall, c->idx.chunks.size() * 8);
     if (c->d_tiles_wall) dev_free(c, c->d_tiles_wall, (size_t)c->n_tiles_wall * TILE_INTS * 4);
+    if (c->d_units_wall) dev_free(c, c->d_units_wall, (size_t)c->n_units_wall * UNIT_INTS * 4);
+    c->d_units_wall = nullptr;
+    c->n_units_wall = 0;
     if (c->d_items_wall) dev_free(c, c->d_items_wall, (size_t)c->n_items_wall * 8);
     if (c->d_rest_wall) dev_free(c, c->d_rest_wall, (size_t)c->n_rest_wall * 8);
     c->d_items_wall = nullptr;
@@ -167,6 +174,8 @@ void release_geometry(lbm_ctx *c) {
     dev_free(c, c->d_bnodes, c->idx.bnodes.size() * 16);
     dev_free(c, c->d_slot_of_active, c->idx.slot_of_active.size() * 4);
     dev_free(c, c->d_tiles, c->idx.tiles.size() * 4);
+    dev_free(c, c->d_units, c->idx.units.size() * 4);
+    c->d_units = nullptr;
     dev_free(c, c->d_items, c->idx.pair_items.size() * 8);
     dev_free(c, c->d_rest, c->idx.rest_chunks.size() * 8);
     c->d_tiles = nullptr;
@@ -240,6 +249,22 @@ bool tiled(const lbm_ctx *c) {
                         (k == FluidKernel::AUTO && c->desc.precision == LBM_FP32);
     return wanted && c->desc.precision != LBM_FP64 && c->ghost1 && !wide_offsets(c) && tile_count(c) > 0;
 }
+// Whether the next FP16S steps run the staged unit kernel (the same
+// conditions, and STAGE_ROUNDS units for each resident warp; steps with a health check keep the chunk kernel, whose partial
+// sums have a fixed order).
+int64_t unit_count(const lbm_ctx *c) {
+    return c->d_units_wall ? c->n_units_wall : (int64_t)c->idx.units.size() / UNIT_INTS;
+}
+bool staged(const lbm_ctx *c) {
+    const int64_t least = c->fluid_kernel == FluidKernel::STAGED ? 1
+                          : c->fluid_kernel == FluidKernel::AUTO ? (int64_t)STAGE_ROUNDS * c->stage_blocks * (STEP_THREADS / 32)
+                                                                 : INT64_MAX;
+    return c->desc.precision == LBM_FP16S && c->ghost1 && !wide_offsets(c) && c->stage_blocks > 0 &&
+           unit_count(c) >= least;
+}
+// Words of the status allocation (256 bytes): 0 the status, TICKET_WORD and
+// the next the staged kernel's counters, on a cache line of their own.
+constexpr int TICKET_WORD = 32;
 // LBM_FLUID_KERNEL=pairs splits the FP16S fluid cells: pairs of fast tiles
 // run on the pair kernel, the chunks of every other tile on the chunk kernel.
 bool pairs(const lbm_ctx *c) { return c->desc.precision == LBM_FP16S && c->fluid_kernel == FluidKernel::PAIRS; }
@@ -344,6 +369,12 @@ void ctx_step_args(lbm_ctx *c, StepArgs *out) {
             a.nchunks = (int32_t)rest_count(c);
         }
     }
+    if (staged(c)) {
+        a.units = c->d_units_wall ? c->d_units_wall : c->d_units;
+        a.nunits = (int32_t)unit_count(c);
+        a.tickets = reinterpret_cast<int32_t *>(c->d_status) + TICKET_WORD;
+        a.stage_blocks = c->stage_blocks;
+    }
     const int key = (c->ghost1 ? 2 : 0) + (wide ? 1 : 0);
     if (c->prefetch_key != key) {
         c->prefetch_ahead = DISPATCH(c->desc.precision, step_prefetch_ahead, c->ghost1, wide, c->desc.device);
@@ -373,6 +404,8 @@ void ctx_chunk_step_args(lbm_ctx *c, StepArgs *out) {
     out->nbnodes = (int32_t)c->idx.bnodes.size();
     out->tiles = nullptr;
     out->ntiles = 0;
+    out->units = nullptr;
+    out->nunits = 0;
     out->items = nullptr;
     out->nitems = 0;
     out->fluid_blocks = c->fluid_blocks;
@@ -454,11 +487,13 @@ lbm_status lbm_create(const lbm_desc *desc, lbm_ctx **out) {
     const char *wide = std::getenv("LBM_WIDE_OFFSETS");
     c->wide_offsets = wide && wide[0] == '1';
     // LBM_FLUID_KERNEL selects another fluid kernel than the default (FP32:
-    // tile kernel, FP16S / FP64: chunk kernel), for testing every variant on
-    // the same lattices: "chunk", "tile" or "pairs" (FP16S pair + chunk kernel)
+    // tile kernel, FP16S: staged or chunk kernel by size, FP64: chunk kernel),
+    // for testing every variant on the same lattices: "chunk", "tile", "pairs"
+    // (FP16S pair + chunk kernel) or "staged" (FP16S, any size)
     const char *fk = std::getenv("LBM_FLUID_KERNEL");
     if (fk && std::strcmp(fk, "chunk") == 0) c->fluid_kernel = FluidKernel::CHUNK;
     if (fk && std::strcmp(fk, "tile") == 0) c->fluid_kernel = FluidKernel::TILE;
+    if (fk && std::strcmp(fk, "staged") == 0) c->fluid_kernel = FluidKernel::STAGED;
     if (fk && std::strcmp(fk, "pairs") == 0) c->fluid_kernel = FluidKernel::PAIRS;
     lbm_params_default(&c->params);
     {
@@ -562,6 +597,9 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
     const std::vector<int32_t> tiles =
         wn.empty() ? std::vector<int32_t>()
                    : build_tiles(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
+    const std::vector<int32_t> units =
+        wn.empty() ? std::vector<int32_t>()
+                   : build_units(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
     const std::vector<int2> items = build_pair_items(tiles);
     const std::vector<int2> rest = build_rest_chunks(chunks, tiles, items);
     c->d_wall_qidx = (int32_t *)dev_alloc(c, qidx.size() * 4);
@@ -573,6 +611,8 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
     if (!wn.empty()) {
         c->n_tiles_wall = (int64_t)tiles.size() / TILE_INTS;
         c->d_tiles_wall = (int32_t *)dev_alloc(c, tiles.size() * 4);
+        c->n_units_wall = (int64_t)units.size() / UNIT_INTS;
+        c->d_units_wall = (int32_t *)dev_alloc(c, units.size() * 4);
         c->n_items_wall = (int64_t)items.size();
         c->d_items_wall = (int2 *)dev_alloc(c, items.size() * 8);
         c->n_rest_wall = (int64_t)rest.size();
@@ -589,8 +629,8 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
         }
     }
     if (!c->d_wall_qidx || !c->d_wall_q ||
-        (!wn.empty() && (!c->d_wnodes || !c->d_chunks_wall || !c->d_tiles_wall || !c->d_items_wall ||
-                         !c->d_rest_wall)) ||
+        (!wn.empty() && (!c->d_wnodes || !c->d_chunks_wall || !c->d_tiles_wall || !c->d_units_wall ||
+                         !c->d_items_wall || !c->d_rest_wall)) ||
         !partials) {
         release_wall_q(c);
         return fail(c, LBM_ERR_OOM, "wall-distance allocation failed");
@@ -607,6 +647,9 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
     if (!tiles.empty())
         CK(cudaMemcpyAsync(c->d_tiles_wall, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice, c->stream),
            "copy tile records");
+    if (!units.empty())
+        CK(cudaMemcpyAsync(c->d_units_wall, units.data(), units.size() * 4, cudaMemcpyHostToDevice, c->stream),
+           "copy unit records");
     if (!items.empty())
         CK(cudaMemcpyAsync(c->d_items_wall, items.data(), items.size() * 8, cudaMemcpyHostToDevice, c->stream),
            "copy pair items");
@@ -639,7 +682,7 @@ int64_t ctx_footprint(const lbm_desc &d, const HostIndex &ix) {
                                              node_blocks(ix.n_active));
     return 2 * pop + (ix.nslots + 2 * MASK_MARGIN) * 4 + (int64_t)ix.row_nb.size() * 4 + (int64_t)ix.chunks.size() * 8 +
            (int64_t)ix.bnodes.size() * 16 + ix.n_active * 4 + (int64_t)ix.tiles.size() * 4 +
-           (int64_t)ix.pair_items.size() * 8 + (int64_t)ix.rest_chunks.size() * 8 +
+           (int64_t)ix.units.size() * 4 + (int64_t)ix.pair_items.size() * 8 + (int64_t)ix.rest_chunks.size() * 8 +
            blocks * REDUCE_SLOTS * 8 + 64 + 256;
 }
 
@@ -651,6 +694,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     const size_t ns = (size_t)c->idx.nslots;
     c->fluid_blocks = DISPATCH(c->desc.precision, step_fluid_blocks, (int32_t)c->idx.chunks.size());
     c->nblocks = partial_capacity(c, 0);
+    c->stage_blocks = DISPATCH(c->desc.precision, step_stage_blocks, c->desc.device);
     for (int k = 0; k < 2; ++k) {
         c->f_raw[k] = dev_alloc(c, raw_pop_bytes(c));
         c->f[k] = c->f_raw[k] ? static_cast<char *>(c->f_raw[k]) + margin_bytes(c) : nullptr;
@@ -662,13 +706,14 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->d_bnodes = (int4 *)dev_alloc(c, c->idx.bnodes.size() * 16);
     c->d_slot_of_active = (int32_t *)dev_alloc(c, c->idx.slot_of_active.size() * 4);
     c->d_tiles = (int32_t *)dev_alloc(c, c->idx.tiles.size() * 4);
+    c->d_units = (int32_t *)dev_alloc(c, c->idx.units.size() * 4);
     c->d_items = (int2 *)dev_alloc(c, c->idx.pair_items.size() * 8);
     c->d_rest = (int2 *)dev_alloc(c, c->idx.rest_chunks.size() * 8);
     c->d_partials = (double *)dev_alloc(c, (size_t)c->nblocks * REDUCE_SLOTS * 8);
     c->d_health = (double *)dev_alloc(c, 8 * 8);
     c->d_status = (uint32_t *)dev_alloc(c, 256);
     if (!c->f[0] || !c->f[1] || !c->d_mask || !c->d_row_nb || !c->d_chunks || !c->d_bnodes || !c->d_slot_of_active ||
-        !c->d_tiles || !c->d_items || !c->d_rest || !c->d_partials || !c->d_health || !c->d_status) {
+        !c->d_tiles || !c->d_units || !c->d_items || !c->d_rest || !c->d_partials || !c->d_health || !c->d_status) {
         release_geometry(c);
         return fail(c, LBM_ERR_OOM, "device allocation failed in lbm_set_geometry");
     }
@@ -691,6 +736,10 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
         CK(cudaMemcpyAsync(c->d_tiles, c->idx.tiles.data(), c->idx.tiles.size() * 4, cudaMemcpyHostToDevice,
                            c->stream),
            "copy tile records");
+    if (!c->idx.units.empty())
+        CK(cudaMemcpyAsync(c->d_units, c->idx.units.data(), c->idx.units.size() * 4, cudaMemcpyHostToDevice,
+                           c->stream),
+           "copy unit records");
     if (!c->idx.pair_items.empty())
         CK(cudaMemcpyAsync(c->d_items, c->idx.pair_items.data(), c->idx.pair_items.size() * 8,
                            cudaMemcpyHostToDevice, c->stream),
@@ -703,7 +752,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     // that checkpoints and dumps are deterministic.
     CK(cudaMemsetAsync(c->f_raw[0], 0, raw_pop_bytes(c), c->stream), "clear f0");
     CK(cudaMemsetAsync(c->f_raw[1], 0, raw_pop_bytes(c), c->stream), "clear f1");
-    CK(cudaMemsetAsync(c->d_status, 0, 4, c->stream), "clear status");
+    CK(cudaMemsetAsync(c->d_status, 0, 256, c->stream), "clear status");
     CK(cudaStreamSynchronize(c->stream), "sync geometry upload");
     c->has_geom = true;
     c->has_state = false;

@@ -269,9 +269,38 @@ std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int period
         }
     if ((int64_t)out.chunks.size() > (int64_t)INT32_MAX / CHUNK) return "too many chunks";
     out.tiles = build_tiles(out.chunks, out.row_nb, out.mask, F.np, F.pp);
+    out.units = build_units(out.chunks, out.row_nb, out.mask, F.np, F.pp);
     out.pair_items = build_pair_items(out.tiles);
     out.rest_chunks = build_rest_chunks(out.chunks, out.tiles, out.pair_items);
     return "";
+}
+
+std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
+                                 const std::vector<uint32_t> &mask, int n_row, bool periodic_row) {
+    std::vector<int32_t> units;
+    for (size_t k = 0; k < chunks.size();) {
+        const int32_t *nb = &row_nb[(size_t)chunks[k].x * ROW_RECORD_INTS];
+        const int x = (int)((uint32_t)chunks[k].y & CHUNK_X0_MASK);
+        const int p0 = x - (nb[4] + x) % UNIT_ALIGN;  // at most one chunk before the first
+        uint64_t fluid = 0, present = 0;
+        const int row = chunks[k].x;
+        for (; k < chunks.size() && chunks[k].x == row; ++k) {
+            const int x0 = (int)((uint32_t)chunks[k].y & CHUNK_X0_MASK), l = x0 - p0;
+            if (l >= UNIT_CELLS) break;
+            fluid |= (uint64_t)(((uint32_t)chunks[k].y >> CHUNK_LANES_SHIFT) & 0xFFu) << l;
+            present |= (uint64_t)0xFF << l;
+        }
+        bool plain = fluid == ~(uint64_t)0;
+        for (int l = 0; plain && l < UNIT_CELLS; ++l) plain = (mask[(size_t)(nb[4] + p0 + l)] & LINK_MASK) == 0u;
+        const bool wrap = plain && periodic_row && (p0 == 0 || p0 + UNIT_CELLS >= n_row);
+        const uint32_t lo = (uint32_t)__builtin_ctzll(present) / CHUNK, hi = (63u - (uint32_t)__builtin_clzll(present)) / CHUNK;
+        const int32_t head[UNIT_NB] = {p0, (int32_t)(uint32_t)fluid, (int32_t)(uint32_t)(fluid >> 32),
+                                       (int32_t)(uint32_t)present, (int32_t)(uint32_t)(present >> 32),
+                                       (int32_t)(lo | hi << UNIT_HI_SHIFT), (plain ? UNIT_PLAIN : 0) | (wrap ? UNIT_WRAP : 0)};
+        units.insert(units.end(), head, head + UNIT_NB);
+        units.insert(units.end(), nb, nb + 9);
+    }
+    return units;
 }
 
 std::vector<int2> build_pair_items(const std::vector<int32_t> &tiles) {
@@ -508,6 +537,46 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
     }
     for (int64_t b = 0; b < (int64_t)in_tile.size(); ++b)
         if ((flags[b] == LBM_FLUID) != (in_tile[b] == 1)) return "fluid cell not in exactly one tile lane";
+    // Units of the staged kernel: every fluid cell in exactly one fluid lane,
+    // at its own slot, with the bases of its own row; units on a multiple of
+    // UNIT_ALIGN slots; the pieces copied for the present chunks (one chunk
+    // further on either side) inside the buffer margins, their link words
+    // inside theirs; the plain and wrap flags only where they hold.
+    const int64_t nu = (int64_t)ix.units.size() / UNIT_INTS;
+    if ((int64_t)ix.units.size() != nu * UNIT_INTS) return "unit record size";
+    std::vector<uint8_t> in_unit((size_t)nx * ny * nz, 0);
+    for (int64_t u = 0; u < nu; ++u) {
+        const int32_t *rec = &ix.units[(size_t)u * UNIT_INTS];
+        const int32_t *ub = rec + UNIT_NB;
+        const int lo = rec[5] & ((1 << UNIT_HI_SHIFT) - 1), hi = rec[5] >> UNIT_HI_SHIFT;
+        if (lo < 0 || hi < lo || hi > 7 || ((int64_t)ub[4] + rec[0]) % UNIT_ALIGN || rec[0] % CHUNK) return "unit start or pieces";
+        for (int j = 0; j < 9; ++j) {
+            const int64_t first = (int64_t)ub[j] + rec[0] + CHUNK * (lo - 1), end = (int64_t)ub[j] + rec[0] + CHUNK * (hi + 2);
+            if (first < -margin || end > ns + margin) return "unit window outside the buffer";
+        }
+        bool plain = true, ends = false;
+        for (int l = 0; l < UNIT_CELLS; ++l) {
+            const bool fluid = ((uint32_t)rec[1 + l / 32] >> (l % 32)) & 1u, there = ((uint32_t)rec[3 + l / 32] >> (l % 32)) & 1u;
+            const int64_t s = (int64_t)ub[4] + rec[0] + l;
+            if (there && (l / CHUNK < lo || l / CHUNK > hi || s < 0 || s >= ns)) return "unit lane outside its pieces or the buffer";
+            plain = plain && fluid;
+            if (!fluid) continue;
+            if (!there) return "fluid lane of an absent chunk";
+            const int64_t bx = box_of_slot[(size_t)s];
+            if (bx < 0 || flags[bx] != LBM_FLUID || in_unit[(size_t)bx]++) return "unit lane is not a unique fluid cell";
+            int p, a, b;
+            pab_of(bx, p, a, b);
+            if (p != rec[0] + l) return "unit lane position";
+            for (int j = 0; j < 9; ++j)
+                if (ix.row_nb[(size_t)row_e(a, b) * ROW_RECORD_INTS + j] != ub[j]) return "unit bases";
+            plain = plain && !(ix.mask[(size_t)s] & LINK_MASK);
+            ends = ends || (pp && (p == 0 || p == np - 1));
+        }
+        if (plain != ((rec[6] & UNIT_PLAIN) != 0)) return "unit plain flag";
+        if ((plain && ends) != ((rec[6] & UNIT_WRAP) != 0)) return "unit wrap flag";
+    }
+    for (int64_t b = 0; b < (int64_t)in_unit.size(); ++b)
+        if ((flags[b] == LBM_FLUID) != (in_unit[b] == 1)) return "fluid cell not in exactly one unit lane";
     // FP16S split: pairs of fast tiles, each tile in at most one pair; the
     // chunks of the pairs' tiles (four full chunks from p0, on the tile's own
     // row) and the rest chunks together are the chunk list, as a multiset

@@ -278,6 +278,18 @@ __device__ __forceinline__ F2 &operator+=(F2 &a, F2 b) { return a = a + b; }
 __device__ __forceinline__ F2 &operator*=(F2 &a, F2 b) { return a = a * b; }
 __device__ __forceinline__ F2 recip(F2 x) { return F2(make_float2(__frcp_rn(x.v.x), __frcp_rn(x.v.y))); }
 
+// Arithmetic with the rounding written out (no contraction by the compiler),
+// so that one cell per thread (float) and two cells per thread (F2) round
+// alike whatever kernel the code is inlined into.
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ F2 fma_(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ F2 add_(F2 a, F2 b) { return a + b; }
+__device__ __forceinline__ F2 sub_(F2 a, F2 b) { return a - b; }
+__device__ __forceinline__ F2 mul_(F2 a, F2 b) { return a * b; }
+
 // Shared inputs of the per-line inverse (see collide_ghost1).
 struct PairCoef {
     float Axx, Ayy, Azz, Axy, Axz, Ayz, rho_o, drho_o, ux, ux2h, uxh;
@@ -490,6 +502,103 @@ __device__ __forceinline__ void ghost1_finish(const R (&m)[10], R omega, R &rho,
     }
 }
 
+// The FP16S form of the two parts above, for one cell (R = float) or two
+// (R = F2).  ld(i) gives the stored value (f_i - w_i) / in_scale.
+//
+// The moment sums run axis by axis (x within a line, then y, then z), each
+// +-1 pair summed and differenced once: 67 operations.
+template <class R, class Load>
+__device__ __forceinline__ void scaled_sums(const Load &ld, R (&m)[10]) {
+    R t0[3], e0[3], d0[3], t1[3], d1[3], t2[3];  // per cz: sums over cy of s0, s2-in-y, s1-in-y, ...
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        R s0[3], s1[3], s2[3];
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const int j = 3 * (3 * z + y);
+            const R a = ld(j), b = ld(j + 1), c = ld(j + 2);
+            s2[y] = add_(c, a);
+            s0[y] = add_(s2[y], b);
+            s1[y] = sub_(c, a);
+        }
+        e0[z] = add_(s0[2], s0[0]);
+        t0[z] = add_(e0[z], s0[1]);
+        d0[z] = sub_(s0[2], s0[0]);
+        t1[z] = add_(add_(s1[2], s1[0]), s1[1]);
+        d1[z] = sub_(s1[2], s1[0]);
+        t2[z] = add_(add_(s2[2], s2[0]), s2[1]);
+    }
+    m[6] = add_(t0[2], t0[0]);                  // pzz
+    m[0] = add_(m[6], t0[1]);                   // drho
+    m[1] = add_(add_(t1[2], t1[0]), t1[1]);     // jx
+    m[2] = add_(add_(d0[2], d0[0]), d0[1]);     // jy
+    m[3] = sub_(t0[2], t0[0]);                  // jz
+    m[4] = add_(add_(t2[2], t2[0]), t2[1]);     // pxx
+    m[5] = add_(add_(e0[2], e0[0]), e0[1]);     // pyy
+    m[7] = add_(add_(d1[2], d1[0]), d1[1]);     // pxy
+    m[8] = sub_(t1[2], t1[0]);                  // pxz
+    m[9] = sub_(d0[2], d0[0]);                  // pyz
+}
+
+// Relaxation and inverse transform.  With the half coefficients
+//   P0 = rho gz0 + Azz g2z, P1 = Ayz gz1, P2 = Ayy gz0   (cz level)
+//   T = uy^2/2 P0 + uy P1 + P2/2,  O = (uy P0 + P1) / 2  (cy = +-1: +-O)
+// a line's coefficients are Bd = gy0 P0 + gy1 P1 + g2y P2 = w P0 + T +- O and
+// Bw = Bd - wy wz in the form w W0 + T +- O, W0 = rho dz + drho wz + Azz g2z,
+// which has no O(1) cancellation; cy = 0 takes -2 T.  Along x, with
+// u = ux^2/2 Bd + ux B1 + B2/2: f*_0 = 2/3 Bw - 2 u and f*_+- = Bw/6 + u
+// +- (ux Bd + B1)/2.  About 180 operations, against 230 line by line.
+template <class R, class Out>
+__device__ __forceinline__ void scaled_finish(const R (&m)[10], R omega, R &rho, R &ux, R &uy, R &uz, R in_scale,
+                                              R out_scale, const Out &sink) {
+    const R drho = mul_(m[0], in_scale), jx = mul_(m[1], in_scale), jy = mul_(m[2], in_scale), jz = mul_(m[3], in_scale);
+    rho = add_(R(1), drho);
+    const R inv = recip(rho);
+    ux = mul_(jx, inv);
+    uy = mul_(jy, inv);
+    uz = mul_(jz, inv);
+    const R mjx = -jx, mjy = -jy, mth = -theta0<R>();
+    // second-order central Hermite moments p_ab - rho u_a u_b - theta0 drho delta_ab
+    const R a2[6] = {fma_(mjx, ux, fma_(mth, drho, mul_(m[4], in_scale))),
+                     fma_(mjy, uy, fma_(mth, drho, mul_(m[5], in_scale))),
+                     fma_(-jz, uz, fma_(mth, drho, mul_(m[6], in_scale))),
+                     fma_(mjx, uy, mul_(m[7], in_scale)),
+                     fma_(mjx, uz, mul_(m[8], in_scale)),
+                     fma_(mjy, uz, mul_(m[9], in_scale))};
+    sink.moments(omega, a2);
+    const R h = R(0.5), w0 = cst<R>(2, 3), w1_ = cst<R>(1, 6), m2 = R(-2);
+    const R k = mul_(sub_(R(1), omega), out_scale), hk = mul_(h, k);
+    const R ro = mul_(rho, out_scale), dro = mul_(drho, out_scale);
+    const R hAxx = mul_(hk, a2[0]), hAyy = mul_(hk, a2[1]), hAzz = mul_(hk, a2[2]), nAzz = mul_(m2, hAzz);
+    const R hAxy = mul_(hk, a2[3]), hAxz = mul_(hk, a2[4]), hAyz = mul_(hk, a2[5]);
+    const R hux = mul_(h, ux), huy = mul_(h, uy), huz = mul_(h, uz);
+    const R ux2h = mul_(hux, ux), uy2h = mul_(huy, uy), uz2h = mul_(huz, uz);
+    const R u2x = mul_(R(2), ux), u2y = mul_(R(2), uy);
+    const R gy0[3] = {add_(w1_, sub_(uy2h, huy)), fma_(m2, uy2h, w0), add_(w1_, add_(uy2h, huy))};
+    const R gy1[3] = {sub_(uy, h), mul_(m2, uy), add_(uy, h)};
+    const R Y1 = fma_(dro, w1_, hAzz), Y0 = fma_(dro, w0, nAzz);
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        const R dz = z == 0 ? sub_(uz2h, huz) : (z == 1 ? mul_(m2, uz2h) : add_(uz2h, huz));
+        const R gz0 = add_(z == 1 ? w0 : w1_, dz);
+        const R gz1 = z == 0 ? sub_(uz, h) : (z == 1 ? mul_(m2, uz) : add_(uz, h));
+        const R P0 = fma_(ro, gz0, z == 1 ? nAzz : hAzz), W0 = fma_(ro, dz, z == 1 ? Y0 : Y1);
+        const R hP1 = mul_(hAyz, gz1), hP2 = mul_(hAyy, gz0);
+        const R hQ0 = mul_(hAxz, gz1), hQ1 = mul_(hAxy, gz0), hR0 = mul_(hAxx, gz0);
+        const R T = fma_(uy2h, P0, fma_(u2y, hP1, hP2)), O = fma_(huy, P0, hP1), n2T = mul_(m2, T);
+        const R e1 = fma_(w1_, W0, T), e2 = fma_(w1_, P0, T);
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const R Bw = y == 0 ? sub_(e1, O) : (y == 1 ? fma_(w0, W0, n2T) : add_(e1, O));
+            const R Bd = y == 0 ? sub_(e2, O) : (y == 1 ? fma_(w0, P0, n2T) : add_(e2, O));
+            const R hB1 = fma_(gy0[y], hQ0, mul_(gy1[y], hQ1)), hB2 = mul_(gy0[y], hR0);
+            const R u = fma_(ux2h, Bd, fma_(u2x, hB1, hB2));
+            const R A = fma_(hux, Bd, hB1), S = fma_(w1_, Bw, u);
+            sink(3 * z + y, sub_(S, A), fma_(m2, u, mul_(w0, Bw)), add_(S, A));
+        }
+    }
+}
+
 // Collision with the default ghost rates (all 1).  d holds f_i - w_i on entry;
 // the post-collision f*_i - w_i go to the sink line by line, or back into d
 // without one.  rho, u receive the (conserved) moments.  With SCALED, d holds
@@ -498,11 +607,16 @@ template <class R, bool SCALED = false, class Out = ToArray<R>>
 __device__ __forceinline__ void collide_ghost1(R (&d)[27], R omega, R &rho, R &ux, R &uy, R &uz,
                                                R in_scale = R(1), R out_scale = R(1), const Out *sink = nullptr) {
     R m[10];
-    ghost1_sums(d, SameInput{}, m);
-    if (sink)
-        ghost1_finish<R, SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, *sink);
-    else
-        ghost1_finish<R, SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, ToArray<R>{d});
+    if constexpr (SCALED) {
+        scaled_sums<R>([&](int i) { return d[i]; }, m);
+        scaled_finish<R>(m, omega, rho, ux, uy, uz, in_scale, out_scale, *sink);
+    } else {
+        ghost1_sums(d, SameInput{}, m);
+        if (sink)
+            ghost1_finish<R, SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, *sink);
+        else
+            ghost1_finish<R, SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, ToArray<R>{d});
+    }
 }
 
 // 1-D forward central Hermite factor h_k(c - u): 1, c - u, (c - u)^2 - theta0.
@@ -1404,8 +1518,8 @@ __device__ __forceinline__ void pair_update(const StepArgs &a, int t, int k, dou
     __half2 d[27];
     gather_pair<AX>(a, nb, x, d);
     F2 m[10], rho, ux, uy, uz;
-    ghost1_sums(d, Half2ToF2{}, m);
-    ghost1_finish<F2, true>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale), PairStore{a, slot});
+    scaled_sums<F2>([&](int i) { return Half2ToF2{}(d[i]); }, m);
+    scaled_finish<F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale), PairStore{a, slot});
     double h0[6] = {0, 0, 0, 0, 0, 0}, h1[6] = {0, 0, 0, 0, 0, 0};
     record_cell(a, slot, rho.v.x, ux.v.x, uy.v.x, uz.v.x, h0);
     record_cell(a, slot + 1, rho.v.y, ux.v.y, uy.v.y, uz.v.y, h1);
@@ -1428,6 +1542,279 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_PAIR_MIN_BLOCKS) k_step_pair
         pair_update<AX>(a, lane < 16 ? item.x : item.y, lane & 15, hv);
     }
     if (a.flags & STEP_REDUCE) block_reduce_write(hv, a.partials);
+}
+
+// ------------------------------------------------ staged unit kernel (FP16S)
+//
+// The FP16S fluid kernel of larger lattices: persistent warps over units of
+// up to 64 cells of a row.  In FP16S a step moves half the bytes of FP32 for
+// the same work, so what bounds a one-cell-per-thread kernel is not HBM but
+// the loads a warp can have in flight in its registers (long-scoreboard waits
+// were 6.5 of the 12.1 cycles between a warp's issues) and its 700
+// instructions per cell.  Here each warp copies the pull windows of its next
+// unit (27 arrays, 64 cells and one 16-byte piece on the side they pull from)
+// into its own shared-memory stages, nine 16-byte cp.async per lane, while it
+// computes the current one, so its loads in flight do not depend on registers
+// or on other warps.  Each thread updates two adjacent cells on the packed
+// FP32 pipe, one instruction stream for every unit (the output sink alone
+// tells plain units, 64 fluid cells without wall links, from the others).
+//
+// Measured per step, before (chunk kernel) and now: Re 6500 nozzle 448 ->
+// 339 us (4.61 TB/s of algorithmic bytes), Re 3500 nozzle 150 -> 126 us,
+// periodic 256^3 515 -> 349 us (5.20 TB/s).  Two stages and 4 blocks of 4
+// warps per SM: 3 blocks 361 us on the Re 6500 nozzle, 5 blocks (96
+// registers, no spills) 395 us, three stages 347 us; more bytes in flight
+// only widen the span of the arrays that is open at a time.
+#ifndef LBM_STAGE_DEPTH
+#define LBM_STAGE_DEPTH 2
+#endif
+#ifndef LBM_STAGE_BLOCKS
+#define LBM_STAGE_BLOCKS 4
+#endif
+#ifndef LBM_STAGE_RUN
+#define LBM_STAGE_RUN 3
+#endif
+constexpr int STAGE_SHORT = 6;                       // lists of fewer rounds are handed out by position
+constexpr int STAGE_DEPTH = LBM_STAGE_DEPTH;
+constexpr int STAGE_RUN = LBM_STAGE_RUN;             // units per ticket
+constexpr int STAGE_WINDOW = 160;                    // bytes of one population's window: 128 + 2 x 16
+constexpr int STAGE_MASK = 27 * STAGE_WINDOW;        // windows in (line, c_row) order, then the link words
+constexpr int STAGE_REC = STAGE_MASK + 64 * 4;       // and the unit's record
+constexpr int STAGE_BYTES = STAGE_REC + UNIT_INTS * 4;
+constexpr int STAGE_WARPS = STEP_THREADS / 32;
+constexpr int STAGE_SMEM = STAGE_WARPS * STAGE_DEPTH * STAGE_BYTES;
+
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Byte offset, in a stage, of population i's value for the cell at unit
+// position 0: its window, 16 bytes in, shifted by the pull.
+template <int AX>
+__host__ __device__ constexpr int stage_offset(int i) {
+    return (row_line<AX>(i) * 3 + c_row<AX>(i) + 1) * STAGE_WINDOW + 16 - 2 * c_row<AX>(i);
+}
+
+// Start the copies of a unit (rec: lane l holds word l of its record) into a
+// stage: the pull windows, lane 10 k + q copying piece q of the c_row = k - 1
+// population of each line; the link words, unless the unit is plain; and the
+// record.  lane_src is fin plus the lane's part of the element offset.
+template <int AX>
+__device__ __forceinline__ void stage_issue(const StepArgs &a, int rec, char *stage, uint32_t dst,
+                                            const char *lane_src, int lane) {
+    const int p0 = __shfl_sync(0xffffffffu, rec, 0);
+    const int pieces = __shfl_sync(0xffffffffu, rec, 5), flags = __shfl_sync(0xffffffffu, rec, 6);
+    // pieces needed: the present chunks lo .. hi, one position further on the
+    // side that c_row pulls from
+    const int lo = pieces & ((1 << UNIT_HI_SHIFT) - 1), hi = pieces >> UNIT_HI_SHIFT;
+    const int k = lane / 10, q = lane % 10;
+    const bool on = lane < 30 && q >= (k == 2 ? lo : lo + 1) && q <= (k == 0 ? hi + 2 : hi + 1);
+    const uint32_t lane_dst = dst + (k * STAGE_WINDOW + 16 * q);
+    const int64_t line_stride = (AX == 0 ? 3 : 1) * a.stride;
+    int own = 0;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+        const int nb = __shfl_sync(0xffffffffu, rec, UNIT_NB + j);
+        if (j == 4) own = nb;
+        if (on) copy16(lane_dst + j * 3 * STAGE_WINDOW, lane_src + 2 * (j * line_stride + (int64_t)(nb + p0)));
+    }
+    if (!(flags & UNIT_PLAIN) && lane >= 2 * lo && lane <= 2 * hi + 1)
+        copy16(dst + STAGE_MASK + 16 * lane, a.mask + (own + p0 + 4 * lane));
+    if (lane < UNIT_INTS) *reinterpret_cast<int *>(stage + STAGE_REC + 4 * lane) = rec;
+}
+
+// Output sink of a unit: the adjacent cells x (first half of each value) and
+// x + 1 of a thread.  A plain unit stores both cells of each population as
+// one 32-bit word; otherwise each cell has its own-slot predicates (bit i of
+// own; OWN_FLUID marks a fluid cell), its wall links' ghost slots and its
+// wrap-around copies, as LineStore has for one cell.  plain and wrap are
+// uniform over the warp.  nb: the neighbour bases in shared memory.
+template <int AX>
+struct UnitStore {
+    const StepArgs &a;
+    const int *nb;
+    int x, slot;
+    bool plain, wrap;
+    uint32_t links[2], both, own[2];  // both: own of both cells; own: of one cell only
+    uint32_t fluid;                   // bit h: cell x + h is a fluid cell
+    __device__ __forceinline__ void moments(F2 omega, const F2 (&a2)[6]) const {
+        if ((a.flags & (STEP_STATS | STEP_STATS_FULL)) != (STEP_STATS | STEP_STATS_FULL)) return;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float s[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) s[q] = h ? a2[q].v.y : a2[q].v.x;
+            if (fluid & (1u << h)) record_stress(a, slot + h, h ? omega.v.y : omega.v.x, s);
+        }
+    }
+    __device__ __forceinline__ void put(int i, int s, __half v) const {
+        static_cast<__half *>(a.fout)[elem<false>(i, a.stride, s)] = v;
+    }
+    __device__ __forceinline__ void operator()(int j, F2 vm, F2 v0, F2 vp) const {
+        const __half2 v[3] = {__float22half2_rn(vm.v), __float22half2_rn(v0.v), __float22half2_rn(vp.v)};
+        __half *out = static_cast<__half *>(a.fout);
+        const uint32_t st = (uint32_t)a.stride;
+        __half *pj = out + ((uint32_t)(3 * j) * st + (uint32_t)slot);
+        __half *p[3] = {pj, pj + st, pj + 2 * st};
+        if (plain) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) *reinterpret_cast<__half2 *>(p[c]) = v[c];
+        } else {
+            const int jl = 8 - j;  // links 26 - i of this line's values sit in line 8 - j
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (both & (1u << (3 * j + c))) *reinterpret_cast<__half2 *>(p[c]) = v[c];
+            if ((own[0] | own[1]) & (7u << (3 * j))) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    if (own[0] & (1u << (3 * j + c))) p[c][0] = __low2half(v[c]);
+                    if (own[1] & (1u << (3 * j + c))) p[c][1] = __high2half(v[c]);
+                }
+            }
+            if ((links[0] | links[1]) & (7u << (3 * jl))) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const int k = 26 - (3 * j + c);  // wall link k takes value 3j + c
+                    const int s = nb[row_line<AX>(k)] + x - c_row<AX>(k);
+                    if (links[0] & (1u << k)) put(k, s, __low2half(v[c]));
+                    if (links[1] & (1u << k)) put(k, s + 1, __high2half(v[c]));
+                }
+            }
+        }
+        if (wrap) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (!(fluid & (1u << h))) continue;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const int i = 3 * j + c;
+                    const __half w = h ? __high2half(v[c]) : __low2half(v[c]);
+                    if (c_row<AX>(i) == 1 && x + h == a.n_row - 1) put(i, nb[4] - 1, w);
+                    if (c_row<AX>(i) == -1 && x + h == 0) put(i, nb[4] + a.n_row, w);
+                }
+            }
+        }
+    }
+};
+
+// Update of the unit in a stage: two adjacent cells per thread.
+template <int AX>
+__device__ __forceinline__ void stage_update(const StepArgs &a, const char *st, int lane) {
+    const int *rec = reinterpret_cast<const int *>(st + STAGE_REC);
+    const int x = rec[0] + 2 * lane, slot = rec[UNIT_NB + 4] + x;
+    UnitStore<AX> sink{a, rec + UNIT_NB, x, slot, (rec[6] & UNIT_PLAIN) != 0, (rec[6] & UNIT_WRAP) != 0,
+                       {0u, 0u}, 0u, {0u, 0u}, 3u};
+    if (!sink.plain) {
+        const uint2 mk2 = *reinterpret_cast<const uint2 *>(st + STAGE_MASK + 8 * lane);  // not copied where absent
+        const uint32_t fl = (uint32_t)rec[1 + (lane >> 4)] >> (2 * (lane & 15));
+        const uint32_t pr = (uint32_t)rec[3 + (lane >> 4)] >> (2 * (lane & 15));
+        uint32_t own[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t mk = h ? mk2.y : mk2.x;
+            const bool fluid = (fl >> h) & 1u;
+            sink.links[h] = fluid ? (mk & LINK_MASK) : 0u;
+            own[h] = fluid ? LINK_MASK
+                           : (((pr >> h) & 1u) && ((mk >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~mk & LINK_MASK) : 0u);
+        }
+        sink.both = own[0] & own[1];
+        sink.own[0] = own[0] & ~own[1];
+        sink.own[1] = own[1] & ~own[0];
+        sink.fluid = fl & 3u;
+        sink.wrap = a.periodic_row != 0;
+    }
+    const char *sl = st + 4 * lane;
+    auto ld = [&](int i) {
+        const char *p = sl + stage_offset<AX>(i);
+        if (c_row<AX>(i) == 0) return F2(__half22float2(*reinterpret_cast<const __half2 *>(p)));
+        return F2(make_float2(__half2float(*reinterpret_cast<const __half *>(p)),
+                              __half2float(*reinterpret_cast<const __half *>(p + 2))));
+    };
+    F2 m[10], rho, ux, uy, uz;
+    scaled_sums<F2>(ld, m);
+    scaled_finish<F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale), sink);
+    if (a.flags & STEP_STATS) {
+        double hv[6];
+        if (sink.fluid & 1u) record_cell(a, slot, rho.v.x, ux.v.x, uy.v.x, uz.v.x, hv);
+        if (sink.fluid & 2u) record_cell(a, slot + 1, rho.v.y, ux.v.y, uy.v.y, uz.v.y, hv);
+    }
+}
+
+// The units a warp takes: runs of STAGE_RUN consecutive units from the work
+// counter (one address takes an atomic about every 2 ns: single-unit runs
+// throughout take 551 us a step on the Re 6500 nozzle, runs of three 339 us),
+// and single ones over the last two rounds of the warps, so that they finish
+// together.  The next ticket is drawn while the current run is handed out.
+struct UnitQueue {
+    int32_t *counter;
+    int n, n_long, pos, end, ticket;
+    __device__ __forceinline__ UnitQueue(int32_t *counter_, int n_, int warps)
+        : counter(counter_), n(n_), n_long(max(0, n_ - 2 * warps) / STAGE_RUN), pos(0), end(0), ticket(0) {}
+    __device__ __forceinline__ void draw(int lane) { ticket = lane == 0 ? atomicAdd(counter, 1) : 0; }
+    __device__ __forceinline__ int next(int lane) {  // -1 when none is left
+        if (pos >= end) {
+            const int t = __shfl_sync(0xffffffffu, ticket, 0);
+            pos = t < n_long ? t * STAGE_RUN : n_long * STAGE_RUN + (t - n_long);
+            end = pos + (t < n_long ? STAGE_RUN : 1);
+            if (pos >= n) {
+                end = pos;
+                return -1;  // and at every later call: the ticket stays past the end
+            }
+            draw(lane);
+        }
+        return pos++;
+    }
+};
+
+template <int AX>
+__global__ void __launch_bounds__(STEP_THREADS, LBM_STAGE_BLOCKS) k_step_units(const StepArgs a) {
+    extern __shared__ __align__(16) char stages[];
+    const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    char *base = stages + warp * (STAGE_DEPTH * STAGE_BYTES);
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(base);
+    const int k = lane / 10, q = lane % 10;
+    const char *lane_src = static_cast<const char *>(a.fin) + 2 * ((AX == 0 ? k : 9 * k) * a.stride + 8 * q - 8);
+    UnitQueue queue(a.tickets, a.nunits, (int)gridDim.x * STAGE_WARPS);
+    queue.draw(lane);
+    constexpr int NONE = -1;  // as word 0 of a record: no unit (p0 is a multiple of CHUNK)
+    auto fetch = [&]() {
+        const int u = queue.next(lane);
+        return u < 0 ? NONE : __ldg(a.units + (size_t)u * UNIT_INTS + (lane & (UNIT_INTS - 1)));
+    };
+    auto there = [&](int r) { return __shfl_sync(0xffffffffu, r, 0) != NONE; };  // uniform
+    int in_flight = 0;  // units being copied or ready
+    int ahead = fetch();
+#pragma unroll
+    for (int s = 0; s < STAGE_DEPTH - 1; ++s) {
+        if (there(ahead)) {
+            stage_issue<AX>(a, ahead, base + s * STAGE_BYTES, sbase + s * STAGE_BYTES, lane_src, lane);
+            ++in_flight;
+            ahead = fetch();
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int cur = 0;  // stage of the current unit
+    while (in_flight > 0) {
+        if (there(ahead)) {  // into the stage read in the last round
+            const int s = cur == 0 ? STAGE_DEPTH - 1 : cur - 1;
+            stage_issue<AX>(a, ahead, base + s * STAGE_BYTES, sbase + s * STAGE_BYTES, lane_src, lane);
+            ++in_flight;
+            ahead = fetch();
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGE_DEPTH - 1) : "memory");
+        __syncwarp();
+        stage_update<AX>(a, base + cur * STAGE_BYTES, lane);
+        __syncwarp();  // every lane is done with the stage before it is refilled
+        --in_flight;
+        cur = cur == STAGE_DEPTH - 1 ? 0 : cur + 1;
+    }
+    // the last block to finish clears the counters for the next launch
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.tickets + 1, 1) == (int)gridDim.x - 1) {
+        a.tickets[0] = 0;
+        a.tickets[1] = 0;
+    }
 }
 
 // ---------------------------------------------------------- utility kernels
@@ -1615,6 +2002,22 @@ int step_fluid_blocks(int32_t nchunks) {
 }
 
 template <int P>
+int step_stage_blocks(int device) {
+    if constexpr (P == 2) {
+        int per_sm = 0, sms = 0;
+        cudaError_t e = cudaFuncSetAttribute(k_step_units<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_step_units<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_SMEM);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_units<2>, STEP_THREADS, STAGE_SMEM);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+        if (e == cudaSuccess) return per_sm * sms;
+        cudaGetLastError();
+    }
+    return 0;
+}
+
+template <int P>
 int step_prefetch_ahead(bool ghost1, bool wide, int device) {
     int per_sm = 0, sms = 0;
     cudaError_t e;
@@ -1655,6 +2058,7 @@ template <int P, bool G, bool WD, int AX>
 cudaError_t launch_step_ax(const StepArgs &a, cudaStream_t s, const SideStream *side, int &launches) {
     const int bb = (int)((a.nbnodes + STEP_THREADS - 1) / STEP_THREADS);
     const bool tiled = G && !WD && P != 0 && a.tiles != nullptr;
+    bool fluid_done = false;
     const bool fused = !tiled && LBM_FUSE_BOUNDARY && P == 1 && a.nchunks > 0;  // nodes in trailing blocks of k_step
     const bool nodes = a.nwnodes > 0 || (bb > 0 && !fused);
     const bool aside = nodes && side && side->stream;
@@ -1690,7 +2094,15 @@ cudaError_t launch_step_ax(const StepArgs &a, cudaStream_t s, const SideStream *
             }
         }
     }
-    if (!tiled && a.nchunks > 0) {
+    if constexpr (P == 2 && G && !WD) {
+        if (a.units && !(a.flags & STEP_REDUCE)) {
+            const int blocks = std::min(a.stage_blocks, (a.nunits + STAGE_WARPS - 1) / STAGE_WARPS);
+            k_step_units<AX><<<blocks, STEP_THREADS, STAGE_SMEM, s>>>(a);
+            ++launches;
+            fluid_done = true;
+        }
+    }
+    if (!tiled && !fluid_done && a.nchunks > 0) {
         k_step<P, G, WD, AX><<<step_blocks(a.nchunks) + (fused ? bb : 0), STEP_THREADS, 0, s>>>(a);
         ++launches;
     }
@@ -1794,6 +2206,7 @@ cudaError_t launch_init_eq(void *f, const int32_t *soa, int64_t n, int64_t strid
 #define LBM_INSTANTIATE(P)                                                                                         \
     template cudaError_t launch_step<P>(const StepArgs &, bool, cudaStream_t, int *, const SideStream *);                                     \
     template int step_fluid_blocks<P>(int32_t);                                                                     \
+    template int step_stage_blocks<P>(int);                                                                         \
     template int step_prefetch_ahead<P>(bool, bool, int);                                                          \
     template cudaError_t launch_reduce<P>(const void *, const int32_t *, int64_t, int64_t, float, double *,       \
                                           cudaStream_t);                                                           \

@@ -105,9 +105,36 @@ std::vector<int2> build_pair_items(const std::vector<int32_t> &tiles);
 std::vector<int2> build_rest_chunks(const std::vector<int2> &chunks, const std::vector<int32_t> &tiles,
                                     const std::vector<int2> &pairs);
 
+// Unit records of the staged FP16S fluid kernel: a unit is the chunks of one
+// row within the UNIT_CELLS positions from p0, 128 bytes of every FP16
+// population array.  Units start on a multiple of UNIT_ALIGN slots, one
+// 32-byte sector, whatever the alignment of the row (on the Re 3500 nozzle,
+// whose rows all start half way into a sector, units from the row's first
+// chunk on take 162 us a step, aligned ones 125 us; aligning to whole lines
+// gains nothing more).  A record holds p0 (possibly one chunk before the
+// row's first), the fluid-lane and the present-lane masks (64 bits each, low
+// word first), the first and the last present chunk, the flags UNIT_PLAIN (64
+// fluid cells, none with a wall link) and UNIT_WRAP (plain, with a row end
+// that writes wrap-around copies), and the row's nine neighbour bases: 64
+// bytes.
+constexpr int UNIT_ALIGN = 16;
+constexpr int UNIT_CELLS = 64;
+constexpr int UNIT_INTS = 16;
+constexpr int UNIT_NB = 7;  // first of the nine neighbour bases in a record
+constexpr int UNIT_HI_SHIFT = 8;
+constexpr int UNIT_PLAIN = 1, UNIT_WRAP = 2;
+// The staged kernel takes over from the chunk kernel at this many units per
+// resident warp (about 0.9 M cells): its warps start and end on atomics of one
+// address, a few us a launch.  At 4.4 rounds (96^3) it takes 36.5 us against
+// the chunk kernel's 34.6, at 13.5 rounds (128^3) 59.5 against 69.7.
+constexpr int STAGE_ROUNDS = 6;
+std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
+                                 const std::vector<uint32_t> &mask, int n_row, bool periodic_row);
+
 // Fluid kernel of the FP32 / FP16S steps: AUTO is the tile kernel in FP32
-// and the chunk kernel in FP16S; the others are kept for testing.
-enum class FluidKernel { AUTO, CHUNK, TILE, PAIRS };
+// and, in FP16S, the staged unit kernel for larger lattices and the chunk
+// kernel for smaller ones; the others are kept for testing.
+enum class FluidKernel { AUTO, CHUNK, TILE, PAIRS, STAGED };
 
 // A second stream and its fork / join events: a step's wall-cell and
 // inlet/outlet kernels run on it beside the fluid kernel.  They read the
@@ -160,6 +187,10 @@ struct alignas(16) StepArgs {
     int32_t wide_offsets;      // 1: 64-bit element offsets even when 32 bits would do (LBM_WIDE_OFFSETS=1)
     const int32_t *tiles;      // tile records of the tile fluid kernels (NULL: chunk kernel)
     int32_t ntiles;
+    const int32_t *units;      // unit records of the staged FP16S fluid kernel (NULL: chunk kernel)
+    int32_t nunits;
+    int32_t *tickets;          // its work counter and its count of finished warps, both 0 between launches
+    int32_t stage_blocks;      // its grid: the blocks resident on the device at once
     const int2 *items;         // FP16S pairs of fast tiles (NULL: tile kernel); chunks then holds the rest
     int32_t nitems;
 };
@@ -176,6 +207,10 @@ cudaError_t launch_step(const StepArgs &a, bool ghost1, cudaStream_t s, int *lau
 // blocks resident on the device at once (occupancy x SM count); 0 = off.
 template <int P>
 int step_prefetch_ahead(bool ghost1, bool wide, int device);
+// Blocks of the staged unit kernel that are resident on the device at once
+// (0 if it has none for this precision).
+template <int P>
+int step_stage_blocks(int device);
 // Blocks of one step's fluid kernel (partial-sum slots it writes).
 template <int P>
 int step_fluid_blocks(int32_t nchunks);
@@ -226,6 +261,7 @@ struct HostIndex {
     std::vector<int32_t> row_nb;          // [rows][ROW_RECORD_INTS]
     std::vector<int2> chunks;             // chunk records (fluid cells)
     std::vector<int32_t> tiles;           // [tiles][TILE_INTS] records of the tile fluid kernels
+    std::vector<int32_t> units;           // [units][UNIT_INTS] records of the staged FP16S fluid kernel
     std::vector<int2> pair_items;         // pairs of fast tiles, for the FP16S pair kernel
     std::vector<int2> rest_chunks;        // chunks of the other tiles, for the chunk kernel beside it
     std::vector<int4> bnodes;             // inlet/outlet nodes: x, row, slot, link word
@@ -236,7 +272,7 @@ struct HostIndex {
 
 // Slack (elements) allocated before and after every population buffer and
 // around the link-word array (keeps 256-byte alignment of the buffers).
-inline int64_t buffer_margin(int nx) { return ((int64_t)nx + 64 + 63) & ~(int64_t)63; }
+inline int64_t buffer_margin(int nx) { return ((int64_t)nx + 128 + 63) & ~(int64_t)63; }
 constexpr int64_t MASK_MARGIN = 64;
 
 // Returns "" on success, else a description of the inconsistency.  With
