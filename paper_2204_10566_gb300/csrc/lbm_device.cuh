@@ -252,7 +252,15 @@ __device__ __forceinline__ void record_stress(const StepArgs &a, int slot, R ome
 // --------------------------------------------------------------- collision
 
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// 1/x from the hardware's approximation x0 (about 20 bits) and one
+// third-order step, x0 (1 + e + e^2) with e = 1 - x x0, whose remainder e^3 is
+// below rounding: four FP64 operations.
+__device__ __forceinline__ double recip(double x) {
+    double x0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(x));
+    const double e = __fma_rn(-x, x0, 1.0);
+    return __fma_rn(x0, __fma_rn(e, e, e), x0);
+}
 
 // Packed FP32 (two values per instruction, sm_100 and later) for the inverse
 // transform of the rate-1 collision.  Off: -DLBM_PACKED_F32=0.
@@ -285,6 +293,10 @@ __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf
 __device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ F2 fma_(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 __device__ __forceinline__ F2 add_(F2 a, F2 b) { return a + b; }
 __device__ __forceinline__ F2 sub_(F2 a, F2 b) { return a - b; }
@@ -503,7 +515,8 @@ __device__ __forceinline__ void ghost1_finish(const R (&m)[10], R omega, R &rho,
 }
 
 // The FP16S form of the two parts above, for one cell (R = float) or two
-// (R = F2).  ld(i) gives the stored value (f_i - w_i) / in_scale.
+// (R = F2).  ld(i) gives the stored value (f_i - w_i) / in_scale (FP64 takes
+// the sums too).
 //
 // The moment sums run axis by axis (x within a line, then y, then z), each
 // +-1 pair summed and differenced once: 67 operations.
@@ -599,6 +612,102 @@ __device__ __forceinline__ void scaled_finish(const R (&m)[10], R omega, R &rho,
     }
 }
 
+// The FP64 form of the second part.  FP64 is bound by its arithmetic pipe, so
+// this form is the one with the fewest operations: the post-collision state
+// is written in raw moments M_abc = sum c_x^a c_y^b c_z^c (f* - w) / 2^n, n
+// the number of non-zero exponents, whose inverse is three operations a line
+// (f*_+- = M_2 +- M_1, f*_0 = M_0 - 2 M_2) and holds no velocity.  With the
+// 1-D moments (1, u, u^2 + theta) of the equilibrium factor and (0, 1, 2 u)
+// of a first-order column, the 27 moments follow from rho, u and the relaxed
+// second-order central moments A_ab = (1 - omega) a_ab, each from the ones
+// of lower order:
+//   p*_ab = p_ab - omega a_ab;  M(xxy) = u_y P_xx + 2 u_x A_xy, P = p* + theta;
+//   M(xyz) = u_z p*_xy + u_y A_xz + u_x A_yz;
+//   M(xxyy) = p*_xx E_y + A_yy E_x + 4 u_x u_y A_xy + theta u_y^2, E = u^2 + theta;
+//   M(xxyz) = u_z M(xxy) + 2 u_x u_y A_xz + A_yz E_x;
+//   M(xxyyz) = u_z (M(xxyy) + theta^2) + 2 u_x A_xz E_y + 2 u_y A_yz E_x; ...
+// 254 FP64 instructions a cell with the moment sums, against about 390 for
+// the line-by-line inverse; at the pipe's 86-87 % either way, the Re 3500
+// nozzle's step takes 2.09 ms instead of 3.12 ms (1 372 -> 2 050 MLUPS).
+template <class R, class Out>
+__device__ __forceinline__ void raw_finish(const R (&m)[10], R omega, R &rho, R &ux, R &uy, R &uz, const Out &sink) {
+    const R drho = m[0], jx = m[1], jy = m[2], jz = m[3], th = theta0<R>(), h = R(0.5), q = R(0.25), m2 = R(-2);
+    rho = add_(R(1), drho);
+    const R inv = recip(rho);
+    ux = mul_(jx, inv);
+    uy = mul_(jy, inv);
+    uz = mul_(jz, inv);
+    const R a2[6] = {fma_(-jx, ux, fma_(-th, drho, m[4])), fma_(-jy, uy, fma_(-th, drho, m[5])),
+                     fma_(-jz, uz, fma_(-th, drho, m[6])), fma_(-jx, uy, m[7]),
+                     fma_(-jx, uz, m[8]),                  fma_(-jy, uz, m[9])};
+    sink.moments(omega, a2);
+    const R k = sub_(R(1), omega), hk = mul_(h, k);
+    const R Axy = mul_(k, a2[3]), Axz = mul_(k, a2[4]), Ayz = mul_(k, a2[5]);
+    const R hAyy = mul_(hk, a2[1]), hAzz = mul_(hk, a2[2]);
+    const R qAxy = mul_(q, Axy), qAxz = mul_(q, Axz), qAyz = mul_(q, Ayz);
+    const R hx = mul_(h, ux), hy = mul_(h, uy), hz = mul_(h, uz), u2y = add_(uy, uy), u2z = add_(uz, uz);
+    const R sx = mul_(ux, ux), sy = mul_(uy, uy), sz = mul_(uz, uz);
+    const R Ex = fma_(h, sx, R(h * th)), Ey = fma_(h, sy, R(h * th)), Ez = fma_(h, sz, R(h * th));
+    const R ty = mul_(R(q * th), sy), tz = mul_(R(q * th), sz), t2 = R(q * th * th);
+    const R kx_y = mul_(hx, Axy), ky_x = mul_(hy, Axy), kx_z = mul_(hx, Axz), kz_x = mul_(hz, Axz),
+            ky_z = mul_(hy, Ayz), kz_y = mul_(hz, Ayz);
+    R M[3][3][3];  // [a][b][c]
+    M[0][0][0] = drho;
+    M[1][0][0] = mul_(h, jx);
+    M[0][1][0] = mul_(h, jy);
+    M[0][0][1] = mul_(h, jz);
+    M[2][0][0] = mul_(h, fma_(-omega, a2[0], m[4]));
+    M[0][2][0] = mul_(h, fma_(-omega, a2[1], m[5]));
+    M[0][0][2] = mul_(h, fma_(-omega, a2[2], m[6]));
+    M[1][1][0] = mul_(q, fma_(-omega, a2[3], m[7]));
+    M[1][0][1] = mul_(q, fma_(-omega, a2[4], m[8]));
+    M[0][1][1] = mul_(q, fma_(-omega, a2[5], m[9]));
+    const R Qxx = add_(M[2][0][0], R(h * th)), Qyy = add_(M[0][2][0], R(h * th)), Qzz = add_(M[0][0][2], R(h * th));
+    M[2][1][0] = fma_(hy, Qxx, kx_y);
+    M[2][0][1] = fma_(hz, Qxx, kx_z);
+    M[1][2][0] = fma_(hx, Qyy, ky_x);
+    M[0][2][1] = fma_(hz, Qyy, ky_z);
+    M[1][0][2] = fma_(hx, Qzz, kz_x);
+    M[0][1][2] = fma_(hy, Qzz, kz_y);
+    M[1][1][1] = fma_(hz, M[1][1][0], fma_(hy, qAxz, mul_(hx, qAyz)));
+    M[2][2][0] = fma_(M[2][0][0], Ey, fma_(hAyy, Ex, fma_(u2y, kx_y, ty)));
+    M[2][0][2] = fma_(M[2][0][0], Ez, fma_(hAzz, Ex, fma_(u2z, kx_z, tz)));
+    M[0][2][2] = fma_(M[0][2][0], Ez, fma_(hAzz, Ey, fma_(u2z, ky_z, tz)));
+    M[2][1][1] = fma_(hz, M[2][1][0], fma_(hy, kx_z, mul_(qAyz, Ex)));
+    M[1][2][1] = fma_(hz, M[1][2][0], fma_(hx, ky_z, mul_(qAxz, Ey)));
+    M[1][1][2] = fma_(hy, M[1][0][2], fma_(hx, kz_y, mul_(qAxy, Ez)));
+    const R T = fma_(kx_z, Ey, mul_(ky_z, Ex));
+    M[2][2][1] = fma_(hz, add_(M[2][2][0], t2), T);
+    M[2][1][2] = fma_(hy, add_(M[2][0][2], t2), fma_(kx_y, Ez, mul_(kz_y, Ex)));
+    M[1][2][2] = fma_(hx, add_(M[0][2][2], t2), fma_(ky_x, Ez, mul_(kz_x, Ey)));
+    M[2][2][2] = fma_(M[2][2][0], Ez, fma_(u2z, T, fma_(hAzz, mul_(Ex, Ey), mul_(R(h * th), tz))));
+    // the inverse, axis by axis: index 0, 1, 2 is c = -1, 0, 1 afterwards
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const R n0 = M[a][b][0], n1 = M[a][b][1], n2 = M[a][b][2];
+            M[a][b][0] = sub_(n2, n1);
+            M[a][b][1] = fma_(m2, n2, n0);
+            M[a][b][2] = add_(n2, n1);
+        }
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const R n0 = M[a][0][z], n1 = M[a][1][z], n2 = M[a][2][z];
+            M[a][0][z] = sub_(n2, n1);
+            M[a][1][z] = fma_(m2, n2, n0);
+            M[a][2][z] = add_(n2, n1);
+        }
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const R n0 = M[0][y][z], n1 = M[1][y][z], n2 = M[2][y][z];
+            sink(3 * z + y, sub_(n2, n1), fma_(m2, n2, n0), add_(n2, n1));
+        }
+    }
+}
+
 // Collision with the default ghost rates (all 1).  d holds f_i - w_i on entry;
 // the post-collision f*_i - w_i go to the sink line by line, or back into d
 // without one.  rho, u receive the (conserved) moments.  With SCALED, d holds
@@ -610,6 +719,12 @@ __device__ __forceinline__ void collide_ghost1(R (&d)[27], R omega, R &rho, R &u
     if constexpr (SCALED) {
         scaled_sums<R>([&](int i) { return d[i]; }, m);
         scaled_finish<R>(m, omega, rho, ux, uy, uz, in_scale, out_scale, *sink);
+    } else if constexpr (std::is_same<R, double>::value) {
+        scaled_sums<R>([&](int i) { return d[i]; }, m);
+        if (sink)
+            raw_finish<R>(m, omega, rho, ux, uy, uz, *sink);
+        else
+            raw_finish<R>(m, omega, rho, ux, uy, uz, ToArray<R>{d});
     } else {
         ghost1_sums(d, SameInput{}, m);
         if (sink)
@@ -1559,9 +1674,9 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_PAIR_MIN_BLOCKS) k_step_pair
 // FP32 pipe, one instruction stream for every unit (the output sink alone
 // tells plain units, 64 fluid cells without wall links, from the others).
 //
-// Measured per step, before (chunk kernel) and now: Re 6500 nozzle 448 ->
-// 339 us (4.61 TB/s of algorithmic bytes), Re 3500 nozzle 150 -> 126 us,
-// periodic 256^3 515 -> 349 us (5.20 TB/s).  Two stages and 4 blocks of 4
+// Measured per step, before (chunk kernel) and now: Re 6500 nozzle 445 ->
+// 339 us (4.61 TB/s of algorithmic bytes), Re 3500 nozzle 151 -> 126 us,
+// periodic 256^3 497 -> 349 us (5.20 TB/s).  Two stages and 4 blocks of 4
 // warps per SM: 3 blocks 361 us on the Re 6500 nozzle, 5 blocks (96
 // registers, no spills) 395 us, three stages 347 us; more bytes in flight
 // only widen the span of the arrays that is open at a time.
