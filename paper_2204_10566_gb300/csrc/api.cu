@@ -13,11 +13,6 @@
 
 #include "lbm_internal.h"
 
-namespace lbm {
-// Per-cell (rho, u) in active order -> rho[n], u[n][3] on the device (common.cu).
-cudaError_t launch_split_moments(const double *in, int64_t n, double *rho, double *u, cudaStream_t s);
-}  // namespace lbm
-
 using namespace lbm;
 
 struct lbm_ctx {
@@ -35,7 +30,7 @@ struct lbm_ctx {
     int4 *d_row_nb = nullptr;
     int2 *d_chunks = nullptr;
     int4 *d_bnodes = nullptr;
-    int32_t *d_slot_of_active = nullptr;
+    int32_t *d_act = nullptr;        // per slot: its cell in the active order, or -1
     int32_t *d_wall_qidx = nullptr;  // per slot: wall-distance record or -1 (lbm_set_wall_q)
     uint8_t *d_wall_q = nullptr;     // 32-byte records
     int64_t n_wall_q = 0;
@@ -172,7 +167,7 @@ void release_geometry(lbm_ctx *c) {
     dev_free(c, c->d_row_nb, c->idx.row_nb.size() * 4);
     dev_free(c, c->d_chunks, c->idx.chunks.size() * 8);
     dev_free(c, c->d_bnodes, c->idx.bnodes.size() * 16);
-    dev_free(c, c->d_slot_of_active, c->idx.slot_of_active.size() * 4);
+    dev_free(c, c->d_act, ns * 4);
     dev_free(c, c->d_tiles, c->idx.tiles.size() * 4);
     dev_free(c, c->d_units, c->idx.units.size() * 4);
     c->d_units = nullptr;
@@ -192,7 +187,7 @@ void release_geometry(lbm_ctx *c) {
     c->d_row_nb = nullptr;
     c->d_chunks = nullptr;
     c->d_bnodes = nullptr;
-    c->d_slot_of_active = nullptr;
+    c->d_act = nullptr;
     c->d_partials = nullptr;
     c->d_health = nullptr;
     c->d_status = nullptr;
@@ -288,7 +283,46 @@ int partial_capacity(const lbm_ctx *c, int64_t n_wnodes) {
     const int tiles = tile_blocks(std::max<int64_t>((int64_t)c->idx.tiles.size() / TILE_INTS, c->n_tiles_wall));
     const int split = std::max(split_blocks((int64_t)c->idx.rest_chunks.size(), (int64_t)c->idx.pair_items.size()),
                                split_blocks(c->n_rest_wall, c->n_items_wall));
-    return std::max({c->fluid_blocks + nodes, tiles + nodes, split + nodes, node_blocks(c->idx.n_active)});
+    return std::max({c->fluid_blocks + nodes, tiles + nodes, split + nodes, reduce_blocks(c->idx.nslots)});
+}
+
+// Transfers of per-cell arrays in the active order run in TRANSFER_PARTS parts
+// beside the kernel that reads or writes them, from this many cells on: the
+// copies go on the context's second stream, each part's kernel after (or
+// before) its copy.  On the 256^3 vortex (537 MB each way), moments 5.8 ->
+// 3.8 ms and fields 7.3 -> 5.6 ms; below, the extra launches cost more than the overlap gives.
+constexpr int TRANSFER_PARTS = 4;
+constexpr int64_t TRANSFER_SPLIT = 1 << 20;
+
+// Runs part(k0, k1, stream, last) for parts of the n cells: copies on one
+// stream and kernels on the other, part by part, `first` before `second`.
+// Without a second stream, or for few cells, one part on c->stream.  Both
+// streams are idle when it returns.
+template <class First, class Second>
+cudaError_t in_parts(lbm_ctx *c, int64_t n, cudaStream_t first_on, cudaStream_t second_on, First first, Second second) {
+    const bool split = c->side.stream && n >= TRANSFER_SPLIT;
+    const int parts = split ? TRANSFER_PARTS : 1;
+    if (!split) first_on = second_on = c->stream;
+    cudaEvent_t done[TRANSFER_PARTS] = {};
+    cudaError_t e = cudaSuccess;
+    if (split) {  // the second stream starts after what c->stream holds
+        e = cudaEventRecord(c->side.fork, c->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side.stream, c->side.fork, 0);
+    }
+    for (int p = 0; p < parts && e == cudaSuccess; ++p) {
+        e = first(n * p / parts, n * (p + 1) / parts, first_on);
+        if (split && e == cudaSuccess) e = cudaEventCreateWithFlags(&done[p], cudaEventDisableTiming);
+        if (split && e == cudaSuccess) e = cudaEventRecord(done[p], first_on);
+    }
+    for (int p = 0; p < parts && e == cudaSuccess; ++p) {
+        if (split) e = cudaStreamWaitEvent(second_on, done[p], 0);
+        if (e == cudaSuccess) e = second(n * p / parts, n * (p + 1) / parts, second_on);
+    }
+    const cudaError_t e1 = split ? cudaStreamSynchronize(c->side.stream) : cudaSuccess;
+    const cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    for (cudaEvent_t ev : done)
+        if (ev) cudaEventDestroy(ev);
+    return e != cudaSuccess ? e : (e1 != cudaSuccess ? e1 : e2);
 }
 
 // Ghost slots and periodic copies of the current buffer from its active cells.
@@ -679,9 +713,9 @@ int64_t ctx_footprint(const lbm_desc &d, const HostIndex &ix) {
     const int S = storage_bytes(d.precision);
     const int64_t pop = 27 * ix.nslots * S + 2 * buffer_margin(ix.n_row) * S;
     const int64_t blocks = std::max<int64_t>(fluid_blocks((int32_t)ix.chunks.size()) + node_blocks((int64_t)ix.bnodes.size()),
-                                             node_blocks(ix.n_active));
+                                             reduce_blocks(ix.nslots));
     return 2 * pop + (ix.nslots + 2 * MASK_MARGIN) * 4 + (int64_t)ix.row_nb.size() * 4 + (int64_t)ix.chunks.size() * 8 +
-           (int64_t)ix.bnodes.size() * 16 + ix.n_active * 4 + (int64_t)ix.tiles.size() * 4 +
+           (int64_t)ix.bnodes.size() * 16 + ix.nslots * 4 + (int64_t)ix.tiles.size() * 4 +
            (int64_t)ix.units.size() * 4 + (int64_t)ix.pair_items.size() * 8 + (int64_t)ix.rest_chunks.size() * 8 +
            blocks * REDUCE_SLOTS * 8 + 64 + 256;
 }
@@ -704,7 +738,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->d_row_nb = (int4 *)dev_alloc(c, c->idx.row_nb.size() * 4);
     c->d_chunks = (int2 *)dev_alloc(c, c->idx.chunks.size() * 8);
     c->d_bnodes = (int4 *)dev_alloc(c, c->idx.bnodes.size() * 16);
-    c->d_slot_of_active = (int32_t *)dev_alloc(c, c->idx.slot_of_active.size() * 4);
+    c->d_act = (int32_t *)dev_alloc(c, ns * 4);
     c->d_tiles = (int32_t *)dev_alloc(c, c->idx.tiles.size() * 4);
     c->d_units = (int32_t *)dev_alloc(c, c->idx.units.size() * 4);
     c->d_items = (int2 *)dev_alloc(c, c->idx.pair_items.size() * 8);
@@ -712,7 +746,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->d_partials = (double *)dev_alloc(c, (size_t)c->nblocks * REDUCE_SLOTS * 8);
     c->d_health = (double *)dev_alloc(c, 8 * 8);
     c->d_status = (uint32_t *)dev_alloc(c, 256);
-    if (!c->f[0] || !c->f[1] || !c->d_mask || !c->d_row_nb || !c->d_chunks || !c->d_bnodes || !c->d_slot_of_active ||
+    if (!c->f[0] || !c->f[1] || !c->d_mask || !c->d_row_nb || !c->d_chunks || !c->d_bnodes || !c->d_act ||
         !c->d_tiles || !c->d_units || !c->d_items || !c->d_rest || !c->d_partials || !c->d_health || !c->d_status) {
         release_geometry(c);
         return fail(c, LBM_ERR_OOM, "device allocation failed in lbm_set_geometry");
@@ -729,9 +763,9 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
         CK(cudaMemcpyAsync(c->d_bnodes, c->idx.bnodes.data(), c->idx.bnodes.size() * 16, cudaMemcpyHostToDevice,
                            c->stream),
            "copy boundary nodes");
-    CK(cudaMemcpyAsync(c->d_slot_of_active, c->idx.slot_of_active.data(), c->idx.slot_of_active.size() * 4,
-                       cudaMemcpyHostToDevice, c->stream),
-       "copy slot map");
+    std::vector<int32_t> act(ns, -1);
+    for (int64_t k = 0; k < c->idx.n_active; ++k) act[(size_t)c->idx.slot_of_active[(size_t)k]] = (int32_t)k;
+    CK(cudaMemcpyAsync(c->d_act, act.data(), ns * 4, cudaMemcpyHostToDevice, c->stream), "copy slot map");
     if (!c->idx.tiles.empty())
         CK(cudaMemcpyAsync(c->d_tiles, c->idx.tiles.data(), c->idx.tiles.size() * 4, cudaMemcpyHostToDevice,
                            c->stream),
@@ -877,7 +911,7 @@ lbm_status lbm_init_equilibrium(lbm_ctx *c, double rho, const double u[3]) {
     if (!u || !(rho > 0.0)) return fail(c, LBM_ERR_ARG, "need rho > 0 and u");
     DeviceGuard g(c->desc.device);
     c->cur = 0;
-    CK(DISPATCH(c->desc.precision, launch_init_eq, c->f[0], c->d_slot_of_active, c->idx.n_active, c->idx.nslots,
+    CK(DISPATCH(c->desc.precision, launch_init_eq, c->f[0], c->d_act, (int64_t)0, c->idx.n_active, c->idx.nslots,
                 fp16_scale(c), nullptr, nullptr, rho, u[0], u[1], u[2], c->stream),
        "init equilibrium");
     st = reset_state(c);
@@ -896,23 +930,30 @@ lbm_status lbm_init_fields(lbm_ctx *c, const double *rho, const double *u, int32
     double *d = (double *)dev_alloc(c, (size_t)n * 4 * 8);
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     cudaError_t e;
-    if (layout == LBM_LAYOUT_ACTIVE) {  // the caller's arrays are already in the device's order: copy them as they are
-        e = cudaMemcpyAsync(d, rho, (size_t)n * 8, cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d + n, u, (size_t)n * 3 * 8, cudaMemcpyHostToDevice, c->stream);
-    } else {
-        std::vector<double> h((size_t)n * 4);
+    std::vector<double> h;
+    const double *hr = rho, *hu = u;  // in the active order the caller's arrays are copied as they are
+    if (layout == LBM_LAYOUT_BOX) {
+        h.resize((size_t)n * 4);
         for_active(c, layout, [&](int64_t k, int64_t r) {
             h[(size_t)k] = rho[r];
             for (int a = 0; a < 3; ++a) h[(size_t)n + 3 * (size_t)k + a] = u[3 * r + a];
         });
-        e = cudaMemcpyAsync(d, h.data(), (size_t)n * 4 * 8, cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // h leaves scope
+        hr = h.data();
+        hu = h.data() + n;
     }
     c->cur = 0;
-    if (e == cudaSuccess)
-        e = DISPATCH(c->desc.precision, launch_init_eq, c->f[0], c->d_slot_of_active, n, c->idx.nslots,
-                     fp16_scale(c), d, d + n, 1.0, 0.0, 0.0, 0.0, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    e = in_parts(
+        c, n, c->side.stream, c->stream,
+        [&](int64_t k0, int64_t k1, cudaStream_t s) {
+            cudaError_t r = cudaMemcpyAsync(d + k0, hr + k0, (size_t)(k1 - k0) * 8, cudaMemcpyHostToDevice, s);
+            if (r == cudaSuccess)
+                r = cudaMemcpyAsync(d + n + 3 * k0, hu + 3 * k0, (size_t)(k1 - k0) * 24, cudaMemcpyHostToDevice, s);
+            return r;
+        },
+        [&](int64_t k0, int64_t k1, cudaStream_t s) {
+            return DISPATCH(c->desc.precision, launch_init_eq, c->f[0], c->d_act, k0, k1, c->idx.nslots, fp16_scale(c),
+                            d, d + n, 1.0, 0.0, 0.0, 0.0, s);
+        });
     dev_free(c, d, (size_t)n * 4 * 8);
     if (e != cudaSuccess) return cuda_fail(c, e, "init fields");
     return reset_state(c);
@@ -939,8 +980,8 @@ lbm_status lbm_set_populations(lbm_ctx *c, const double *f, int32_t layout) {
     }
     c->cur = 0;
     if (e == cudaSuccess)
-        e = DISPATCH(c->desc.precision, launch_set_populations, c->f[0], c->d_slot_of_active, n, c->idx.nslots,
-                     fp16_scale(c), d, c->stream);
+        e = DISPATCH(c->desc.precision, launch_set_populations, c->f[0], c->d_act, c->idx.nslots, fp16_scale(c), d,
+                     c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "set populations");
@@ -957,8 +998,8 @@ lbm_status lbm_get_populations(lbm_ctx *c, double *f, int32_t layout) {
     const size_t bytes = (size_t)n * 27 * 8;
     double *d = (double *)dev_alloc(c, bytes);
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-    cudaError_t e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_slot_of_active, n,
-                             c->idx.nslots, 1.0f / fp16_scale(c), d, c->stream);
+    cudaError_t e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_act, c->idx.nslots,
+                             1.0f / fp16_scale(c), d, c->stream);
     if (layout == LBM_LAYOUT_ACTIVE) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, bytes, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1049,37 +1090,37 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
     DeviceGuard g(c->desc.device);
     const int64_t n = c->idx.n_active;
     const size_t bytes = (size_t)n * 4 * 8;
-    if (layout == LBM_LAYOUT_ACTIVE) {
-        // split on the device, then one copy straight into each of the caller's arrays
-        double *d = (double *)dev_alloc(c, 2 * bytes);
-        if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-        double *dr = d + 4 * n, *du = d + 5 * n;
-        cudaError_t e = DISPATCH(c->desc.precision, launch_moments, c->f[c->cur], c->d_slot_of_active, n,
-                                 c->idx.nslots, 1.0f / fp16_scale(c), d, c->stream);
-        if (e == cudaSuccess) e = launch_split_moments(d, n, dr, du, c->stream);
-        if (e == cudaSuccess && rho) e = cudaMemcpyAsync(rho, dr, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess && u) e = cudaMemcpyAsync(u, du, (size_t)n * 3 * 8, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        dev_free(c, d, 2 * bytes);
-        if (e != cudaSuccess) return cuda_fail(c, e, "get moments");
-        return LBM_OK;
-    }
-    double *d = (double *)dev_alloc(c, bytes);
+    double *d = (double *)dev_alloc(c, bytes);  // rho[n], then u[n][3]
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-    std::vector<double> h((size_t)n * 4);
-    cudaError_t e = DISPATCH(c->desc.precision, launch_moments, c->f[c->cur], c->d_slot_of_active, n, c->idx.nslots,
-                             1.0f / fp16_scale(c), d, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, bytes, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n * 4 : 0);
+    double *hr = rho, *hu = u;  // in the active order each part goes straight into the caller's arrays
+    if (layout == LBM_LAYOUT_BOX) {
+        hr = h.data();
+        hu = h.data() + n;
+    }
+    const cudaError_t e = in_parts(
+        c, n, c->stream, c->side.stream,
+        [&](int64_t k0, int64_t k1, cudaStream_t s) {
+            return DISPATCH(c->desc.precision, launch_moments, c->f[c->cur], c->d_act, k0, k1, c->idx.nslots,
+                            1.0f / fp16_scale(c), rho ? d : nullptr, u ? d + n : nullptr, s);
+        },
+        [&](int64_t k0, int64_t k1, cudaStream_t s) {
+            cudaError_t r = cudaSuccess;
+            if (rho) r = cudaMemcpyAsync(hr + k0, d + k0, (size_t)(k1 - k0) * 8, cudaMemcpyDeviceToHost, s);
+            if (u && r == cudaSuccess)
+                r = cudaMemcpyAsync(hu + 3 * k0, d + n + 3 * k0, (size_t)(k1 - k0) * 24, cudaMemcpyDeviceToHost, s);
+            return r;
+        });
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "get moments");
+    if (layout == LBM_LAYOUT_ACTIVE) return LBM_OK;
     const int64_t total = layout_count(c, layout);
     if (rho) memset(rho, 0, (size_t)total * 8);
     if (u) memset(u, 0, (size_t)total * 3 * 8);
     for_active(c, layout, [&](int64_t k, int64_t r) {
-        if (rho) rho[r] = h[4 * (size_t)k];
+        if (rho) rho[r] = h[(size_t)k];
         if (u)
-            for (int a = 0; a < 3; ++a) u[3 * r + a] = h[4 * (size_t)k + 1 + a];
+            for (int a = 0; a < 3; ++a) u[3 * r + a] = h[(size_t)n + 3 * (size_t)k + a];
     });
     return LBM_OK;
 }
@@ -1089,10 +1130,10 @@ lbm_status lbm_get_totals(lbm_ctx *c, double *mass, double mom[3]) {
     lbm_status st = need(c, true, false, true);
     if (st) return st;
     DeviceGuard g(c->desc.device);
-    CK(DISPATCH(c->desc.precision, launch_reduce, c->f[c->cur], c->d_slot_of_active, c->idx.n_active, c->idx.nslots,
-                1.0f / fp16_scale(c), c->d_partials, c->stream),
+    CK(DISPATCH(c->desc.precision, launch_reduce, c->f[c->cur], c->d_act, c->idx.nslots, 1.0f / fp16_scale(c),
+                c->d_partials, c->stream),
        "reduce");
-    CK(launch_finalize(c->d_partials, node_blocks(c->idx.n_active), c->d_health, c->d_status, c->stream), "finalize");
+    CK(launch_finalize(c->d_partials, reduce_blocks(c->idx.nslots), c->d_health, c->d_status, c->stream), "finalize");
     CK(cudaMemcpyAsync(c->health, c->d_health, 6 * 8, cudaMemcpyDeviceToHost, c->stream), "read totals");
     CK(cudaStreamSynchronize(c->stream), "sync totals");
     if (mass) *mass = c->health[0];
@@ -1160,42 +1201,35 @@ lbm_status lbm_stats_reset(lbm_ctx *c) {
     return LBM_OK;
 }
 
-// Means of the first ncomp accumulator rows, per active cell, to the host
-// ([n_active][ncomp]).
-lbm_status stats_means(lbm_ctx *c, int ncomp, std::vector<double> &h) {
-    const int64_t n = c->idx.n_active;
-    const size_t bytes = (size_t)n * ncomp * 8;
-    h.assign((size_t)n * ncomp, 0.0);
-    if (n == 0) return LBM_OK;
-    double *d = (double *)dev_alloc(c, bytes);
-    if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-    cudaError_t e = launch_stats_mean(c->d_stats, ncomp, c->d_slot_of_active, n, c->idx.nslots,
-                                      1.0 / (double)c->stats_samples, d, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, bytes, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    dev_free(c, d, bytes);
-    if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
-    return LBM_OK;
-}
-
 lbm_status lbm_stats_get(lbm_ctx *c, double *mean_uz, double *mean_uzuz, int64_t *n_samples, int32_t layout) {
     lbm_status st = need(c, true, false, false);
     if (st) return st;
     if (layout != LBM_LAYOUT_ACTIVE && layout != LBM_LAYOUT_BOX) return fail(c, LBM_ERR_ARG, "bad layout");
     if (n_samples) *n_samples = c->stats_samples;
     if (!mean_uz && !mean_uzuz) return LBM_OK;
-    const int64_t total = layout_count(c, layout);
-    if (mean_uz) memset(mean_uz, 0, (size_t)total * 8);
-    if (mean_uzuz) memset(mean_uzuz, 0, (size_t)total * 8);
+    const int64_t n = c->idx.n_active;
+    const size_t total = (size_t)layout_count(c, layout) * 8, bytes = (size_t)n * 2 * 8;
+    double *out[2] = {mean_uz, mean_uzuz};
+    if (!c->d_stats || c->stats_samples == 0 || layout == LBM_LAYOUT_BOX)
+        for (double *o : out)
+            if (o) memset(o, 0, total);
     if (!c->d_stats || c->stats_samples == 0) return LBM_OK;
     DeviceGuard g(c->desc.device);
-    std::vector<double> h;
-    st = stats_means(c, STATS_AXIAL, h);
-    if (st) return st;
-    for_active(c, layout, [&](int64_t k, int64_t r) {
-        if (mean_uz) mean_uz[r] = h[2 * (size_t)k];
-        if (mean_uzuz) mean_uzuz[r] = h[2 * (size_t)k + 1];
-    });
+    double *d = (double *)dev_alloc(c, bytes);  // <u_z>[n], then <u_z^2>[n]
+    if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
+    std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n : 0);
+    cudaError_t e = launch_stats_mean(c->d_stats, STATS_AXIAL, c->d_act, c->idx.nslots, 1.0 / (double)c->stats_samples,
+                                      d, d + n, c->stream);
+    for (int q = 0; q < 2; ++q) {
+        if (e != cudaSuccess || !out[q]) continue;
+        double *to = layout == LBM_LAYOUT_BOX ? h.data() : out[q];  // the active order goes straight to the caller
+        e = cudaMemcpyAsync(to, d + q * n, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e == cudaSuccess && layout == LBM_LAYOUT_BOX)
+            for_active(c, layout, [&](int64_t k, int64_t r) { out[q][r] = h[(size_t)k]; });
+    }
+    dev_free(c, d, bytes);
+    if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
     return LBM_OK;
 }
 
@@ -1207,17 +1241,25 @@ lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int3
     if (!mean) return LBM_OK;
     if (c->stats_ncomp != STATS_FULL && c->stats_samples > 0)
         return fail(c, LBM_ERR_STATE, "the accumulators hold axial statistics only");
-    const int64_t total = layout_count(c, layout);
-    memset(mean, 0, (size_t)total * LBM_STATS_FULL_COMPONENTS * 8);
+    constexpr int Q = LBM_STATS_FULL_COMPONENTS;  // the rows after the axial ones
+    const int64_t n = c->idx.n_active;
+    const size_t bytes = (size_t)n * Q * 8;
+    if (!c->d_stats || c->stats_samples == 0 || layout == LBM_LAYOUT_BOX)
+        memset(mean, 0, (size_t)layout_count(c, layout) * Q * 8);
     if (!c->d_stats || c->stats_samples == 0) return LBM_OK;
     DeviceGuard g(c->desc.device);
-    std::vector<double> h;
-    st = stats_means(c, STATS_FULL, h);
-    if (st) return st;
-    for_active(c, layout, [&](int64_t k, int64_t r) {
-        for (int q = 0; q < LBM_STATS_FULL_COMPONENTS; ++q)
-            mean[(size_t)r * LBM_STATS_FULL_COMPONENTS + q] = h[(size_t)k * STATS_FULL + STATS_AXIAL + q];
-    });
+    double *d = (double *)dev_alloc(c, bytes);
+    if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
+    std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n * Q : 0);
+    double *to = layout == LBM_LAYOUT_BOX ? h.data() : mean;
+    cudaError_t e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act,
+                                      c->idx.nslots, 1.0 / (double)c->stats_samples, d, nullptr, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(to, d, bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    dev_free(c, d, bytes);
+    if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
+    if (layout == LBM_LAYOUT_BOX)
+        for_active(c, layout, [&](int64_t k, int64_t r) { memcpy(mean + r * Q, &h[(size_t)k * Q], Q * 8); });
     return LBM_OK;
 }
 

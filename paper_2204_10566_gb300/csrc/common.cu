@@ -1,5 +1,7 @@
 // Precision-independent kernels: the fixed-order final pass of the FP64
 // health reduction and the time-average readback.
+#include <algorithm>
+
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -8,6 +10,10 @@ int fluid_blocks(int32_t nchunks) {
     const int64_t threads = (int64_t)nchunks * CHUNK;
     return (int)((threads + STEP_THREADS - 1) / STEP_THREADS);
 }
+
+// Enough blocks to fill the device; a block's slots follow from this count
+// alone, so the totals stay bitwise reproducible.
+int reduce_blocks(int64_t nslots) { return (int)std::min<int64_t>((nslots + STEP_THREADS - 1) / STEP_THREADS, 152 * 12); }
 
 int node_blocks(int64_t n) { return (int)((n + STEP_THREADS - 1) / STEP_THREADS); }
 
@@ -49,35 +55,23 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *health,
     return cudaGetLastError();
 }
 
-__global__ void k_stats_mean(const double *stats, int ncomp, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                             double inv_n, double *out) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int slot = slot_of_active[k];
-    for (int q = 0; q < ncomp; ++q) out[(size_t)ncomp * k + q] = stats[(size_t)q * stride + slot] * inv_n;
+__global__ void k_stats_mean(const double *stats, int ncomp, const int32_t *act, int64_t stride, double inv_n,
+                             double *out, double *out2) {
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= stride) return;
+    const int64_t k = act[slot];
+    if (k < 0) return;
+    if (out2) {
+        out[k] = stats[slot] * inv_n;
+        out2[k] = stats[stride + slot] * inv_n;
+        return;
+    }
+    for (int q = 0; q < ncomp; ++q) out[(int64_t)ncomp * k + q] = stats[(int64_t)q * stride + slot] * inv_n;
 }
 
-cudaError_t launch_stats_mean(const double *stats, int ncomp, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                              double inv_n, double *out, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_stats_mean<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(stats, ncomp, slot_of_active, n, stride, inv_n, out);
-    return cudaGetLastError();
-}
-
-// Split per-cell moments (rho, ux, uy, uz) in active order into rho[n] and
-// u[n][3], so that both go to the caller's host arrays in one copy each.
-__global__ void k_split_moments(const double *in, int64_t n, double *rho, double *u) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    rho[k] = in[4 * k];
-    u[3 * k] = in[4 * k + 1];
-    u[3 * k + 1] = in[4 * k + 2];
-    u[3 * k + 2] = in[4 * k + 3];
-}
-
-cudaError_t launch_split_moments(const double *in, int64_t n, double *rho, double *u, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_split_moments<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, n, rho, u);
+cudaError_t launch_stats_mean(const double *stats, int ncomp, const int32_t *act, int64_t stride, double inv_n,
+                              double *out, double *out2, cudaStream_t s) {
+    k_stats_mean<<<(unsigned)((stride + 255) / 256), 256, 0, s>>>(stats, ncomp, act, stride, inv_n, out, out2);
     return cudaGetLastError();
 }
 

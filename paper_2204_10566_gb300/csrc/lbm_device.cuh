@@ -188,27 +188,6 @@ struct Axis {
 template <class R>
 __device__ __forceinline__ R g2(int c) { return c == 0 ? R(-1) : R(0.5); }
 
-// Equilibrium deviation f^eq_i(rho, u) - w_i in product form, written so
-// that no O(1) cancellation occurs:
-//   rho prod(w + d) - prod w = (rho - 1) w_i + rho (dx gy gz + wx (dy gz + wy dz)).
-template <class R>
-__device__ __forceinline__ void eq_deviation(R rho, const Axis<R> &X, const Axis<R> &Y, const Axis<R> &Z,
-                                             R (&out)[27]) {
-    const R drho = rho - R(1);
-#pragma unroll
-    for (int j = 0; j < 9; ++j) {
-        const int cy = j % 3 - 1, cz = j / 3 - 1;
-        const R wy = w1<R>(cy), wz = w1<R>(cz);
-        const R E = Y.g0[cy + 1] * Z.g0[cz + 1];
-        const R D = Y.d[cy + 1] * Z.g0[cz + 1] + wy * Z.d[cz + 1];
-#pragma unroll
-        for (int cx = -1; cx <= 1; ++cx) {
-            const R wx = w1<R>(cx);
-            out[3 * j + cx + 1] = drho * (wx * wy * wz) + rho * (X.d[cx + 1] * E + wx * D);
-        }
-    }
-}
-
 // d_i += f^eq_i(rho_b, u_b) - f^eq_i(rho_f, u_f), line by line so that only
 // a few values are live besides d (keeps the boundary path from raising the
 // register count of the whole kernel).
@@ -1934,6 +1913,19 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STAGE_BLOCKS) k_step_units(c
 
 // ---------------------------------------------------------- utility kernels
 
+// The stored values of a cell, without the FP16 scale.
+template <int P>
+__device__ __forceinline__ void load_stored(const void *f, int64_t stride, int slot, double (&d)[27]) {
+    const typename Storage<P>::T *p = static_cast<const typename Storage<P>::T *>(f);
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        if constexpr (P == 2)
+            d[i] = (double)__half2float(p[(int64_t)i * stride + slot]);
+        else
+            d[i] = (double)p[(int64_t)i * stride + slot];
+    }
+}
+
 template <int P>
 __device__ __forceinline__ void load_cell(const void *f, int64_t stride, int slot, float inv_scale,
                                           double (&d)[27]) {
@@ -1948,33 +1940,63 @@ __device__ __forceinline__ void load_cell(const void *f, int64_t stride, int slo
     }
 }
 
-__device__ __forceinline__ void moments_of(const double (&d)[27], double &rho, double &ux, double &uy,
-                                           double &uz) {
-    double drho = 0, jx = 0, jy = 0, jz = 0;
+// Whether x is neither zero, subnormal, infinite nor NaN (integer pipe).
+__device__ __forceinline__ bool normal(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7ff00000u) - 0x00100000u < 0x7fe00000u;
+}
+
+// j / rho for a normal rho from its reciprocal inv, corrected once: the last
+// bit of the division at three operations.  An infinite j stays infinite.
+__device__ __forceinline__ double quotient(double j, double rho, double inv) {
+    const double q = __dmul_rn(j, inv);
+    return normal(q) ? __fma_rn(__fma_rn(-rho, q, j), inv, q) : q;
+}
+
+// Density and velocity from the stored populations of a cell, in FP64 (the
+// FP16 scale, a power of two, acts on the sums).  The FP64 pipe is what
+// bounds the kernels that use this (a multiplication by every direction's
+// components, 0 included, and three divisions took 130 us per million cells),
+// so the sums share their partial sums: 49 additions.
+template <int P>
+__device__ __forceinline__ void moments_of(const double (&d)[27], double inv_scale, double &rho, double &ux,
+                                           double &uy, double &uz) {
+    const double sc = Storage<P>::SCALED ? inv_scale : 1.0;
+    double s[9], jx = 0.0;  // sums over cx of each line (cy, cz)
 #pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        drho += d[i];
-        jx += cx_of(i) * d[i];
-        jy += cy_of(i) * d[i];
-        jz += cz_of(i) * d[i];
+    for (int j = 0; j < 9; ++j) {
+        s[j] = (d[3 * j] + d[3 * j + 2]) + d[3 * j + 1];
+        jx += d[3 * j + 2] - d[3 * j];
     }
+    const double lo = (s[0] + s[3]) + s[6], mid = (s[1] + s[4]) + s[7], hi = (s[2] + s[5]) + s[8];  // cy = -1, 0, 1
+    double jy = hi - lo, jz = ((s[6] - s[0]) + (s[8] - s[2])) + (s[7] - s[1]), drho = (lo + hi) + mid;
+    if constexpr (Storage<P>::SCALED) drho *= sc, jx *= sc, jy *= sc, jz *= sc;
     rho = 1.0 + drho;
-    ux = jx / rho;
-    uy = jy / rho;
-    uz = jz / rho;
+    if (normal(rho)) {
+        const double inv = recip(rho);
+        ux = quotient(jx, rho, inv);
+        uy = quotient(jy, rho, inv);
+        uz = quotient(jz, rho, inv);
+    } else {  // a diverged state: whatever the division gives
+        ux = jx / rho;
+        uy = jy / rho;
+        uz = jz / rho;
+    }
 }
 
 // Health reduction of a stored state (mass, momentum, max |u|, non-finite count).
 template <int P>
-__global__ void __launch_bounds__(STEP_THREADS) k_reduce(const void *f, const int32_t *slot_of_active, int64_t n,
-                                                         int64_t stride, float inv_scale, double *partials) {
-    const int64_t k = (int64_t)blockIdx.x * STEP_THREADS + threadIdx.x;
+__global__ void __launch_bounds__(STEP_THREADS) k_reduce(const void *f, const int32_t *act, int64_t stride,
+                                                         float inv_scale, double *partials) {
     double hv[6] = {0, 0, 0, 0, 0, 0};
-    if (k < n) {
-        double d[27], rho, ux, uy, uz;
-        load_cell<P>(f, stride, slot_of_active[k], inv_scale, d);
-        moments_of(d, rho, ux, uy, uz);
-        health_values(rho, ux, uy, uz, hv);
+    for (int64_t slot = (int64_t)blockIdx.x * STEP_THREADS + threadIdx.x; slot < stride;
+         slot += (int64_t)gridDim.x * STEP_THREADS) {
+        if (__ldg(act + slot) < 0) continue;
+        double d[27], rho, ux, uy, uz, v[6];
+        load_stored<P>(f, stride, (int)slot, d);
+        moments_of<P>(d, inv_scale, rho, ux, uy, uz);
+        health_values(rho, ux, uy, uz, v);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) hv[q] = q == 4 ? fmax(hv[q], v[q]) : hv[q] + v[q];
     }
     block_reduce_write(hv, partials);
 }
@@ -2038,18 +2060,27 @@ __global__ void __launch_bounds__(STEP_THREADS) k_fill_periodic_nodes(void *f, c
             if (c_row<AX>(i) == -1) p[(int64_t)i * stride + base + n_row] = p[(int64_t)i * stride + slot];
 }
 
+// Moments of the active cells k0 .. k1 - 1.  Neighbouring slots of a row along z are far
+// apart in the active order, but the rows around them are written at about
+// the same time, so L2 merges the 8-byte stores into whole sectors; reading
+// along the active order instead took every population's sector eight times
+// over (1.26 ms on the Re 3500 nozzle, now 0.5 ms).
 template <int P>
-__global__ void k_moments(const void *f, const int32_t *slot_of_active, int64_t n, int64_t stride, float inv_scale,
-                          double *out4) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+__global__ void k_moments(const void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float inv_scale,
+                          double *rho_out, double *u_out) {
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= stride) return;
+    const int64_t k = __ldg(act + slot);
+    if (k < k0 || k >= k1) return;
     double d[27], rho, ux, uy, uz;
-    load_cell<P>(f, stride, slot_of_active[k], inv_scale, d);
-    moments_of(d, rho, ux, uy, uz);
-    out4[4 * k] = rho;
-    out4[4 * k + 1] = ux;
-    out4[4 * k + 2] = uy;
-    out4[4 * k + 3] = uz;
+    load_stored<P>(f, stride, (int)slot, d);
+    moments_of<P>(d, inv_scale, rho, ux, uy, uz);
+    if (rho_out) rho_out[k] = rho;
+    if (u_out) {
+        u_out[3 * k] = ux;
+        u_out[3 * k + 1] = uy;
+        u_out[3 * k + 2] = uz;
+    }
 }
 
 __device__ __forceinline__ double wd(int i) {
@@ -2057,12 +2088,14 @@ __device__ __forceinline__ double wd(int i) {
 }
 
 template <int P>
-__global__ void k_get_populations(const void *f, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                                  float inv_scale, double *out27) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+__global__ void k_get_populations(const void *f, const int32_t *act, int64_t stride, float inv_scale,
+                                  double *out27) {
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= stride) return;
+    const int64_t k = __ldg(act + slot);
+    if (k < 0) return;
     double d[27];
-    load_cell<P>(f, stride, slot_of_active[k], inv_scale, d);
+    load_cell<P>(f, stride, (int)slot, inv_scale, d);
 #pragma unroll
     for (int i = 0; i < 27; ++i) out27[27 * k + i] = wd(i) + d[i];
 }
@@ -2081,26 +2114,53 @@ __device__ __forceinline__ void store_cell(void *f, int64_t stride, int slot, fl
 }
 
 template <int P>
-__global__ void k_set_populations(void *f, const int32_t *slot_of_active, int64_t n, int64_t stride, float scale,
-                                  const double *in27) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+__global__ void k_set_populations(void *f, const int32_t *act, int64_t stride, float scale, const double *in27) {
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= stride) return;
+    const int64_t k = __ldg(act + slot);
+    if (k < 0) return;
     double d[27];
 #pragma unroll
     for (int i = 0; i < 27; ++i) d[i] = in27[27 * k + i] - wd(i);
-    store_cell<P>(f, stride, slot_of_active[k], scale, d);
+    store_cell<P>(f, stride, (int)slot, scale, d);
 }
 
+// Equilibrium deviations f^eq_i(rho, u) - w_i of a cell in FP64, by the
+// factors of scaled_finish without relaxed moments (about 120 operations;
+// bound by the FP64 pipe).
+__device__ __forceinline__ void eq_populations(double rho, double ux, double uy, double uz, double (&d)[27]) {
+    const double drho = rho - 1.0, w0 = 2.0 / 3.0, wp = 1.0 / 6.0;
+    const double hx = 0.5 * ux, hy = 0.5 * uy, hz = 0.5 * uz, x2 = hx * ux, y2 = hy * uy, z2 = hz * uz;
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        const double wz = z == 1 ? w0 : wp, dz = z == 0 ? z2 - hz : (z == 1 ? -2.0 * z2 : z2 + hz);
+        const double P0 = rho * (wz + dz), W0 = fma_(rho, dz, drho * wz);
+        const double T = y2 * P0, O = hy * P0, e1 = fma_(wp, W0, T), e2 = fma_(wp, P0, T);
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const double Bw = y == 0 ? e1 - O : (y == 1 ? fma_(w0, W0, -2.0 * T) : e1 + O);
+            const double Bd = y == 0 ? e2 - O : (y == 1 ? fma_(w0, P0, -2.0 * T) : e2 + O);
+            const double t = x2 * Bd, S = fma_(wp, Bw, t), A = hx * Bd;
+            d[9 * z + 3 * y] = S - A;
+            d[9 * z + 3 * y + 1] = fma_(-2.0, t, w0 * Bw);
+            d[9 * z + 3 * y + 2] = S + A;
+        }
+    }
+}
+
+// Equilibrium of the active cells k0 .. k1 - 1.
 template <int P>
-__global__ void k_init_eq(void *f, const int32_t *slot_of_active, int64_t n, int64_t stride, float scale,
+__global__ void k_init_eq(void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float scale,
                           const double *rho, const double *u, double rho0, double ux0, double uy0, double uz0) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= stride) return;
+    const int64_t k = __ldg(act + slot);
+    if (k < k0 || k >= k1) return;
     const double r = rho ? rho[k] : rho0;
     const double ux = u ? u[3 * k] : ux0, uy = u ? u[3 * k + 1] : uy0, uz = u ? u[3 * k + 2] : uz0;
     double d[27];
-    eq_deviation<double>(r, Axis<double>(ux), Axis<double>(uy), Axis<double>(uz), d);
-    store_cell<P>(f, stride, slot_of_active[k], scale, d);
+    eq_populations(r, ux, uy, uz, d);
+    store_cell<P>(f, stride, (int)slot, scale, d);
 }
 
 // --------------------------------------------------------------- launchers
@@ -2252,11 +2312,9 @@ cudaError_t launch_step(const StepArgs &a, bool ghost1, cudaStream_t s, int *lau
 }
 
 template <int P>
-cudaError_t launch_reduce(const void *f, const int32_t *slot_of_active, int64_t n, int64_t stride, float inv_scale,
-                          double *partials, cudaStream_t s) {
-    const int blocks = (int)((n + STEP_THREADS - 1) / STEP_THREADS);
-    if (blocks == 0) return cudaSuccess;
-    k_reduce<P><<<blocks, STEP_THREADS, 0, s>>>(f, slot_of_active, n, stride, inv_scale, partials);
+cudaError_t launch_reduce(const void *f, const int32_t *act, int64_t stride, float inv_scale, double *partials,
+                          cudaStream_t s) {
+    k_reduce<P><<<reduce_blocks(stride), STEP_THREADS, 0, s>>>(f, act, stride, inv_scale, partials);
     return cudaGetLastError();
 }
 
@@ -2287,34 +2345,31 @@ cudaError_t launch_fill_ghosts(void *f, const uint32_t *mask, const int2 *chunks
 inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 template <int P>
-cudaError_t launch_moments(const void *f, const int32_t *soa, int64_t n, int64_t stride, float inv_scale,
-                           double *out4, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_moments<P><<<grid_for(n, 256), 256, 0, s>>>(f, soa, n, stride, inv_scale, out4);
+cudaError_t launch_moments(const void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float inv_scale,
+                           double *rho, double *u, cudaStream_t s) {
+    k_moments<P><<<grid_for(stride, 256), 256, 0, s>>>(f, act, k0, k1, stride, inv_scale, rho, u);
     return cudaGetLastError();
 }
 
 template <int P>
-cudaError_t launch_get_populations(const void *f, const int32_t *soa, int64_t n, int64_t stride, float inv_scale,
-                                   double *out27, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_get_populations<P><<<grid_for(n, 128), 128, 0, s>>>(f, soa, n, stride, inv_scale, out27);
+cudaError_t launch_get_populations(const void *f, const int32_t *act, int64_t stride, float inv_scale, double *out27,
+                                   cudaStream_t s) {
+    k_get_populations<P><<<grid_for(stride, 128), 128, 0, s>>>(f, act, stride, inv_scale, out27);
     return cudaGetLastError();
 }
 
 template <int P>
-cudaError_t launch_set_populations(void *f, const int32_t *soa, int64_t n, int64_t stride, float scale,
-                                   const double *in27, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_set_populations<P><<<grid_for(n, 128), 128, 0, s>>>(f, soa, n, stride, scale, in27);
+cudaError_t launch_set_populations(void *f, const int32_t *act, int64_t stride, float scale, const double *in27,
+                                   cudaStream_t s) {
+    k_set_populations<P><<<grid_for(stride, 128), 128, 0, s>>>(f, act, stride, scale, in27);
     return cudaGetLastError();
 }
 
 template <int P>
-cudaError_t launch_init_eq(void *f, const int32_t *soa, int64_t n, int64_t stride, float scale, const double *rho,
-                           const double *u, double rho0, double ux, double uy, double uz, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_init_eq<P><<<grid_for(n, 128), 128, 0, s>>>(f, soa, n, stride, scale, rho, u, rho0, ux, uy, uz);
+cudaError_t launch_init_eq(void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float scale,
+                           const double *rho, const double *u, double rho0, double ux, double uy, double uz,
+                           cudaStream_t s) {
+    k_init_eq<P><<<grid_for(stride, 128), 128, 0, s>>>(f, act, k0, k1, stride, scale, rho, u, rho0, ux, uy, uz);
     return cudaGetLastError();
 }
 
@@ -2323,18 +2378,17 @@ cudaError_t launch_init_eq(void *f, const int32_t *soa, int64_t n, int64_t strid
     template int step_fluid_blocks<P>(int32_t);                                                                     \
     template int step_stage_blocks<P>(int);                                                                         \
     template int step_prefetch_ahead<P>(bool, bool, int);                                                          \
-    template cudaError_t launch_reduce<P>(const void *, const int32_t *, int64_t, int64_t, float, double *,       \
-                                          cudaStream_t);                                                           \
+    template cudaError_t launch_reduce<P>(const void *, const int32_t *, int64_t, float, double *, cudaStream_t);  \
     template cudaError_t launch_fill_ghosts<P>(void *, const uint32_t *, const int2 *, const int4 *, int32_t,      \
                                                const int4 *, int32_t, int64_t, int32_t, int32_t, int32_t,          \
                                                cudaStream_t);                                                      \
-    template cudaError_t launch_moments<P>(const void *, const int32_t *, int64_t, int64_t, float, double *,       \
-                                           cudaStream_t);                                                          \
-    template cudaError_t launch_get_populations<P>(const void *, const int32_t *, int64_t, int64_t, float,         \
-                                                   double *, cudaStream_t);                                        \
-    template cudaError_t launch_set_populations<P>(void *, const int32_t *, int64_t, int64_t, float,               \
-                                                   const double *, cudaStream_t);                                  \
-    template cudaError_t launch_init_eq<P>(void *, const int32_t *, int64_t, int64_t, float, const double *,       \
-                                           const double *, double, double, double, double, cudaStream_t);
+    template cudaError_t launch_moments<P>(const void *, const int32_t *, int64_t, int64_t, int64_t, float,         \
+                                           double *, double *, cudaStream_t);                                                          \
+    template cudaError_t launch_get_populations<P>(const void *, const int32_t *, int64_t, float, double *,        \
+                                                   cudaStream_t);                                                  \
+    template cudaError_t launch_set_populations<P>(void *, const int32_t *, int64_t, float, const double *,        \
+                                                   cudaStream_t);                                                  \
+    template cudaError_t launch_init_eq<P>(void *, const int32_t *, int64_t, int64_t, int64_t, float,              \
+                                           const double *, const double *, double, double, double, double, cudaStream_t);
 
 }  // namespace lbm

@@ -220,35 +220,46 @@ __host__ __device__ inline int tile_blocks(int64_t ntiles) {
     return (int)((ntiles + STEP_THREADS / 32 - 1) / (STEP_THREADS / 32));
 }
 __host__ __device__ inline int pair_blocks(int64_t nfast) { return (int)((nfast * 16 + STEP_THREADS - 1) / STEP_THREADS); }
+// The kernels below that touch every active cell walk the storage slots, so
+// that the populations are read and written along the rows whatever the row
+// axis; act gives each slot's cell in the active order (-1: none).  One block
+// partial of launch_reduce covers as many slots as reduce_blocks says.
+int reduce_blocks(int64_t nslots);
 template <int P>
-cudaError_t launch_reduce(const void *f, const int32_t *slot_of_active, int64_t n, int64_t stride, float inv_scale,
-                          double *partials, cudaStream_t s);
+cudaError_t launch_reduce(const void *f, const int32_t *act, int64_t stride, float inv_scale, double *partials,
+                          cudaStream_t s);
 // Write the bounce-back ghost slots and periodic-x copies of buffer f from
 // its active cells (after any host-side change of the state).
 template <int P>
 cudaError_t launch_fill_ghosts(void *f, const uint32_t *mask, const int2 *chunks, const int4 *row_nb,
                                int32_t nchunks, const int4 *bnodes, int32_t nbnodes, int64_t stride, int32_t n_row,
                                int32_t periodic_row, int32_t row_axis, cudaStream_t s);
+// rho[n] and u[n][3] (either may be NULL) of the active cells k0 .. k1 - 1 of
+// a stored state; the other entries stay as they are.
 template <int P>
-cudaError_t launch_moments(const void *f, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                           float inv_scale, double *out4, cudaStream_t s);
+cudaError_t launch_moments(const void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float inv_scale,
+                           double *rho, double *u, cudaStream_t s);
 template <int P>
-cudaError_t launch_get_populations(const void *f, const int32_t *slot_of_active, int64_t n,
-                                   int64_t stride, float inv_scale, double *out27, cudaStream_t s);
+cudaError_t launch_get_populations(const void *f, const int32_t *act, int64_t stride, float inv_scale, double *out27,
+                                   cudaStream_t s);
 template <int P>
-cudaError_t launch_set_populations(void *f, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                                   float scale, const double *in27, cudaStream_t s);
+cudaError_t launch_set_populations(void *f, const int32_t *act, int64_t stride, float scale, const double *in27,
+                                   cudaStream_t s);
+// Equilibrium of the active cells k0 .. k1 - 1, from rho[n], u[n][3] or (where
+// they are NULL) from one density and velocity.
 template <int P>
-cudaError_t launch_init_eq(void *f, const int32_t *slot_of_active, int64_t n, int64_t stride,
-                           float scale, const double *rho, const double *u, double rho0,
-                           double ux, double uy, double uz, cudaStream_t s);
+cudaError_t launch_init_eq(void *f, const int32_t *act, int64_t k0, int64_t k1, int64_t stride, float scale,
+                           const double *rho, const double *u, double rho0, double ux, double uy, double uz,
+                           cudaStream_t s);
 
 int fluid_blocks(int32_t nchunks);
 int node_blocks(int64_t n);
 cudaError_t launch_finalize(const double *partials, int nblocks, double *health, uint32_t *status,
                             cudaStream_t s);
-cudaError_t launch_stats_mean(const double *stats, int ncomp, const int32_t *slot_of_active, int64_t n,
-                              int64_t stride, double inv_n, double *out, cudaStream_t s);
+// Means of ncomp accumulator rows per active cell: out[n][ncomp], or with
+// out2 (ncomp = 2) the first row's to out[n] and the second's to out2[n].
+cudaError_t launch_stats_mean(const double *stats, int ncomp, const int32_t *act, int64_t stride, double inv_n,
+                              double *out, double *out2, cudaStream_t s);
 
 // Host-side sparse index (built by geometry.cpp).
 struct HostIndex {

@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(NOALLOC_THREADS)
         const int64_t cell = first + (int64_t)k * NOALLOC_THREADS;
         if (cell >= n) break;
         double d[27], rho, ux, uy, uz, v[6];
-        lbm::load_cell<P>(f, stride, (int)cell, inv_scale, d);
-        lbm::moments_of(d, rho, ux, uy, uz);
+        lbm::load_stored<P>(f, stride, (int)cell, d);
+        lbm::moments_of<P>(d, inv_scale, rho, ux, uy, uz);
         lbm::health_values(rho, ux, uy, uz, v);
         for (int q = 0; q < 6; ++q) hv[q] = (q == 4) ? fmax(hv[q], v[q]) : hv[q] + v[q];
     }
