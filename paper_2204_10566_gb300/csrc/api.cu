@@ -53,6 +53,7 @@ struct lbm_ctx {
     int32_t *d_units_wall = nullptr; // the same without the cells with interpolated walls
     int64_t n_units_wall = 0;
     int stage_blocks = 0;            // grid of the staged kernel
+    int run_blocks = 0, run_mode = -1;  // largest grid of the several-step kernel, and for which collision form
     double *d_partials = nullptr;
     double *d_health = nullptr;
     uint32_t *d_status = nullptr;
@@ -64,7 +65,7 @@ struct lbm_ctx {
     // parameters and state
     lbm_params params{};
     double omega = 0.0;
-    bool ghost1 = true;
+    int mode = RATE_ONE;  // form of the collision
     int prefetch_ahead = 0, prefetch_key = -1;  // L2 prefetch lookahead of the fluid kernel, per variant
     int64_t t = 0;
     int64_t check_every = 0;
@@ -166,7 +167,7 @@ void release_geometry(lbm_ctx *c) {
     dev_free(c, c->d_mask_raw, raw_mask_bytes(c));
     dev_free(c, c->d_row_nb, c->idx.row_nb.size() * 4);
     dev_free(c, c->d_chunks, c->idx.chunks.size() * 8);
-    dev_free(c, c->d_bnodes, c->idx.bnodes.size() * 16);
+    dev_free(c, c->d_bnodes, c->idx.bnodes.size() * NODE_BYTES);
     dev_free(c, c->d_act, ns * 4);
     dev_free(c, c->d_tiles, c->idx.tiles.size() * 4);
     dev_free(c, c->d_units, c->idx.units.size() * 4);
@@ -224,6 +225,38 @@ lbm_status need(lbm_ctx *c, bool geom, bool params, bool state) {
     return LBM_OK;
 }
 
+// Several steps go in one launch (k_run) from RUN_MIN_STEPS on, for lattices
+// whose warp items are at most RUN_ROUNDS for each resident warp (about 310 000
+// cells; measured at k_run).  A launch takes RUN_MAX_STEPS at most, so that it
+// stays well under a second.
+constexpr int RUN_MIN_STEPS = 8, RUN_MAX_STEPS = 4096, RUN_ROUNDS = 4;
+
+// Device records of the inlet/outlet nodes (NODE_INT4S) from the index's list.
+std::vector<int32_t> node_records(const lbm_ctx *c) {
+    const HostIndex &ix = c->idx;
+    const int n[3] = {c->desc.nx, c->desc.ny, c->desc.nz};
+    const bool zrows = ix.row_axis == 2;
+    std::vector<int32_t> out;
+    out.reserve(ix.bnodes.size() * NODE_INT4S * 4);
+    for (const int4 &b : ix.bnodes) {  // row position, row, slot, link word
+        const int ra = b.y % ix.na_e - 1, rb = b.y / ix.na_e - 1;
+        const int at[3] = {zrows ? ra : b.x, zrows ? rb : ra, zrows ? b.x : rb};
+        int to[3] = {at[0], at[1], at[2]};  // the partner, one step along the node's direction
+        const int dir = (int)((uint32_t)b.w >> DIR_SHIFT), axis = dir / 2;
+        to[axis] += dir % 2 ? -1 : 1;
+        to[axis] = (to[axis] + n[axis]) % n[axis];
+        const int pf = zrows ? to[2] : to[0];
+        const int row_f = zrows ? (to[0] + 1) + ix.na_e * (to[1] + 1) : (to[1] + 1) + ix.na_e * (to[2] + 1);
+        const int64_t id = (int64_t)at[0] + (int64_t)n[0] * ((int64_t)at[1] + (int64_t)n[1] * at[2]);
+        const int32_t head[NODE_NB] = {b.z, b.w, b.x, pf, at[0], at[1], (int32_t)(uint32_t)id, (int32_t)(id >> 32)};
+        const int32_t *nb = &ix.row_nb[(size_t)row_f * ROW_RECORD_INTS];
+        out.insert(out.end(), head, head + NODE_NB);
+        out.insert(out.end(), nb, nb + 9);
+        out.resize((out.size() + 3) / 4 * 4, 0);
+    }
+    return out;
+}
+
 // Whether the row axis of the context's index is periodic.
 int periodic_rows(const lbm_ctx *c) {
     return (c->desc.periodic & (c->idx.row_axis == 2 ? LBM_PERIODIC_Z : LBM_PERIODIC_X)) ? 1 : 0;
@@ -242,7 +275,7 @@ bool tiled(const lbm_ctx *c) {
     const FluidKernel k = c->fluid_kernel;
     const bool wanted = k == FluidKernel::TILE || k == FluidKernel::PAIRS ||
                         (k == FluidKernel::AUTO && c->desc.precision == LBM_FP32);
-    return wanted && c->desc.precision != LBM_FP64 && c->ghost1 && !wide_offsets(c) && tile_count(c) > 0;
+    return wanted && c->desc.precision != LBM_FP64 && c->mode == RATE_ONE && !wide_offsets(c) && tile_count(c) > 0;
 }
 // Whether the next FP16S steps run the staged unit kernel (the same
 // conditions, and STAGE_ROUNDS units for each resident warp; steps with a health check keep the chunk kernel, whose partial
@@ -254,12 +287,13 @@ bool staged(const lbm_ctx *c) {
     const int64_t least = c->fluid_kernel == FluidKernel::STAGED ? 1
                           : c->fluid_kernel == FluidKernel::AUTO ? (int64_t)STAGE_ROUNDS * c->stage_blocks * (STEP_THREADS / 32)
                                                                  : INT64_MAX;
-    return c->desc.precision == LBM_FP16S && c->ghost1 && !wide_offsets(c) && c->stage_blocks > 0 &&
+    return c->desc.precision == LBM_FP16S && c->mode == RATE_ONE && !wide_offsets(c) && c->stage_blocks > 0 &&
            unit_count(c) >= least;
 }
 // Words of the status allocation (256 bytes): 0 the status, TICKET_WORD and
-// the next the staged kernel's counters, on a cache line of their own.
-constexpr int TICKET_WORD = 32;
+// the next the staged kernel's counters, BARRIER_WORD and the next those of
+// the several-step kernel, each pair in a sector of its own.
+constexpr int TICKET_WORD = 32, BARRIER_WORD = 48;
 // LBM_FLUID_KERNEL=pairs splits the FP16S fluid cells: pairs of fast tiles
 // run on the pair kernel, the chunks of every other tile on the chunk kernel.
 bool pairs(const lbm_ctx *c) { return c->desc.precision == LBM_FP16S && c->fluid_kernel == FluidKernel::PAIRS; }
@@ -325,6 +359,30 @@ cudaError_t in_parts(lbm_ctx *c, int64_t n, cudaStream_t first_on, cudaStream_t 
     return e != cudaSuccess ? e : (e1 != cudaSuccess ? e1 : e2);
 }
 
+// Grid of the several-step kernel for the next n steps, 0 when they run one
+// by one: FP64 (bound by its arithmetic, not by launches), 64-bit offsets, a
+// fluid kernel asked for by name, a stream that is being captured (one
+// recorded step is then the same kernels as ever), or a larger lattice.
+int run_blocks(lbm_ctx *c, int64_t n) {
+    if (n < RUN_MIN_STEPS || c->desc.precision == LBM_FP64 || wide_offsets(c) || c->fluid_kernel != FluidKernel::AUTO)
+        return 0;
+    if (c->run_mode != c->mode) {
+        c->run_blocks = DISPATCH(c->desc.precision, step_run_blocks, c->mode, c->idx.row_axis, c->desc.device);
+        c->run_mode = c->mode;
+    }
+    const int64_t fluid = c->mode == RATE_ONE ? tile_count(c) : ((int64_t)c->idx.chunks.size() + 3) / 4;
+    const int64_t items = fluid + ((int64_t)c->idx.bnodes.size() + 31) / 32 + (c->n_wnodes + 31) / 32;
+    const int warps = STEP_THREADS / 32;
+    if (items > (int64_t)RUN_ROUNDS * warps * c->run_blocks) return 0;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (cs != cudaStreamCaptureStatusNone) return 0;
+    return (int)std::min<int64_t>(c->run_blocks, (items + warps - 1) / warps);
+}
+
 // Ghost slots and periodic copies of the current buffer from its active cells.
 cudaError_t fill_ghosts(lbm_ctx *c) {
     return DISPATCH(c->desc.precision, launch_fill_ghosts, c->f[c->cur], c->d_mask, c->d_chunks, c->d_row_nb,
@@ -363,7 +421,6 @@ void ctx_step_args(lbm_ctx *c, StepArgs *out) {
     a.nx = c->desc.nx;
     a.ny = c->desc.ny;
     a.nz = c->desc.nz;
-    a.na_e = c->idx.na_e;
     a.n_row = c->idx.n_row;
     a.row_axis = c->idx.row_axis;
     a.periodic_row = periodic_rows(c);
@@ -409,9 +466,9 @@ void ctx_step_args(lbm_ctx *c, StepArgs *out) {
         a.tickets = reinterpret_cast<int32_t *>(c->d_status) + TICKET_WORD;
         a.stage_blocks = c->stage_blocks;
     }
-    const int key = (c->ghost1 ? 2 : 0) + (wide ? 1 : 0);
+    const int key = 2 * c->mode + (wide ? 1 : 0);
     if (c->prefetch_key != key) {
-        c->prefetch_ahead = DISPATCH(c->desc.precision, step_prefetch_ahead, c->ghost1, wide, c->desc.device);
+        c->prefetch_ahead = DISPATCH(c->desc.precision, step_prefetch_ahead, c->mode, wide, c->desc.device);
         c->prefetch_key = key;
     }
     a.prefetch_ahead = c->prefetch_ahead;
@@ -453,7 +510,7 @@ void ctx_advance(lbm_ctx *c, int64_t steps) {
 int64_t ctx_steps(const lbm_ctx *c) { return c->t; }
 int64_t ctx_device_bytes(const lbm_ctx *c) { return c->device_bytes; }
 bool ctx_ready(const lbm_ctx *c) { return c->has_geom && c->has_params && c->has_state; }
-bool ctx_ghost1(const lbm_ctx *c) { return c->ghost1; }
+bool ctx_ghost1(const lbm_ctx *c) { return c->mode == RATE_ONE; }
 int ctx_precision(const lbm_ctx *c) { return c->desc.precision; }
 int64_t ctx_slots(const lbm_ctx *c) { return c->idx.nslots; }
 
@@ -715,7 +772,7 @@ int64_t ctx_footprint(const lbm_desc &d, const HostIndex &ix) {
     const int64_t blocks = std::max<int64_t>(fluid_blocks((int32_t)ix.chunks.size()) + node_blocks((int64_t)ix.bnodes.size()),
                                              reduce_blocks(ix.nslots));
     return 2 * pop + (ix.nslots + 2 * MASK_MARGIN) * 4 + (int64_t)ix.row_nb.size() * 4 + (int64_t)ix.chunks.size() * 8 +
-           (int64_t)ix.bnodes.size() * 16 + ix.nslots * 4 + (int64_t)ix.tiles.size() * 4 +
+           (int64_t)(ix.bnodes.size() * NODE_BYTES) + ix.nslots * 4 + (int64_t)ix.tiles.size() * 4 +
            (int64_t)ix.units.size() * 4 + (int64_t)ix.pair_items.size() * 8 + (int64_t)ix.rest_chunks.size() * 8 +
            blocks * REDUCE_SLOTS * 8 + 64 + 256;
 }
@@ -728,6 +785,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     const size_t ns = (size_t)c->idx.nslots;
     c->fluid_blocks = DISPATCH(c->desc.precision, step_fluid_blocks, (int32_t)c->idx.chunks.size());
     c->nblocks = partial_capacity(c, 0);
+    c->run_mode = -1;
     c->stage_blocks = DISPATCH(c->desc.precision, step_stage_blocks, c->desc.device);
     for (int k = 0; k < 2; ++k) {
         c->f_raw[k] = dev_alloc(c, raw_pop_bytes(c));
@@ -737,7 +795,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->d_mask = c->d_mask_raw ? c->d_mask_raw + MASK_MARGIN : nullptr;
     c->d_row_nb = (int4 *)dev_alloc(c, c->idx.row_nb.size() * 4);
     c->d_chunks = (int2 *)dev_alloc(c, c->idx.chunks.size() * 8);
-    c->d_bnodes = (int4 *)dev_alloc(c, c->idx.bnodes.size() * 16);
+    c->d_bnodes = (int4 *)dev_alloc(c, c->idx.bnodes.size() * NODE_BYTES);
     c->d_act = (int32_t *)dev_alloc(c, ns * 4);
     c->d_tiles = (int32_t *)dev_alloc(c, c->idx.tiles.size() * 4);
     c->d_units = (int32_t *)dev_alloc(c, c->idx.units.size() * 4);
@@ -759,9 +817,9 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     CK(cudaMemcpyAsync(c->d_chunks, c->idx.chunks.data(), c->idx.chunks.size() * 8, cudaMemcpyHostToDevice,
                        c->stream),
        "copy chunks");
-    if (!c->idx.bnodes.empty())
-        CK(cudaMemcpyAsync(c->d_bnodes, c->idx.bnodes.data(), c->idx.bnodes.size() * 16, cudaMemcpyHostToDevice,
-                           c->stream),
+    const std::vector<int32_t> nodes = node_records(c);
+    if (!nodes.empty())
+        CK(cudaMemcpyAsync(c->d_bnodes, nodes.data(), nodes.size() * 4, cudaMemcpyHostToDevice, c->stream),
            "copy boundary nodes");
     std::vector<int32_t> act(ns, -1);
     for (int64_t k = 0; k < c->idx.n_active; ++k) act[(size_t)c->idx.slot_of_active[(size_t)k]] = (int32_t)k;
@@ -891,7 +949,8 @@ lbm_status lbm_set_params(lbm_ctx *c, const lbm_params *p) {
     if (c->params.axis_x < 0.0) c->params.axis_x = c->desc.nx / 2.0;
     if (c->params.axis_y < 0.0) c->params.axis_y = c->desc.ny / 2.0;
     c->omega = omega;
-    c->ghost1 = g[0] == 1.0 && g[1] == 1.0 && g[2] == 1.0 && g[3] == 1.0;
+    const auto all = [&g](double r) { return g[0] == r && g[1] == r && g[2] == r && g[3] == r; };
+    c->mode = all(1.0) ? RATE_ONE : (all(omega) ? RATE_BGK : RATE_GENERAL);
     c->has_params = true;
     c->err.clear();
     return LBM_OK;
@@ -1025,8 +1084,33 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
     DeviceGuard g(c->desc.device);
     StepArgs a{};
     lbm::ctx_step_args(c, &a);
+    const int run_grid = run_blocks(c, n);
     for (int64_t k = 0; k < n; ++k) {
         const int64_t t_new = c->t + 1;
+        // steps up to the next health check in one launch
+        const int64_t plain = std::min(n - k, c->check_every > 0 ? (c->check_every - t_new % c->check_every) % c->check_every
+                                                                 : (int64_t)RUN_MAX_STEPS);
+        if (run_grid > 0 && plain >= RUN_MIN_STEPS) {
+            const int m = (int)std::min<int64_t>(plain, RUN_MAX_STEPS);
+            StepArgs r = a;
+            r.fin = c->f[c->cur];
+            r.fout = c->f[1 - c->cur];
+            r.t_new = t_new;
+            r.tiles = c->d_tiles_wall ? c->d_tiles_wall : c->d_tiles;  // whatever the per-step kernel takes
+            r.ntiles = (int32_t)tile_count(c);
+            RunArgs run{m, 0, c->stats_start, c->stats_stride, reinterpret_cast<int32_t *>(c->d_status) + BARRIER_WORD};
+            if (c->stats_on) run.stats_flags = STEP_STATS | (c->stats_ncomp == STATS_FULL ? STEP_STATS_FULL : 0);
+            CK(DISPATCH(c->desc.precision, launch_run, r, run, c->mode, run_grid, c->stream), "steps kernel");
+            ++c->kernel_launches;
+            if (c->stats_on) {  // sampled steps among t_new .. t_new + m - 1
+                const int64_t lo = std::max(t_new, c->stats_start) - c->stats_start, hi = t_new + m - 1 - c->stats_start;
+                if (hi >= lo) c->stats_samples += hi / c->stats_stride - (lo + c->stats_stride - 1) / c->stats_stride + 1;
+            }
+            if (m & 1) c->cur = 1 - c->cur;
+            c->t += m;
+            k += m - 1;
+            continue;
+        }
         a.fin = c->f[c->cur];
         a.fout = c->f[1 - c->cur];
         a.t_new = t_new;
@@ -1038,7 +1122,7 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
             ++c->stats_samples;
         }
         int launched = 0;
-        CK(DISPATCH(c->desc.precision, launch_step, a, c->ghost1, c->stream, &launched, &c->side), "step kernel");
+        CK(DISPATCH(c->desc.precision, launch_step, a, c->mode, c->stream, &launched, &c->side), "step kernel");
         c->kernel_launches += launched;
         if (check) {
             CK(launch_finalize(c->d_partials, step_partials(c), c->d_health, c->d_status, c->stream), "finalize");

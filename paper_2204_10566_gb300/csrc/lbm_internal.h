@@ -105,6 +105,13 @@ std::vector<int2> build_pair_items(const std::vector<int32_t> &tiles);
 std::vector<int2> build_rest_chunks(const std::vector<int2> &chunks, const std::vector<int32_t> &tiles,
                                     const std::vector<int2> &pairs);
 
+// Inlet/outlet node records on the device, 80 bytes each: slot, link word, row
+// position, its interior partner's row position; x, y and the box index (two
+// words) of the node; the nine neighbour bases of the partner's row.  One
+// record load and the partner's pulls are the only dependent loads of a node.
+constexpr int NODE_INT4S = 5, NODE_NB = 8;
+constexpr size_t NODE_BYTES = NODE_INT4S * 16;
+
 // Unit records of the staged FP16S fluid kernel: a unit is the chunks of one
 // row within the UNIT_CELLS positions from p0, 128 bytes of every FP16
 // population array.  Units start on a multiple of UNIT_ALIGN slots, one
@@ -130,6 +137,10 @@ constexpr int UNIT_PLAIN = 1, UNIT_WRAP = 2;
 constexpr int STAGE_ROUNDS = 6;
 std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
                                  const std::vector<uint32_t> &mask, int n_row, bool periodic_row);
+
+// Form of the collision: general ghost rates (the 27-moment cascade), all
+// ghost rates 1 (the default), or all ghost rates equal to omega (lattice BGK).
+enum : int { RATE_GENERAL = 0, RATE_ONE = 1, RATE_BGK = 2 };
 
 // Fluid kernel of the FP32 / FP16S steps: AUTO is the tile kernel in FP32
 // and, in FP16S, the staged unit kernel for larger lattices and the chunk
@@ -159,12 +170,11 @@ struct alignas(16) StepArgs {
     const int4 *row_nb;     // [rows][3] row records
     const int2 *chunks;     // chunk records (fluid cells)
     int32_t nchunks;
-    const int4 *bnodes;     // boundary nodes (x, row, slot, link word)
+    const int4 *bnodes;     // [nbnodes][NODE_INT4S] inlet/outlet node records
     int32_t nbnodes;
     int32_t fluid_blocks;   // blocks of the fluid kernel (offset of the boundary kernel's partials)
     uint32_t *status;       // bit 1: a bounded device wait gave up
     int32_t nx, ny, nz;     // box (physical x, y, z)
-    int32_t na_e;           // extended extent of the first cross axis (decodes a row index)
     int32_t n_row;          // cells along the row axis
     int32_t row_axis;       // 0: rows along x, 2: rows along z
     int32_t flags;          // STEP_REDUCE | STEP_STATS
@@ -195,18 +205,36 @@ struct alignas(16) StepArgs {
     int32_t nitems;
 };
 
+// What several steps in one launch need beside the first step's arguments:
+// the step count, when they sample statistics, and the two barrier words
+// (zero between launches).
+struct RunArgs {
+    int32_t steps;
+    int32_t stats_flags;  // STEP_STATS (| STEP_STATS_FULL), or 0
+    int64_t stats_start, stats_stride;
+    int32_t *barrier;
+};
+// Polls of a barrier wait before it gives up (some seconds).
+constexpr int RUN_SPIN_LIMIT = 1 << 22;
+
 // Launchers, one set per storage precision (P = 0 FP64, 1 FP32, 2 FP16S).
 // Offsets into a population buffer fit in 32 bits (unsigned) when
 // 27 * slots < 2^32; larger lattices use 64-bit offsets.
 constexpr int64_t MAX_SLOTS_32 = (int64_t)0xFFFFFFFFu / 27 - 64;
 
 template <int P>
-cudaError_t launch_step(const StepArgs &a, bool ghost1, cudaStream_t s, int *launches = nullptr,
+cudaError_t launch_step(const StepArgs &a, int mode, cudaStream_t s, int *launches = nullptr,
                         const SideStream *side = nullptr);
 // L2 prefetch lookahead of the fluid kernel in blocks: a fixed share of the
 // blocks resident on the device at once (occupancy x SM count); 0 = off.
 template <int P>
-int step_prefetch_ahead(bool ghost1, bool wide, int device);
+int step_prefetch_ahead(int mode, bool wide, int device);
+// Several steps in one cooperative launch: the blocks resident on the device
+// at once (0: none for this precision or device), and the launch.
+template <int P>
+int step_run_blocks(int mode, int row_axis, int device);
+template <int P>
+cudaError_t launch_run(const StepArgs &a, const RunArgs &run, int mode, int blocks, cudaStream_t s);
 // Blocks of the staged unit kernel that are resident on the device at once
 // (0 if it has none for this precision).
 template <int P>
