@@ -78,20 +78,63 @@ struct Frame {
     }
 };
 
+// The flags copied into storage order, rows along p contiguous, with a layer
+// of halo on every side that holds what a pull from there meets: the wrapped
+// cell on a periodic axis, SOLID outside otherwise.  The index is built from
+// this copy row by row instead of jumping through the box a plane per cell,
+// and near() spares the 27 links of the cells that have no solid cell around
+// them, nearly all: 1.5 -> 0.3 s for the 96x96x800 nozzle.
+struct Packed : Frame {
+    int64_t sa, sb;  // strides of a and b
+    std::vector<uint8_t> cell, close;
+    Packed(const Frame &f, const uint8_t *flags) : Frame(f), sa(f.np + 2), sb((int64_t)(f.np + 2) * (f.na + 2)) {
+        cell.assign((size_t)(sb * (nb + 2)), LBM_SOLID);
+        constexpr int TILE = 64;  // cells of the row axis and of x copied together (rows along z: a transpose)
+        for (int b = 0; b < nb; ++b)
+            for (int p0 = 0; p0 < np; p0 += TILE)
+                for (int a0 = 0; a0 < na; a0 += TILE)
+                    for (int p = p0; p < std::min(np, p0 + TILE); ++p)
+                        for (int a = a0; a < std::min(na, a0 + TILE); ++a)
+                            cell[(size_t)box(p, a, b)] = flags[Frame::box(p, a, b)];
+        for (int b = 0; pp && b < nb; ++b)
+            for (int a = 0; a < na; ++a) cell[(size_t)box(-1, a, b)] = cell[(size_t)box(np - 1, a, b)], cell[(size_t)box(np, a, b)] = cell[(size_t)box(0, a, b)];
+        auto copy = [&](int64_t to, int64_t from, int64_t n) { memcpy(&cell[(size_t)to], &cell[(size_t)from], (size_t)n); };
+        for (int b = 0; pa && b < nb; ++b) copy(box(-1, -1, b), box(-1, na - 1, b), sa), copy(box(-1, na, b), box(-1, 0, b), sa);
+        if (pb) copy(box(-1, -1, -1), box(-1, -1, nb - 1), sb), copy(box(-1, -1, nb), box(-1, -1, 0), sb);
+        // close: a solid cell among the 27 around, by one pass per axis
+        const int64_t n = (int64_t)cell.size();
+        std::vector<uint8_t> t((size_t)n, 0), u((size_t)n, 0);
+        for (int64_t k = 1; k + 1 < n; ++k) t[(size_t)k] = (cell[(size_t)k - 1] == LBM_SOLID) | (cell[(size_t)k] == LBM_SOLID) | (cell[(size_t)k + 1] == LBM_SOLID);
+        for (int64_t k = sa; k + sa < n; ++k) u[(size_t)k] = t[(size_t)(k - sa)] | t[(size_t)k] | t[(size_t)(k + sa)];
+        close.assign((size_t)n, 0);
+        for (int64_t k = sb; k + sb < n; ++k) close[(size_t)k] = u[(size_t)(k - sb)] | u[(size_t)k] | u[(size_t)(k + sb)];
+    }
+    int64_t box(int p, int a, int b) const { return (int64_t)(p + 1) + sa * (a + 1) + sb * (b + 1); }
+    bool near(int p, int a, int b) const { return close[(size_t)box(p, a, b)] != 0; }
+    // whether the pull source of direction i of the cell at k = box(p, a, b) is solid or outside
+    bool wall(int64_t k, int i) const {
+        int cp, ca, cb;
+        dir(i, cp, ca, cb);
+        return cell[(size_t)(k - cp - sa * ca - sb * cb)] == LBM_SOLID;
+    }
+};
+
 }  // namespace
 
-std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int periodic, HostIndex &out,
+std::string build_index(const uint8_t *box_flags, int nx, int ny, int nz, int periodic, HostIndex &out,
                         int64_t max_slots, int row_axis) {
     const int64_t ncell = (int64_t)nx * ny * nz;
     for (int64_t b = 0; b < ncell; ++b)
-        if (flags[b] > LBM_OUTLET) {
+        if (box_flags[b] > LBM_OUTLET) {
             char msg[128];
-            snprintf(msg, sizeof msg, "flag value %d at cell %lld is not SOLID/FLUID/INLET/OUTLET", (int)flags[b],
+            snprintf(msg, sizeof msg, "flag value %d at cell %lld is not SOLID/FLUID/INLET/OUTLET", (int)box_flags[b],
                      (long long)b);
             return msg;
         }
     out = HostIndex();
-    const Frame F(choose_row_axis(nx, ny, nz, row_axis), nx, ny, nz, periodic);
+    const Frame frame(choose_row_axis(nx, ny, nz, row_axis), nx, ny, nz, periodic);
+    const Packed F(frame, box_flags);
+    const uint8_t *flags = F.cell.data();  // in storage order: flags[F.box(p, a, b)]
     if (F.np > (int)CHUNK_X0_MASK) return "lattice too long along its row axis (at most 2^20 - 1 cells)";
     const int na_e = F.na + 2, nb_e = F.nb + 2;
     const int64_t nrows = (int64_t)na_e * nb_e;
@@ -136,9 +179,11 @@ std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int period
                 }
                 if (F.pp && p == F.np - 1) need(r, -1);
                 if (F.pp && p == 0) need(r, F.np);
-                if (fl != LBM_FLUID) continue;
+                if (fl != LBM_FLUID || !F.near(p, a, b)) continue;
+                const int64_t k = F.box(p, a, b);
                 for (int i = 0; i < 27; ++i) {
                     int cp, ca, cb, as, bs;
+                    if (!F.wall(k, i)) continue;
                     F.dir(i, cp, ca, cb);
                     if (source(p - cp, a - ca, b - cb, as, bs) == LBM_SOLID) need(row_of(as, bs), p - cp);
                 }
@@ -179,29 +224,38 @@ std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int period
             }
         }
 
-    // link words, inlet/outlet nodes and the active order (increasing box index)
+    // link words of the fluid cells
+    for (int b = 0; b < F.nb; ++b)
+        for (int a = 0; a < F.na; ++a)
+            for (int p = 0; p < F.np; ++p) {
+                if (flags[F.box(p, a, b)] != LBM_FLUID) continue;
+                uint32_t m = 0;
+                const int64_t k = F.box(p, a, b);
+                for (int i = 0; F.close[(size_t)k] && i < 27; ++i)
+                    if (F.wall(k, i)) {
+                        m |= 1u << i;
+                        ++out.n_ghost;
+                    }
+                out.mask[(size_t)(base[row_of(a, b)] + p)] = m | ((uint32_t)TYPE_FLUID << TYPE_SHIFT);
+            }
+
+    // inlet/outlet nodes and the active order (increasing box index)
     static const int dirs[6][3] = {{1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1}};
+    const size_t n_active = (size_t)(ncell - std::count(box_flags, box_flags + ncell, (uint8_t)LBM_SOLID));
+    out.slot_of_active.reserve(n_active);
+    out.box_of_active.reserve(n_active);
     for (int z = 0; z < nz; ++z)
         for (int y = 0; y < ny; ++y)
             for (int x = 0; x < nx; ++x) {
                 const int64_t bx = box_index(x, y, z, nx, ny);
-                const int fl = flags[bx];
+                const int fl = box_flags[bx];
                 if (fl == LBM_SOLID) continue;
                 int p, a, b;
                 F.from_xyz(x, y, z, p, a, b);
                 const int32_t slot = base[row_of(a, b)] + p;
-                uint32_t m = 0, type = TYPE_FLUID, dir = 0;
-                if (fl == LBM_FLUID) {
-                    for (int i = 0; i < 27; ++i) {
-                        int cp, ca, cb, as, bs;
-                        F.dir(i, cp, ca, cb);
-                        if (source(p - cp, a - ca, b - cb, as, bs) == LBM_SOLID) {
-                            m |= 1u << i;
-                            ++out.n_ghost;
-                        }
-                    }
-                } else {
-                    type = fl == LBM_INLET ? TYPE_INLET : TYPE_OUTLET;
+                if (fl != LBM_FLUID) {
+                    const uint32_t type = fl == LBM_INLET ? TYPE_INLET : TYPE_OUTLET;
+                    uint32_t dir = 0;
                     int count = 0;
                     for (int k = 0; k < 6; ++k) {
                         int dp, da, db, as, bs;
@@ -218,10 +272,9 @@ std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int period
                                  fl == LBM_INLET ? "inlet" : "outlet", x, y, z, count);
                         return msg;
                     }
-                }
-                out.mask[(size_t)slot] = m | (type << TYPE_SHIFT) | (dir << DIR_SHIFT);
-                if (type != TYPE_FLUID)
+                    out.mask[(size_t)slot] = (type << TYPE_SHIFT) | (dir << DIR_SHIFT);
                     out.bnodes.push_back(make_int4(p, (int)row_of(a, b), slot, (int)out.mask[(size_t)slot]));
+                }
                 out.slot_of_active.push_back(slot);
                 out.box_of_active.push_back(bx);
             }
@@ -237,9 +290,12 @@ std::string build_index(const uint8_t *flags, int nx, int ny, int nz, int period
             for (int p = 0; p < F.np; ++p) {
                 const int fl = flags[F.box(p, a, b)];
                 if (fl == LBM_SOLID) continue;
-                const int64_t r = row_of(a, b);
+                const bool end = F.pp && (p == 0 || p == F.np - 1);  // has wrap-around copies
+                if (!end && (fl != LBM_FLUID || !F.near(p, a, b))) continue;
+                const int64_t r = row_of(a, b), k = F.box(p, a, b);
                 for (int i = 0; i < 27; ++i) {
                     int cp, ca, cb, as, bs;
+                    if (!end && !F.wall(k, i)) continue;
                     F.dir(i, cp, ca, cb);
                     if (F.pp && p == F.np - 1 && cp == 1) out.mask[(size_t)(base[r] - 1)] |= 1u << i;
                     if (F.pp && p == 0 && cp == -1) out.mask[(size_t)(base[r] + F.np)] |= 1u << i;
