@@ -377,12 +377,12 @@ lbm_status lbm_totals_noalloc(const void *f, int32_t precision, float fp16_scale
 lbm_status lbm_layout_info(lbm_ctx *ctx, int64_t *slots, int64_t *buffer_bytes, int64_t *device_bytes);
 
 /* Kernels lbm_step has launched on this context since its creation, counted
- * at each launch: the fluid kernel(s) of the variant that runs (FP32: the
- * tile kernel; FP16S: the chunk kernel and the pair kernel; FP64 and general
- * ghost rates: the chunk kernel), the interpolated-wall kernel, the
- * inlet/outlet kernel and, on health-check steps, the final reduction pass.
- * The difference of two readings is the launch count of the steps between
- * them.  LBM_ERR_ARG if ctx or n is NULL. */
+ * at each launch.  Steps taken one by one: the fluid kernel(s) of the variant
+ * that runs, the interpolated-wall kernel, the inlet/outlet kernel and, on
+ * health-check steps, the final reduction pass.  On a lattice of up to about
+ * 310 000 cells, runs of eight or more FP32 / FP16S steps between health
+ * checks are one launch each.  The difference of two readings is the launch
+ * count of the steps between them.  LBM_ERR_ARG if ctx or n is NULL. */
 lbm_status lbm_kernel_launches(lbm_ctx *ctx, int64_t *n);
 
 /* ------------------------------------------------------------------ serving
@@ -390,8 +390,8 @@ lbm_status lbm_kernel_launches(lbm_ctx *ctx, int64_t *n);
  * sizes, Re, step counts and storage precisions) on one GPU with continuous
  * batching: queued requests are admitted into resident slots as memory and
  * slots free up (admission by exact device footprint against a budget),
- * and every scheduling tick advances all resident lattices together with one
- * persistent multi-lattice launch per precision and step, replayed from a
+ * and every scheduling tick advances all resident lattices together in one
+ * cooperative launch that takes all of the tick's steps, replayed from a
  * captured CUDA graph.  Finished lattices are read back (rho, u) and freed.
  * Each lattice is advanced by exactly the arithmetic of lbm_step, so a
  * result does not depend on what else is resident.  (This is a service

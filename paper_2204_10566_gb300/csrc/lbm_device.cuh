@@ -1518,17 +1518,28 @@ struct SharedStore {
     }
 };
 
-// One warp's update of tile t (lane = the warp lane, out = the warp's
-// shared-memory slice of TileOut<P>::ELEMS elements).
-template <int P, int AX, bool CG = false>
-__device__ __forceinline__ void tile_update(const StepArgs &a, int t, int lane, typename TileOut<P>::T *out,
+// The record of a tile (48 bytes; the same for every lane).
+struct TileRec {
+    int4 r0, r1, r2;
+    TileRec() = default;
+    __device__ __forceinline__ TileRec(const int32_t *tiles, int t) {
+        const int4 *rec = reinterpret_cast<const int4 *>(tiles) + 3 * (size_t)t;
+        r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
+    }
+};
+
+// One warp's update of a tile (lane = the warp lane, out = the warp's
+// shared-memory slice of TileOut<P>::ELEMS elements).  Without FAST every tile
+// takes the line sink, and out is not used: half the code, for kernels that
+// otherwise wait on the instruction cache.
+template <int P, int AX, bool CG = false, bool FAST = true>
+__device__ __forceinline__ void tile_update(const StepArgs &a, const TileRec &rec, int lane, typename TileOut<P>::T *out,
                                             double (&hv)[6]) {
     using O = TileOut<P>;
     using T = typename O::T;
     using R = typename Storage<P>::R;
     constexpr bool RAW = Storage<P>::SCALED;
-    const int4 *rec = reinterpret_cast<const int4 *>(a.tiles) + 3 * (size_t)t;
-    const int4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2);
+    const int4 &r0 = rec.r0, &r1 = rec.r1, &r2 = rec.r2;
     const int nb[9] = {r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
     const bool fast = ((uint32_t)r0.x & TILE_FAST) != 0u;
     const int p0 = (int)((uint32_t)r0.x & CHUNK_X0_MASK);
@@ -1537,7 +1548,7 @@ __device__ __forceinline__ void tile_update(const StepArgs &a, int t, int lane, 
     R d[27];
     gather<P, false, AX, RAW, CG>(a, nb, x, d);  // every lane's pulls lie inside the buffer margins
     R rho, ux, uy, uz;
-    if (fast) {
+    if (FAST && fast) {
         const SharedStore<P, RAW> sink{a, slot, out + lane};
         collide_ghost1<R, RAW, SharedStore<P, RAW>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
                                                     R(a.scale), &sink);
@@ -1575,7 +1586,7 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_step_tile
     const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
     const int t = (int)blockIdx.x * (STEP_THREADS / 32) + warp;
     double hv[6] = {0, 0, 0, 0, 0, 0};
-    if (t < a.ntiles) tile_update<P, AX>(a, t, lane, staged_out[warp], hv);  // uniform over the warp
+    if (t < a.ntiles) tile_update<P, AX>(a, TileRec(a.tiles, t), lane, staged_out[warp], hv);  // uniform over the warp
     if (a.flags & STEP_REDUCE) block_reduce_write(hv, a.partials);
 }
 
@@ -1967,11 +1978,13 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STAGE_BLOCKS) k_step_units(c
 // in the per-step kernels, to the same bits.
 //
 // Measured per step, one launch each and in one: laminar nozzle 24x24x160 FP32
-// 10.7 -> 8.0 us, FP16S 12.0 -> 8.3; pipe of 237 000 cells FP32 14.0 -> 11.8;
-// 64^3 lattice BGK 14.4 -> 11.6 (FP32 per step 17.4 with the cascade); smooth
-// nozzle of 226 000 cells 24.1 -> 18.0; 32^3 box 6.2 -> 4.1, of which about
+// 10.7 -> 7.6 us, FP16S 12.0 -> 8.4; pipe of 237 000 cells FP32 14.0 -> 11.4;
+// 64^3 lattice BGK 14.4 -> 11.1 (FP32 per step 17.4 with the cascade); smooth
+// nozzle of 226 000 cells 24.1 -> 15.8; 32^3 box 6.2 -> 3.9, of which about
 // 1.5 us is the barrier.  At 80^3 (6.6 rounds) both take 29 us.  4 blocks per
-// SM (128 registers, no spills); 5 and 8 spill and take 10 to 40 % longer.
+// SM (128 registers, no spills); 5 and 8 spill and take 10 to 40 % longer.  The
+// line sink for every tile: with the fast tiles' path as well the nozzle takes
+// 8.3 us.
 #ifndef LBM_RUN_BLOCKS
 #define LBM_RUN_BLOCKS 4
 #endif
@@ -2000,13 +2013,10 @@ __device__ __forceinline__ bool grid_barrier(int32_t *word, int rounds, uint32_t
 template <int P, int G, int AX>
 __global__ void __launch_bounds__(STEP_THREADS, LBM_RUN_BLOCKS) k_run(const StepArgs a0, const RunArgs run) {
     constexpr bool TILES = G == RATE_ONE;
-    using O = TileOut<P>;
-    __shared__ __align__(16) typename O::T staged_out[TILES ? STEP_THREADS / 32 : 1][TILES ? O::ELEMS : 1];
     const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
     // warps of one block take items far apart, so that the nodes spread over the SMs
     const int first = warp * (int)gridDim.x + (int)blockIdx.x, stride = (int)gridDim.x * (STEP_THREADS / 32);
     const int nodes = (a0.nbnodes + 31) / 32, walls = (a0.nwnodes + 31) / 32;
-    const int items = nodes + walls + (TILES ? a0.ntiles : (a0.nchunks + 3) / 4);
     StepArgs a = a0;
     double hv[6];
     for (int s = 0; s < run.steps; ++s) {
@@ -2015,17 +2025,27 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_RUN_BLOCKS) k_run(const Step
         a.fout = s & 1 ? const_cast<void *>(a0.fin) : a0.fout;
         const int64_t since = a.t_new - run.stats_start;
         a.flags = run.stats_flags && since >= 0 && since % run.stats_stride == 0 ? run.stats_flags : 0;
-        for (int i = first; i < items; i += stride) {
-            if (i < nodes) {
-                const int k = 32 * i + lane;
-                if (k < a.nbnodes) boundary_node<P, G, false, AX, true>(a, k, hv);
-            } else if (i < nodes + walls) {
-                const int k = 32 * (i - nodes) + lane;
-                if (k < a.nwnodes) wall_cell<P, G, false, AX, true>(a, k, hv);
-            } else if constexpr (TILES) {
-                tile_update<P, AX, true>(a, i - nodes - walls, lane, staged_out[warp], hv);
-            } else {
-                const int chunk = 4 * (i - nodes - walls) + lane / CHUNK;
+        int i = first;
+        for (; i < nodes; i += stride) {
+            const int k = 32 * i + lane;
+            if (k < a.nbnodes) boundary_node<P, G, false, AX, true>(a, k, hv);
+        }
+        for (; i < nodes + walls; i += stride) {
+            const int k = 32 * (i - nodes) + lane;
+            if (k < a.nwnodes) wall_cell<P, G, false, AX, true>(a, k, hv);
+        }
+        i -= nodes + walls;
+        if constexpr (TILES) {  // the next tile's record is on its way while a tile is updated
+            TileRec next;
+            if (i < a.ntiles) next = TileRec(a.tiles, i);
+            for (; i < a.ntiles; i += stride) {
+                const TileRec rec = next;
+                if (i + stride < a.ntiles) next = TileRec(a.tiles, i + stride);
+                tile_update<P, AX, true, false>(a, rec, lane, nullptr, hv);
+            }
+        } else {
+            for (; i < (a.nchunks + 3) / 4; i += stride) {
+                const int chunk = 4 * i + lane / CHUNK;
                 if (chunk < a.nchunks) fluid_cell<P, G, false, AX, true>(a, chunk, lane % CHUNK, hv);
             }
         }

@@ -5,14 +5,14 @@
 // sparse index while the GPU is busy.  lbm_server_tick admits ready requests
 // into resident slots by exact device footprint against the budget, then
 // advances every resident lattice by up to steps_per_tick steps with one
-// captured CUDA graph: per step, one persistent multi-lattice fluid launch
-// and one boundary launch per precision group.  The blocks of those launches
-// walk a tile list that spans all resident lattices (a tile is one block's
-// worth of chunks of one lattice); the lattice of a tile is found by binary
-// search in a per-tick table that the graph copies to the device first.  The
-// table changes every tick, the graph never does.  Each cell is updated by
-// the same device code as lbm_step, so a lattice's result does not depend on
-// what else is resident.
+// captured CUDA graph, whose one kernel takes all steps of the tick: a
+// cooperative launch with a barrier over the grid between steps, whose warps
+// walk the inlet/outlet nodes and the fluid tiles of all resident lattices of
+// both precisions.  The lattice of a warp's item is found by binary search in
+// a per-tick table that the graph copies to the device first.  The table
+// changes every tick, the graph never does.  Each cell is updated by the same
+// device code as lbm_step, so a lattice's result does not depend on what else
+// is resident.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,33 +34,36 @@ namespace lbm {
 // other value must be a positive power of two; returns 0 when invalid.
 float resolve_fp16_scale(float s);
 
-// A context's step arguments in the chunk kernel's view (api.cu): every
-// chunk and every inlet/outlet node, whichever fluid kernel its own steps run.
-void ctx_chunk_step_args(lbm_ctx *c, StepArgs *out);
+// A context's step arguments in the tile view (api.cu): every fluid tile and
+// every inlet/outlet node, whichever fluid kernel its own steps run.
+void ctx_tile_step_args(lbm_ctx *c, StepArgs *out);
 
 constexpr int MAX_SLOTS = LBM_SERVER_MAX_SLOTS;
-constexpr int NGROUPS = 2;  // 0: FP32, 1: FP16S
 
 struct alignas(16) DomainEntry {
     StepArgs a;        // state at the start of the tick: fin is the current buffer
     int64_t t_base;    // steps done before the tick
     int32_t steps;     // steps this lattice takes in the tick
-    int32_t tile_begin, btile_begin, pad;
+    int32_t precision; // LBM_FP32 or LBM_FP16S
+    int32_t tile_begin, node_begin;  // its first tile item and its first node item (32 nodes) in the tick's list
 };
 
-struct alignas(16) GroupTable {
-    int32_t n_domains, n_tiles, n_btiles, pad;
+struct alignas(16) TickTable {
+    int32_t n_domains, n_tiles, n_nodes, steps;  // steps: the most any lattice takes
     DomainEntry d[MAX_SLOTS];
 };
 
-// Lattice of a tile: the last entry whose first tile is <= tile.
-template <bool BND>
-__device__ __forceinline__ int find_domain(const GroupTable *tab, int tile) {
-    int lo = 0, hi = tab->n_domains - 1;
+// Words after the health flags (one per domain): the tick's status, then the
+// two barrier words.
+constexpr int STATUS_WORD = MAX_SLOTS, BARRIER_WORDS = MAX_SLOTS + 8, FLAG_WORDS = MAX_SLOTS + 16;
+
+// Lattice of an item: the last entry whose first item is <= item.
+template <bool NODES>
+__device__ __forceinline__ int find_domain(const DomainEntry *d, int n, int item) {
+    int lo = 0, hi = n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        const int begin = BND ? tab->d[mid].btile_begin : tab->d[mid].tile_begin;
-        if (begin <= tile)
+        if ((NODES ? d[mid].node_begin : d[mid].tile_begin) <= item)
             lo = mid;
         else
             hi = mid - 1;
@@ -68,81 +71,107 @@ __device__ __forceinline__ int find_domain(const GroupTable *tab, int tile) {
     return lo;
 }
 
-// Step k of the tick for the tile's lattice: copy its arguments to shared
-// memory, swap the buffers on odd steps, set the step number (inlet noise).
-// The lattice's last step of the tick is its health check: every cell then
-// computes its non-finite flag (STEP_REDUCE), and a.status points at the
-// lattice's word of the server's health-flag array.
-__device__ __forceinline__ bool load_domain(const DomainEntry &e, int k, StepArgs &sa) {
-    if (k >= e.steps) return false;
-    for (int w = threadIdx.x; w < (int)(sizeof(StepArgs) / 16); w += blockDim.x)
-        reinterpret_cast<int4 *>(&sa)[w] = reinterpret_cast<const int4 *>(&e.a)[w];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (k & 1) {
-            const void *t = sa.fin;
-            sa.fin = sa.fout;
-            sa.fout = const_cast<void *>(t);
-        }
-        sa.t_new = e.t_base + k + 1;
-        sa.flags = k == e.steps - 1 ? STEP_REDUCE : 0;
-    }
-    __syncthreads();
-    return true;
+// Health check of an item on its lattice's last step of the tick (STEP_REDUCE:
+// record_cell sets hv[5] for a non-finite density or velocity): one atomic
+// per warp that saw one.
+__device__ __forceinline__ void flag_non_finite(const StepArgs &a, double bad) {
+    if (!(a.flags & STEP_REDUCE)) return;  // uniform over the warp
+    if (__any_sync(0xffffffffu, bad != 0.0) && (threadIdx.x & 31) == 0) atomicOr(a.status, 1u);
 }
 
-// Health check of a tile on its lattice's check step: one atomic per warp
-// that saw a non-finite density or velocity (hv[5], set by record_cell).
-__device__ __forceinline__ void flag_non_finite(const StepArgs &sa, const double (&hv)[6]) {
-    if (!(sa.flags & STEP_REDUCE)) return;  // uniform over the block
-    if (__any_sync(0xffffffffu, hv[5] != 0.0) && (threadIdx.x & 31) == 0) atomicOr(sa.status, 1u);
-}
-
-template <int P>
-__global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_multi_fluid(const GroupTable *tab, int k) {
-    __shared__ StepArgs sa;
-    __shared__ int s_dom;
+// The arguments come by value: what an item uses of them is read from shared
+// memory once, not again after every store that might have changed it.
+template <int P, int AX>
+__device__ __forceinline__ void serve_nodes(const StepArgs a, int i, int lane) {
     double hv[6] = {0, 0, 0, 0, 0, 0};
-    const int ntiles = tab->n_tiles;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        __syncthreads();  // the previous tile is done with sa
-        if (threadIdx.x == 0) s_dom = find_domain<false>(tab, tile);
-        __syncthreads();
-        const DomainEntry &e = tab->d[s_dom];
-        if (!load_domain(e, k, sa)) continue;  // uniform over the block
-        const int chunk = (tile - e.tile_begin) * (STEP_THREADS / CHUNK) + threadIdx.x / CHUNK;
-        hv[5] = 0.0;
-        if (chunk < sa.nchunks) {
-            if (sa.row_axis == 2)  // uniform over the block
-                fluid_cell<P, true, false, 2>(sa, chunk, threadIdx.x % CHUNK, hv);
-            else
-                fluid_cell<P, true, false, 0>(sa, chunk, threadIdx.x % CHUNK, hv);
-        }
-        flag_non_finite(sa, hv);
-    }
+    const int k = 32 * i + lane;
+    if (k < a.nbnodes) boundary_node<P, RATE_ONE, false, AX, true>(a, k, hv);
+    flag_non_finite(a, hv[5]);
 }
 
-template <int P>
-__global__ void __launch_bounds__(STEP_THREADS) k_multi_boundary(const GroupTable *tab, int k) {
-    __shared__ StepArgs sa;
-    __shared__ int s_dom;
+template <int P, int AX>
+__device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec, int lane) {
     double hv[6] = {0, 0, 0, 0, 0, 0};
-    const int ntiles = tab->n_btiles;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    tile_update<P, AX, true, false>(a, rec, lane, nullptr, hv);
+    flag_non_finite(a, hv[5]);
+}
+
+// Calls fn<P, AX> for the lattice of an entry.
+#define SERVE_DISPATCH(e, fn, ...)                                                         \
+    do {                                                                                   \
+        if ((e).precision == LBM_FP32) {                                                   \
+            if ((e).a.row_axis == 2) fn<1, 2>((e).a, __VA_ARGS__);                         \
+            else fn<1, 0>((e).a, __VA_ARGS__);                                             \
+        } else {                                                                           \
+            if ((e).a.row_axis == 2) fn<2, 2>((e).a, __VA_ARGS__);                         \
+            else fn<2, 0>((e).a, __VA_ARGS__);                                             \
+        }                                                                                  \
+    } while (0)
+
+// All steps of a tick.  Before, a step was four launches in turn (fluid and
+// nodes of each precision) whose blocks copied a lattice's arguments to
+// shared memory for every 128 cells; here the table stays in shared memory,
+// and a warp looks up the lattice and the record of its next tile while it
+// updates one.  What then bounds it is the instruction cache: FP32 and FP16S
+// lattices in admission order and the fast tiles' own path took 166 us a step
+// for twelve lattices of 2.2 M cells (no_instruction half of the stalls),
+// each precision in one go and the line sink alone 118 us, the four launches
+// 136 us; one lattice of 67 000 cells 17 -> 10 us.  5 blocks per SM: 4 take 2 %
+// and 6 take 8 % longer on the burst of the measured mix.
+#ifndef LBM_SERVE_BLOCKS
+#define LBM_SERVE_BLOCKS 5
+#endif
+__global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const TickTable *tab, int32_t *barrier,
+                                                                        uint32_t *status) {
+    extern __shared__ __align__(16) char serve_smem[];
+    DomainEntry *dom = reinterpret_cast<DomainEntry *>(serve_smem);
+    const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    const int n = tab->n_domains, tiles = tab->n_tiles, nodes = tab->n_nodes, steps = tab->steps;
+    for (int w = threadIdx.x; w < n * (int)(sizeof(DomainEntry) / 16); w += STEP_THREADS)
+        reinterpret_cast<int4 *>(dom)[w] = reinterpret_cast<const int4 *>(tab->d)[w];
+    const int first = warp * (int)gridDim.x + (int)blockIdx.x, stride = (int)gridDim.x * (STEP_THREADS / 32);
+    for (int k = 0; k < steps; ++k) {
         __syncthreads();
-        if (threadIdx.x == 0) s_dom = find_domain<true>(tab, tile);
-        __syncthreads();
-        const DomainEntry &e = tab->d[s_dom];
-        if (!load_domain(e, k, sa)) continue;
-        const int node = (tile - e.btile_begin) * STEP_THREADS + threadIdx.x;
-        hv[5] = 0.0;
-        if (node < sa.nbnodes) {
-            if (sa.row_axis == 2)
-                boundary_node<P, true, false, 2>(sa, node, hv);
-            else
-                boundary_node<P, true, false, 0>(sa, node, hv);
+        if ((int)threadIdx.x < n) {  // the step's buffers, number and check flag
+            DomainEntry &e = dom[threadIdx.x];
+            if (k > 0) {
+                const void *t = e.a.fin;
+                e.a.fin = e.a.fout;
+                e.a.fout = const_cast<void *>(t);
+            }
+            e.a.t_new = e.t_base + k + 1;
+            e.a.flags = k == e.steps - 1 ? STEP_REDUCE : 0;
         }
-        flag_non_finite(sa, hv);
+        __syncthreads();
+        int i = first;
+        for (; i < nodes; i += stride) {
+            const DomainEntry &e = dom[find_domain<true>(dom, n, i)];
+            if (k < e.steps) SERVE_DISPATCH(e, serve_nodes, i - e.node_begin, lane);  // uniform over the warp
+        }
+        i -= nodes;
+        // the next tile's lattice and record are looked up while a tile is updated
+        int d_next = 0;
+        TileRec next;
+        if (i < tiles) {
+            d_next = find_domain<false>(dom, n, i);
+            next = TileRec(dom[d_next].a.tiles, i - dom[d_next].tile_begin);
+        }
+        for (; i < tiles; i += stride) {
+            const DomainEntry &e = dom[d_next];
+            const TileRec rec = next;
+            if (i + stride < tiles) {
+                d_next = find_domain<false>(dom, n, i + stride);
+                next = TileRec(dom[d_next].a.tiles, i + stride - dom[d_next].tile_begin);
+            }
+            if (k < e.steps) SERVE_DISPATCH(e, serve_tile, rec, lane);
+        }
+        if (k + 1 < steps && !grid_barrier(barrier, k + 1, status)) break;
+    }
+    // the last block to leave clears the words for the next tick
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(barrier + 1, 1) == (int)gridDim.x - 1) {
+        barrier[0] = 0;
+        barrier[1] = 0;
     }
 }
 
@@ -168,7 +197,6 @@ struct Request {
     int64_t n_active = -1;
     // resident state
     lbm_ctx *ctx = nullptr;
-    int group = 0;
     // result
     std::vector<double> rho, u;
 };
@@ -195,13 +223,13 @@ struct lbm_server {
     std::deque<Request *> build_queue;
     bool stop = false;
     // device tables and the tick graph
-    GroupTable *h_tab[NGROUPS] = {nullptr, nullptr};
-    GroupTable *d_tab[NGROUPS] = {nullptr, nullptr};
-    // health flags, one word per (group, domain): cleared at the start of
-    // every tick, raised by the check step, copied back at its end
+    TickTable *h_tab = nullptr, *d_tab = nullptr;
+    // health flags, one word per domain: cleared at the start of every tick,
+    // raised by the check step, copied back at its end; then the tick's status
+    // and the kernel's barrier words
     uint32_t *d_flags = nullptr, *h_flags = nullptr;
     cudaGraphExec_t exec = nullptr;
-    int grid_fluid[NGROUPS] = {0, 0}, grid_bnd[NGROUPS] = {0, 0};
+    int grid = 0, smem = 0;  // of the tick's kernel
 };
 
 namespace {
@@ -283,33 +311,39 @@ void worker_loop(lbm_server *s) {
     }
 }
 
-template <int P>
-void occupancy_grids(int sms, int &gf, int &gb) {
-    int nf = 0, nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nf, k_multi_fluid<P>, STEP_THREADS, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_multi_boundary<P>, STEP_THREADS, 0);
-    gf = sms * std::max(1, nf);
-    gb = sms * std::max(1, std::min(nb, 2));
+// Grid and shared memory of the tick's kernel: every block resident at once.
+cudaError_t serve_grid(lbm_server *s) {
+    s->smem = s->desc.max_slots * (int)sizeof(DomainEntry);
+    int per_sm = 0, sms = 0, coop = 0;
+    cudaError_t e = cudaFuncSetAttribute(k_serve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         MAX_SLOTS * (int)sizeof(DomainEntry));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve, STEP_THREADS, s->smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->desc.device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, s->desc.device);
+    if (e == cudaSuccess && (!coop || per_sm < 1)) e = cudaErrorNotSupported;
+    s->grid = per_sm * sms;
+    return e;
 }
 
-// Capture the tick: table copies, then per step the fluid and boundary
-// launches of both precision groups.
+// Capture the tick: table copy, cleared health flags, the kernel, flags back.
 lbm_status capture_tick(lbm_server *s) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("begin capture: ") + cudaGetErrorString(e));
-    for (int q = 0; q < NGROUPS; ++q)
-        cudaMemcpyAsync(s->d_tab[q], s->h_tab[q], sizeof(GroupTable), cudaMemcpyHostToDevice, s->stream);
-    cudaMemsetAsync(s->d_flags, 0, NGROUPS * MAX_SLOTS * sizeof(uint32_t), s->stream);
-    for (int k = 0; k < s->desc.steps_per_tick; ++k) {
-        k_multi_fluid<1><<<s->grid_fluid[0], STEP_THREADS, 0, s->stream>>>(s->d_tab[0], k);
-        k_multi_fluid<2><<<s->grid_fluid[1], STEP_THREADS, 0, s->stream>>>(s->d_tab[1], k);
-        k_multi_boundary<1><<<s->grid_bnd[0], STEP_THREADS, 0, s->stream>>>(s->d_tab[0], k);
-        k_multi_boundary<2><<<s->grid_bnd[1], STEP_THREADS, 0, s->stream>>>(s->d_tab[1], k);
-    }
-    cudaMemcpyAsync(s->h_flags, s->d_flags, NGROUPS * MAX_SLOTS * sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                    s->stream);
+    cudaMemcpyAsync(s->d_tab, s->h_tab, sizeof(TickTable), cudaMemcpyHostToDevice, s->stream);
+    cudaMemsetAsync(s->d_flags, 0, (STATUS_WORD + 1) * sizeof(uint32_t), s->stream);
+    const TickTable *tab = s->d_tab;
+    int32_t *barrier = reinterpret_cast<int32_t *>(s->d_flags) + BARRIER_WORDS;
+    uint32_t *status = s->d_flags + STATUS_WORD;
+    void *params[3] = {&tab, &barrier, &status};
+    const cudaError_t launch = cudaLaunchCooperativeKernel((const void *)k_serve, dim3((unsigned)s->grid),
+                                                           dim3(STEP_THREADS), params, (size_t)s->smem, s->stream);
+    cudaMemcpyAsync(s->h_flags, s->d_flags, (STATUS_WORD + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream);
     e = cudaStreamEndCapture(s->stream, &g);
+    if (e == cudaSuccess && launch != cudaSuccess) {
+        cudaGraphDestroy(g);
+        e = launch;
+    }
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(&s->exec, g, 0);
     cudaGraphDestroy(g);
@@ -360,7 +394,6 @@ lbm_status admit(lbm_server *s, Request *r) {
     }
     r->ctx = c;
     drop_inputs(r);
-    r->group = r->req.precision == LBM_FP16S ? 1 : 0;
     r->state = LBM_REQ_RUNNING;
     s->in_use += r->footprint;
     s->peak = std::max(s->peak, s->in_use);
@@ -388,10 +421,8 @@ lbm_status lbm_server_create(const lbm_server_desc *desc, lbm_server **out) {
     cudaSetDevice(desc->device);
     // on a failure below, free what was made so far (no worker runs yet)
     auto undo = [&](lbm_status st) {
-        for (int q = 0; q < NGROUPS; ++q) {
-            if (s->h_tab[q]) cudaFreeHost(s->h_tab[q]);
-            if (s->d_tab[q]) cudaFree(s->d_tab[q]);
-        }
+        if (s->h_tab) cudaFreeHost(s->h_tab);
+        if (s->d_tab) cudaFree(s->d_tab);
         if (s->h_flags) cudaFreeHost(s->h_flags);
         if (s->d_flags) cudaFree(s->d_flags);
         if (s->own_stream) cudaStreamDestroy(s->stream);
@@ -403,31 +434,27 @@ lbm_status lbm_server_create(const lbm_server_desc *desc, lbm_server **out) {
         if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) return undo(LBM_ERR_CUDA);
         s->own_stream = true;
     }
-    for (int q = 0; q < NGROUPS; ++q) {
-        if (cudaMallocHost(&s->h_tab[q], sizeof(GroupTable)) != cudaSuccess) {
-            s->h_tab[q] = nullptr;
-            return undo(LBM_ERR_CUDA);
-        }
-        memset(s->h_tab[q], 0, sizeof(GroupTable));
-        // the tables are part of the server, not of any lattice: not from the allocator
-        if (cudaMalloc(&s->d_tab[q], sizeof(GroupTable)) != cudaSuccess) {
-            s->d_tab[q] = nullptr;
-            return undo(LBM_ERR_OOM);
-        }
+    if (cudaMallocHost(&s->h_tab, sizeof(TickTable)) != cudaSuccess) {
+        s->h_tab = nullptr;
+        return undo(LBM_ERR_CUDA);
     }
-    if (cudaMallocHost(&s->h_flags, NGROUPS * MAX_SLOTS * sizeof(uint32_t)) != cudaSuccess) {
+    memset(s->h_tab, 0, sizeof(TickTable));
+    // the table and the flags are part of the server, not of any lattice: not from the allocator
+    if (cudaMalloc(&s->d_tab, sizeof(TickTable)) != cudaSuccess) {
+        s->d_tab = nullptr;
+        return undo(LBM_ERR_OOM);
+    }
+    if (cudaMallocHost(&s->h_flags, FLAG_WORDS * sizeof(uint32_t)) != cudaSuccess) {
         s->h_flags = nullptr;
         return undo(LBM_ERR_CUDA);
     }
-    memset(s->h_flags, 0, NGROUPS * MAX_SLOTS * sizeof(uint32_t));
-    if (cudaMalloc(&s->d_flags, NGROUPS * MAX_SLOTS * sizeof(uint32_t)) != cudaSuccess) {
+    memset(s->h_flags, 0, FLAG_WORDS * sizeof(uint32_t));
+    if (cudaMalloc(&s->d_flags, FLAG_WORDS * sizeof(uint32_t)) != cudaSuccess) {
         s->d_flags = nullptr;
         return undo(LBM_ERR_OOM);
     }
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, desc->device);
-    occupancy_grids<1>(sms, s->grid_fluid[0], s->grid_bnd[0]);
-    occupancy_grids<2>(sms, s->grid_fluid[1], s->grid_bnd[1]);
+    if (cudaMemset(s->d_flags, 0, FLAG_WORDS * sizeof(uint32_t)) != cudaSuccess || serve_grid(s.get()) != cudaSuccess)
+        return undo(LBM_ERR_CUDA);
     lbm_server *raw = s.get();
     // Index building is host work that is independent per request: a few
     // threads keep admission fed when many small requests arrive at once.
@@ -451,10 +478,8 @@ lbm_status lbm_server_destroy(lbm_server *s) {
     cudaStreamSynchronize(s->stream);
     for (auto &kv : s->reqs) release(s, kv.second.get());
     if (s->exec) cudaGraphExecDestroy(s->exec);
-    for (int q = 0; q < NGROUPS; ++q) {
-        if (s->h_tab[q]) cudaFreeHost(s->h_tab[q]);
-        if (s->d_tab[q]) cudaFree(s->d_tab[q]);
-    }
+    if (s->h_tab) cudaFreeHost(s->h_tab);
+    if (s->d_tab) cudaFree(s->d_tab);
     if (s->h_flags) cudaFreeHost(s->h_flags);
     if (s->d_flags) cudaFree(s->d_flags);
     if (s->own_stream) cudaStreamDestroy(s->stream);
@@ -545,29 +570,31 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
     if (queued) *queued = (int32_t)s->queue.size();
     if (s->resident.empty()) return LBM_OK;
 
-    // per-tick tables
-    for (int q = 0; q < NGROUPS; ++q) {
-        s->h_tab[q]->n_domains = 0;
-        s->h_tab[q]->n_tiles = 0;
-        s->h_tab[q]->n_btiles = 0;
-    }
+    // the tick's table
+    TickTable *tab = s->h_tab;
+    tab->n_domains = tab->n_tiles = tab->n_nodes = tab->steps = 0;
     const int K = s->desc.steps_per_tick;
     std::vector<int> steps_now(s->resident.size()), flag_of(s->resident.size());
-    for (size_t k = 0; k < s->resident.size(); ++k) {
-        Request *r = s->reqs[s->resident[k]].get();
-        GroupTable *tab = s->h_tab[r->group];
-        flag_of[k] = r->group * MAX_SLOTS + tab->n_domains;
-        DomainEntry &e = tab->d[tab->n_domains++];
-        ctx_chunk_step_args(r->ctx, &e.a);
-        e.a.status = s->d_flags + flag_of[k];  // the lattice's health flag
-        e.t_base = r->steps_done;
-        e.steps = (int32_t)std::min<int64_t>(K, r->req.steps - r->steps_done);
-        steps_now[k] = e.steps;
-        e.tile_begin = tab->n_tiles;
-        e.btile_begin = tab->n_btiles;
-        tab->n_tiles += (int32_t)(((int64_t)e.a.nchunks * CHUNK + STEP_THREADS - 1) / STEP_THREADS);
-        tab->n_btiles += (e.a.nbnodes + STEP_THREADS - 1) / STEP_THREADS;
-    }
+    // FP32 lattices first, then FP16S: the warps, which walk the list together,
+    // then change from one collision's code to the other's once a step
+    for (int q = 0; q < 2; ++q)
+        for (size_t k = 0; k < s->resident.size(); ++k) {
+            Request *r = s->reqs[s->resident[k]].get();
+            if ((r->req.precision == LBM_FP16S) != (q == 1)) continue;
+            flag_of[k] = tab->n_domains;
+            DomainEntry &e = tab->d[tab->n_domains++];
+            ctx_tile_step_args(r->ctx, &e.a);
+            e.a.status = s->d_flags + flag_of[k];  // the lattice's health flag
+            e.t_base = r->steps_done;
+            e.steps = (int32_t)std::min<int64_t>(K, r->req.steps - r->steps_done);
+            steps_now[k] = e.steps;
+            e.precision = r->req.precision;
+            e.tile_begin = tab->n_tiles;
+            e.node_begin = tab->n_nodes;
+            tab->n_tiles += e.a.ntiles;
+            tab->n_nodes += (e.a.nbnodes + 31) / 32;
+            tab->steps = std::max(tab->steps, e.steps);
+        }
     if (!s->exec) {
         lbm_status st = capture_tick(s);
         if (st != LBM_OK) return st;
@@ -579,6 +606,7 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     }
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("tick: ") + cudaGetErrorString(e));
+    if (s->h_flags[STATUS_WORD] & 2u) return sfail(s, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (tick kernel)");
     s->graph_launches += 1;
     s->ticks += 1;
     // account, retire finished lattices
