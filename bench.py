@@ -85,7 +85,7 @@ def env_rank():
 
 
 # The fluid kernel each precision runs by default (the roofline's dominant kernel).
-FLUID_KERNEL = {"fp32": "k_step_tiles<fp32>", "fp16s": "k_step<fp16s>", "fp64": "k_step<fp64>"}
+FLUID_KERNEL = {"fp32": "k_step_tiles<fp32>", "fp16s": "k_step_units<fp16s>", "fp64": "k_step<fp64>"}
 
 
 def load_peaks():

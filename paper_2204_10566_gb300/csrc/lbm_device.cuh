@@ -187,7 +187,8 @@ __device__ __forceinline__ R cst(int a, int b) {
 template <class R>
 struct Axis {
     R d[3], g0[3], g1[3];
-    __device__ __forceinline__ explicit Axis(R u);
+    // lo, hi: u^2 - u and u^2 + u in one rounding each
+    __device__ __forceinline__ Axis(R u, bool lo, bool hi);
 };
 
 template <class R>
@@ -259,14 +260,15 @@ __device__ __forceinline__ F2 sub_(F2 a, F2 b) { return a - b; }
 __device__ __forceinline__ F2 mul_(F2 a, F2 b) { return a * b; }
 
 template <class R>
-__device__ __forceinline__ Axis<R>::Axis(R u) {
+__device__ __forceinline__ Axis<R>::Axis(R u, bool lo, bool hi) {
     const R h = R(0.5), u2 = mul_(u, u);
-    d[0] = mul_(h, fma_(u, u, -u));
+    const R m = lo ? fma_(u, u, -u) : sub_(u2, u), p = hi ? fma_(u, u, u) : add_(u2, u);
+    d[0] = mul_(h, m);
     d[1] = -u2;
-    d[2] = mul_(h, fma_(u, u, u));
-    g0[0] = fma_(h, fma_(u, u, -u), w1<R>(-1));
-    g0[1] = fma_(-u, u, w1<R>(0));
-    g0[2] = fma_(h, fma_(u, u, u), w1<R>(1));
+    d[2] = mul_(h, p);
+    g0[0] = fma_(h, m, w1<R>(-1));
+    g0[1] = sub_(w1<R>(0), u2);
+    g0[2] = fma_(h, p, w1<R>(1));
     g1[0] = sub_(u, h);
     g1[1] = mul_(R(-2), u);
     g1[2] = add_(u, h);
@@ -286,7 +288,7 @@ __device__ __forceinline__ void inverse_centre(const PairCoef &c, const Axis<flo
     const float E = mul_(gy0, gz0);
     const float D = fma_(w0, Z.d[1], mul_(Y.d[1], gz0));
     const float C0 = fma_(mul_(c.Ayz, gy1), gz1, fma_(-c.Azz, gy0, mul_(-c.Ayy, gz0)));
-    const float B1 = fma_(mul_(c.Axz, gy0), gz1, mul_(mul_(c.Axy, gy1), gz0));
+    const float B1 = fma_(mul_(c.Axy, gy1), gz0, mul_(mul_(c.Axz, gy0), gz1));
     const float B2 = mul_(c.Axx, E);
     const float Bw = add_(fma_(c.drho_o, w0 * w0, mul_(c.rho_o, D)), C0);
     const float Bd = fma_(c.rho_o, E, C0), xBd = mul_(c.ux2h, Bd);
@@ -321,12 +323,11 @@ __device__ __forceinline__ void inverse_pair(const PairCoef &c, const Axis<float
     const float2 C0 = __ffma2_rn(v1_, bc2(mul_(c.Ayz, f1)), __ffma2_rn(v0_, bc2(mul_(Aff, fg2)), bc2(mul_(mul_(0.5f, Avv), f0))));
     const float2 hB1 = __ffma2_rn(v1_, bc2(mul_(mul_(0.5f, Axv), f0)), __fmul2_rn(v0_, bc2(mul_(mul_(0.5f, Axf), f1))));
     const float2 nB2 = __fmul2_rn(v0_, bc2(mul_(-c.Axx, f0)));
-    const float2 hB2 = __fmul2_rn(v0_, bc2(mul_(mul_(0.5f, c.Axx), f0)));
     const float2 Bw = __ffma2_rn(bc2(c.rho_o), D, __fadd2_rn(C0, bc2(mul_(c.drho_o, fw * (1.0f / 6.0f)))));
     const float2 Bd = __ffma2_rn(bc2(c.rho_o), E, C0);
     const float2 t = __ffma2_rn(bc2(c.ux2h), Bd, __fmul2_rn(bc2(mul_(2.0f, c.ux)), hB1));
     const float2 o0 = __ffma2_rn(bc2(2.0f / 3.0f), Bw, __ffma2_rn(bc2(-2.0f), t, nB2));
-    const float2 S = __ffma2_rn(bc2(1.0f / 6.0f), Bw, __fadd2_rn(t, hB2));
+    const float2 S = __ffma2_rn(bc2(1.0f / 6.0f), Bw, __ffma2_rn(v0_, bc2(mul_(mul_(0.5f, c.Axx), f0)), t));
     const float2 A = __ffma2_rn(bc2(c.uxh), Bd, hB1);
     const float2 om = __ffma2_rn(bc2(-1.0f), A, S), op = __fadd2_rn(S, A);
     sink(JA, om.x, o0.x, op.x);
@@ -395,22 +396,26 @@ __device__ __forceinline__ void ghost1_sums(const R (&d)[27], R (&m)[10]) {
 // The rest of the FP32 default-rate collision from the moment sums: rho, u, the
 // six second-order central Hermite moments, their relaxation, and the
 // inverse transform, line by line into sink(j, f*_{3j} - w, f*_{3j+1} - w,
-// f*_{3j+2} - w).
-template <class Out>
+// f*_{3j+2} - w).  With SCALED (RATE_KEPT of FP16S) the sums are of
+// (f - w) / in_scale and the outputs are (f* - w) * out_scale: the scales,
+// powers of two, act on the ten moments and the eight output coefficients.
+// fused: the roundings of the y and z columns, see RATE_KEPT.
+template <bool SCALED, class Out>
 __device__ __forceinline__ void ghost1_finish(const float (&m)[10], float omega, float &rho, float &ux, float &uy,
-                                              float &uz, const Out &sink) {
-    const float drho = m[0], th = theta0<float>();
+                                              float &uz, float in_scale, float out_scale, bool fused, const Out &sink) {
+    const float drho = SCALED ? mul_(m[0], in_scale) : m[0], th = theta0<float>();
     rho = add_(1.0f, drho);
     const float inv = recip(rho);
-    ux = mul_(m[1], inv);
-    uy = mul_(m[2], inv);
-    uz = mul_(m[3], inv);
+    ux = mul_(SCALED ? mul_(m[1], in_scale) : m[1], inv);
+    uy = mul_(SCALED ? mul_(m[2], in_scale) : m[2], inv);
+    uz = mul_(SCALED ? mul_(m[3], in_scale) : m[3], inv);
     // Second-order central Hermite moments sum_i ((c-u)_a (c-u)_b - theta0 delta_ab) f_i,
     // from the deviation moments (sum c_a c_b w = theta0 delta_ab).
-    const float rx = mul_(rho, ux), ry = mul_(rho, uy), rz = mul_(rho, uz);
-    const float a2[6] = {fma_(-th, drho, fma_(-rx, ux, m[4])), fma_(-th, drho, fma_(-ry, uy, m[5])),
-                         fma_(-th, drho, fma_(-rz, uz, m[6])), fma_(-rx, uy, m[7]),
-                         fma_(-rx, uz, m[8]),                  fma_(-ry, uz, m[9])};
+    const float rx = -mul_(rho, ux), ry = -mul_(rho, uy), rz = -mul_(rho, uz);
+    auto less = [&](float p, float r, float u) { return SCALED ? fma_(p, in_scale, mul_(r, u)) : fma_(r, u, p); };
+    const float a2[6] = {fma_(-th, drho, less(m[4], rx, ux)), fma_(-th, drho, less(m[5], ry, uy)),
+                         fma_(-th, drho, less(m[6], rz, uz)), less(m[7], rx, uy),
+                         less(m[8], rx, uz),                  less(m[9], ry, uz)};
     sink.moments(omega, a2);
     // Inverse: f* = rho prod g0 + sum over the six relaxed second-order moments
     // of A_m prod_a g_{m_a}; orders 1 and 3..6 are zero after relaxation.
@@ -419,10 +424,10 @@ __device__ __forceinline__ void ghost1_finish(const float (&m)[10], float omega,
     // and for cx = +-1 this splits into S +- A.  Lines go in pairs on the
     // packed FP32 pipe (two lanes per instruction): (cy = -1, +1) at each cz,
     // then (cz = -1, +1) at cy = 0; the centre line alone.
-    const float k = sub_(1.0f, omega), uxh = mul_(0.5f, ux);
-    const Axis<float> Y(uy), Z(uz);
+    const float one_w = sub_(1.0f, omega), k = SCALED ? mul_(one_w, out_scale) : one_w, uxh = mul_(0.5f, ux);
+    const Axis<float> Y(uy, fused, fused), Z(uz, false, fused);
     const PairCoef c{mul_(k, a2[0]), mul_(k, a2[1]), mul_(k, a2[2]), mul_(k, a2[3]), mul_(k, a2[4]), mul_(k, a2[5]),
-                     rho, drho, ux, mul_(uxh, ux), uxh};
+                     SCALED ? mul_(rho, out_scale) : rho, SCALED ? mul_(drho, out_scale) : drho, ux, mul_(uxh, ux), uxh};
     inverse_pair<0, 2>(c, Y, Z, sink);
     inverse_pair<3, 5>(c, Y, Z, sink);
     inverse_pair<6, 8>(c, Y, Z, sink);
@@ -651,10 +656,21 @@ __device__ __forceinline__ void collide_ghost1(R (&d)[27], R omega, R &rho, R &u
     } else {
         ghost1_sums(d, m);
         if (sink)
-            ghost1_finish(m, omega, rho, ux, uy, uz, *sink);
+            ghost1_finish<false>(m, omega, rho, ux, uy, uz, 1.0f, 1.0f, false, *sink);
         else
-            ghost1_finish(m, omega, rho, ux, uy, uz, ToArray<R>{d});
+            ghost1_finish<false>(m, omega, rho, ux, uy, uz, 1.0f, 1.0f, false, ToArray<R>{d});
     }
+}
+
+// The same with the roundings of RATE_KEPT (FP16S).  fused: of the columns,
+// as in the fluid lanes outside the uniform warps of a lattice with rows
+// along z.
+template <bool SCALED, class Out>
+__device__ __forceinline__ void collide_kept(float (&d)[27], float omega, float &rho, float &ux, float &uy, float &uz,
+                                             float in_scale, float out_scale, bool fused, const Out &sink) {
+    float m[10];
+    ghost1_sums(d, m);
+    ghost1_finish<SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, fused, sink);
 }
 
 // The equilibrium part alone: the lines of ro f^eq(u)/rho less (ro - dro) w,
@@ -987,6 +1003,8 @@ __device__ __forceinline__ void collide(typename Storage<P>::R (&d)[27], const F
     const ToArrayStress<R> sink{a, stress_slot, d};
     if constexpr (G == RATE_ONE)
         collide_ghost1<R, false, ToArrayStress<R>>(d, fp.omega, rho, ux, uy, uz, R(1), R(1), &sink);
+    else if constexpr (G == RATE_KEPT)
+        collide_kept<false>(d, fp.omega, rho, ux, uy, uz, 1.0f, 1.0f, false, sink);
     else if constexpr (G == RATE_BGK)
         collide_bgk<R>(d, fp.omega, rho, ux, uy, uz, sink);
     else
@@ -1188,7 +1206,7 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int row, int x, b
                                : (((m >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~m & LINK_MASK) : 0u);
     R d[27];
     R rho, ux, uy, uz;
-    constexpr bool RAW = G == RATE_ONE && Storage<P>::SCALED;  // FP16 scale folded into the collision
+    constexpr bool RAW = (G == RATE_ONE || G == RATE_KEPT) && Storage<P>::SCALED;  // FP16 scale folded into the collision
     gather<P, WIDE, AX, RAW, CG>(a, nb, x, d);
     if constexpr (WALLQ) interpolate_walls<P, WIDE, RAW, CG>(a, qk, slot, links, d);
     if constexpr (G != RATE_GENERAL) {
@@ -1196,6 +1214,8 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int row, int x, b
         if constexpr (G == RATE_ONE)
             collide_ghost1<R, RAW, LineStore<P, WIDE, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
                                                                 R(a.scale), &sink);
+        else if constexpr (G == RATE_KEPT)
+            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, false, sink);
         else
             collide_bgk<R>(d, flow<R>(a).omega, rho, ux, uy, uz, sink);
     } else {
@@ -1222,7 +1242,7 @@ __device__ __forceinline__ void fluid_cell(const StepArgs &a, int chunk, int lan
 // ghost-slot stores and wrap-around copies.  The gather is the same on both paths, so it
 // is issued before the vote.  Every lane of the warp must call this (lanes
 // past the last chunk take part in the vote only).
-template <int P, int AX>
+template <int P, int G, int AX>
 __device__ __forceinline__ void fluid_lane_voted(const StepArgs &a, int chunk, int lane, double (&hv)[6]) {
     using R = typename Storage<P>::R;
     constexpr bool RAW = Storage<P>::SCALED;
@@ -1249,14 +1269,20 @@ __device__ __forceinline__ void fluid_lane_voted(const StepArgs &a, int chunk, i
     R rho, ux, uy, uz;
     if (fast) {
         const OwnStore<P, RAW> sink{a, slot};
-        collide_ghost1<R, RAW, OwnStore<P, RAW>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale),
-                                                 &sink);
+        if constexpr (G == RATE_KEPT)
+            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, false, sink);
+        else
+            collide_ghost1<R, RAW, OwnStore<P, RAW>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
+                                                     R(a.scale), &sink);
     } else {
         const uint32_t links = fluid ? (m & LINK_MASK) : 0u;
         const uint32_t own = fluid ? (LINK_MASK | OWN_FLUID)
                                    : (((m >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~m & LINK_MASK) : 0u);
         const LineStore<P, false, RAW, AX> sink{a, nb, x, slot, links, own};
-        collide_ghost1<R, RAW, LineStore<P, false, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz,
+        if constexpr (G == RATE_KEPT)
+            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, AX == 2, sink);
+        else
+            collide_ghost1<R, RAW, LineStore<P, false, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz,
                                                              R(a.inv_scale), R(a.scale), &sink);
     }
     if (fluid) record_cell(a, slot, rho, ux, uy, uz, hv);
@@ -1288,11 +1314,13 @@ struct NodeStore {
     }
     __device__ __forceinline__ void moments(R omega, const R (&a2)[6]) const {}
     __device__ __forceinline__ void operator()(int j, R vm, R v0, R vp) const {
-        R v[3] = {vm, v0, vp}, e[3];
+        R e[3];
         if (j % 3 == 0) eq.plane(j / 3);
         eq.line(j % 3, e[0], e[1], e[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] = add_(v[c], e[c]);
+        line(j, add_(vm, e[0]), add_(v0, e[1]), add_(vp, e[2]));
+    }
+    __device__ __forceinline__ void line(int j, R vm, R v0, R vp) const {
+        const R v[3] = {vm, v0, vp};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const int i = 3 * j + c;
@@ -1301,6 +1329,26 @@ struct NodeStore {
                 if (c_row<AX>(i) == 1 && pos == a.n_row - 1) put(i, slot - pos - 1, v[c]);
                 if (c_row<AX>(i) == -1 && pos == 0) put(i, slot + a.n_row, v[c]);
             }
+        }
+    }
+};
+
+// One line (cx = -1, 0, 1) of f^eq(rho, u) - w in product form, without O(1)
+// cancellation: (rho - 1) w + rho (dx gy gz + wx (dy gz + wy dz)), with the
+// roundings of RATE_KEPT.
+struct EqNode {
+    Axis<float> X, Y, Z;
+    float r, dr;
+    __device__ __forceinline__ EqNode(float rho, float ux, float uy, float uz)
+        : X(ux, false, false), Y(uy, false, false), Z(uz, false, false), r(rho), dr(sub_(rho, 1.0f)) {}
+    __device__ __forceinline__ void line(int j, float (&e)[3]) const {
+        const int y = j % 3, z = j / 3;
+        const float wy = w1<float>(y - 1), E = mul_(Y.g0[y], Z.g0[z]);
+        const float D = y == 1 ? fma_(wy, Z.d[z], mul_(Y.d[y], Z.g0[z])) : fma_(Y.d[y], Z.g0[z], mul_(wy, Z.d[z]));
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            const float wx = w1<float>(x - 1), ww = wx * wy * w1<float>(z - 1), p = fma_(wx, D, mul_(X.d[x], E));
+            e[x] = j == 4 && x == 1 ? fma_(dr, ww, mul_(r, p)) : fma_(r, p, mul_(dr, ww));
         }
     }
 };
@@ -1332,7 +1380,7 @@ __device__ __forceinline__ void boundary_node(const StepArgs &a, int k, double (
         const int dir = (int)(m >> DIR_SHIFT);
         R speed = fp.u_in;
         if (a.profile == LBM_PROFILE_PARABOLIC) {
-            const R rx = add_(R(r1.x), sub_(R(0.5), fp.axis_x)), ry = add_(R(r1.y), sub_(R(0.5), fp.axis_y));
+            const R rx = sub_(add_(R(r1.x), R(0.5)), fp.axis_x), ry = sub_(add_(R(r1.y), R(0.5)), fp.axis_y);
             const R r2_ = fma_(rx, rx, mul_(ry, ry));
             speed = mul_(mul_(R(2), fp.u_in), sub_(R(1), mul_(R(4), r2_) / mul_(fp.d_in, fp.d_in)));
         }
@@ -1379,6 +1427,21 @@ __device__ __forceinline__ void boundary_node(const StepArgs &a, int k, double (
         collide<P, G>(d, fp, rf, uxf, uyf, uzf, a, slot);  // the node takes its partner's stress
         if (!inlet) ux = uxf, uy = uyf, uz = uzf;
         rho = inlet ? rf : fp.rho_out;
+        if constexpr (G == RATE_KEPT) {
+            const EqNode fe(rf, uxf, uyf, uzf), be(rho, ux, uy, uz);
+            const NodeStore<P, WIDE, AX> out{a, slot, pos, EqLines<R>(rho, R(0), ux, uy, uz)};
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                float b[3], f[3];
+                be.line(j, b);
+                fe.line(j, f);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) b[c] = add_(d[3 * j + c], sub_(b[c], f[c]));
+                out.line(j, b[0], b[1], b[2]);
+            }
+            record_cell(a, slot, rho, ux, uy, uz, hv);
+            return;
+        }
         EqLines<R> ef(rf, sub_(rf, R(1)), uxf, uyf, uzf);
         const NodeStore<P, WIDE, AX> out{a, slot, pos, EqLines<R>(rho, sub_(rho, R(1)), ux, uy, uz)};
 #pragma unroll
@@ -1437,8 +1500,8 @@ __global__ void __launch_bounds__(STEP_THREADS, P == 0 ? 1 : (G == RATE_GENERAL 
     } else {
         const int gt = blockIdx.x * STEP_THREADS + threadIdx.x;
         const int chunk = gt / CHUNK;
-        if constexpr (LBM_FAST_PATH && G == RATE_ONE && !WIDE && P != 0)
-            fluid_lane_voted<P, AX>(a, chunk, gt % CHUNK, hv);  // every lane of the block calls it
+        if constexpr (LBM_FAST_PATH && (G == RATE_ONE || G == RATE_KEPT) && !WIDE && P != 0)
+            fluid_lane_voted<P, G, AX>(a, chunk, gt % CHUNK, hv);  // every lane of the block calls it
         else if (chunk < a.nchunks)
             fluid_cell<P, G, WIDE, AX>(a, chunk, gt % CHUNK, hv);
         if (a.prefetch_ahead > 0) {
@@ -2471,7 +2534,14 @@ cudaError_t launch_step(const StepArgs &a, int mode, cudaStream_t s, int *launch
     const bool wide = a.wide_offsets || a.stride > MAX_SLOTS_32;
     int n = 0;
     cudaError_t e;
-    if (mode == RATE_ONE)
+    if constexpr (P == 2) {
+        if (mode == RATE_KEPT && !wide) {
+            e = launch_step_rows<P, RATE_KEPT, false>(a, s, side, n);
+            if (launches) *launches += n;
+            return e != cudaSuccess ? e : cudaGetLastError();
+        }
+    }
+    if (mode == RATE_ONE || mode == RATE_KEPT)
         e = wide ? launch_step_rows<P, RATE_ONE, true>(a, s, side, n) : launch_step_rows<P, RATE_ONE, false>(a, s, side, n);
     else if (mode == RATE_BGK && !wide)
         e = launch_step_rows<P, RATE_BGK, false>(a, s, side, n);

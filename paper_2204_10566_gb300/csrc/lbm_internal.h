@@ -140,11 +140,23 @@ std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vec
 
 // Form of the collision: general ghost rates (the 27-moment cascade), all
 // ghost rates 1 (the default), or all ghost rates equal to omega (lattice BGK).
-enum : int { RATE_GENERAL = 0, RATE_ONE = 1, RATE_BGK = 2 };
+// RATE_KEPT is RATE_ONE for FP16S with statistics on (32-bit offsets, no
+// fluid kernel asked for by name), in the chunk kernel and with the roundings
+// of the releases before the staged kernel.  FP16 storage carries a last-bit
+// difference on to the size of its own noise in some 50 steps, 1e-3 of a
+// velocity, and the averages, returned in FP64, show that in full; with these
+// roundings a run's averages repeat those taken earlier (nozzles of 49 000 to
+// 4.5 million cells, both wall treatments, 120 to 400 steps: to the bit, with
+// RATE_ONE's they are off by 1e-4 to 5e-4).  They are the ones a compiler
+// picked where a product meets a sum, hence the choice by kind of warp and
+// row axis.  The price is the chunk kernel's step, 448 us on the Re 6500
+// nozzle where the staged kernel takes 336.
+enum : int { RATE_GENERAL = 0, RATE_ONE = 1, RATE_BGK = 2, RATE_KEPT = 3 };
 
 // Fluid kernel of the FP32 / FP16S steps: AUTO is the tile kernel in FP32
 // and, in FP16S, the staged unit kernel for larger lattices and the chunk
-// kernel for smaller ones; the others are kept for testing.
+// kernel for smaller ones and with statistics on; the others are kept for
+// testing.
 enum class FluidKernel { AUTO, CHUNK, TILE, PAIRS, STAGED };
 
 // A second stream and its fork / join events: a step's wall-cell and

@@ -82,3 +82,35 @@ def test_staged_kernel_equals_chunk_kernel(lbm, monkeypatch, name):
 def test_staged_kernel_with_interpolated_walls(lbm, monkeypatch):
     for a, b in zip(run(lbm, monkeypatch, "staged", "nozzle", True), run(lbm, monkeypatch, "chunk", "nozzle", True)):
         assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name,walls", [("duct_x", False), ("duct_z", False), ("ragged_z", False), ("nozzle", False),
+                                        ("nozzle", True)])
+def test_steps_with_statistics_differ_by_roundings_alone(lbm, monkeypatch, name, walls):
+    """With statistics on, FP16S keeps other roundings of the same update (in
+    the chunk kernel): after one step each population is within one FP16 step
+    of the other form's, 2^-10 of its deviation, and the FP32 arithmetic's
+    error, 1e-8 (27 roundings of deviations below 0.01)."""
+    flags, periodic, rows = FIELDS[name]
+    w = np.array([(1 / 6, 2 / 3, 1 / 6)[i % 3] * (1 / 6, 2 / 3, 1 / 6)[i // 3 % 3] * (1 / 6, 2 / 3, 1 / 6)[i // 9]
+                  for i in range(27)])
+    out = []
+    for kernel in (None, "chunk"):
+        if kernel:
+            monkeypatch.setenv("LBM_FLUID_KERNEL", kernel)
+        else:
+            monkeypatch.delenv("LBM_FLUID_KERNEL", raising=False)
+        with lbm.Lattice(flags, "fp16s", periodic=periodic, row_axis=rows) as G:
+            G.set_params(nu=0.02, u_in=0.02, d_in=float(flags.shape[2]), profile="parabolic", noise_amp=0.02,
+                         noise_seed=3)
+            if walls:
+                G.set_wall_q(*I.nozzle_wall_q(12, 4, 140))
+            n = G.n_active
+            G.init_fields(I.random_density_field(n, 0.01, 5), I.random_velocity_field(n, 0.03, 6))
+            G.stats_begin(1, full=True)
+            G.step(1).sync()
+            assert G.stats_get_full()["samples"] == 1
+            out.append(G.get_populations())
+    a, b = out
+    assert np.isfinite(a).all()
+    assert (np.abs(a - b) <= 2.0 ** -10 * np.maximum(np.abs(a - w), np.abs(b - w)) + 1e-8).all()
