@@ -38,10 +38,10 @@ DTYPE = {"fp64": "f64", "fp32": "f32", "fp16s": "f16 storage / f32 arithmetic"}
 LINK_WORD_BYTES = 4
 
 
-# FP64 flops per fluid-cell update of the step kernel (DADD + DMUL + 2 DFMA,
-# counted by ncu on the Re 3500 nozzle).  The FP64 kernel keeps the FP64 pipe
-# ~87 % busy, so its roofline is that pipe, not HBM.
-FP64_FLOPS_PER_CELL = 541
+# FP64 flops per fluid-cell update of the step kernel (130 additions, 44
+# products, 80 fused pairs: 254 instructions).  The FP64 kernel keeps the FP64
+# pipe ~87 % busy, so its roofline is that pipe, not HBM.
+FP64_FLOPS_PER_CELL = 334
 FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 rate
 
 
