@@ -297,9 +297,8 @@ lbm_status lbm_get_health(lbm_ctx *ctx, double out[6]);
 /* Time averages (Sec. 2.2, mean/fluctuation decomposition and Reynolds
  * stress): from the next step on, every stride-th step adds u_z and u_z^2 of
  * every active cell to FP64 accumulators.  lbm_stats_end stops sampling.
- * While sampling, FP16S steps at the default ghost rates run one by one on the
- * chunk kernel, in roundings of their own (within a rounding of the
- * storage per step), so that averages repeat those of earlier releases. */
+ * Sampling changes nothing in the run itself: the populations are the same to
+ * the bit with it and without. */
 lbm_status lbm_stats_begin(lbm_ctx *ctx, int64_t stride);
 lbm_status lbm_stats_end(lbm_ctx *ctx);
 lbm_status lbm_stats_reset(lbm_ctx *ctx);

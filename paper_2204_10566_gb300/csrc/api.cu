@@ -271,12 +271,6 @@ bool wide_offsets(const lbm_ctx *c) { return c->wide_offsets || c->idx.nslots > 
 int64_t tile_count(const lbm_ctx *c) {
     return c->d_tiles_wall ? c->n_tiles_wall : (int64_t)c->idx.tiles.size() / TILE_INTS;
 }
-// Form of the collision of the next steps (see RATE_KEPT).
-int step_mode(const lbm_ctx *c) {
-    const bool kept = c->desc.precision == LBM_FP16S && c->mode == RATE_ONE && c->stats_on && !wide_offsets(c) &&
-                      c->fluid_kernel == FluidKernel::AUTO;
-    return kept ? RATE_KEPT : c->mode;
-}
 bool tiled(const lbm_ctx *c) {
     const FluidKernel k = c->fluid_kernel;
     const bool wanted = k == FluidKernel::TILE || k == FluidKernel::PAIRS ||
@@ -293,7 +287,7 @@ bool staged(const lbm_ctx *c) {
     const int64_t least = c->fluid_kernel == FluidKernel::STAGED ? 1
                           : c->fluid_kernel == FluidKernel::AUTO ? (int64_t)STAGE_ROUNDS * c->stage_blocks * (STEP_THREADS / 32)
                                                                  : INT64_MAX;
-    return c->desc.precision == LBM_FP16S && step_mode(c) == RATE_ONE && !wide_offsets(c) && c->stage_blocks > 0 &&
+    return c->desc.precision == LBM_FP16S && c->mode == RATE_ONE && !wide_offsets(c) && c->stage_blocks > 0 &&
            unit_count(c) >= least;
 }
 // Words of the status allocation (256 bytes): 0 the status, TICKET_WORD and
@@ -378,12 +372,10 @@ cudaError_t in_parts(lbm_ctx *c, int64_t n, cudaStream_t first_on, cudaStream_t 
 
 // Grid of the several-step kernel for the next n steps, 0 when they run one
 // by one: FP64 (bound by its arithmetic, not by launches), 64-bit offsets, a
-// fluid kernel asked for by name, FP16S with statistics on (RATE_KEPT), a
-// stream that is being captured (one recorded step is then the same kernels
-// as ever), or a larger lattice.
+// fluid kernel asked for by name, a stream that is being captured (one
+// recorded step is then the same kernels as ever), or a larger lattice.
 int run_blocks(lbm_ctx *c, int64_t n) {
-    if (n < RUN_MIN_STEPS || c->desc.precision == LBM_FP64 || wide_offsets(c) || c->fluid_kernel != FluidKernel::AUTO ||
-        step_mode(c) == RATE_KEPT)
+    if (n < RUN_MIN_STEPS || c->desc.precision == LBM_FP64 || wide_offsets(c) || c->fluid_kernel != FluidKernel::AUTO)
         return 0;
     if (c->run_mode != c->mode) {
         c->run_blocks = DISPATCH(c->desc.precision, step_run_blocks, c->mode, c->idx.row_axis, c->desc.device);
@@ -696,6 +688,7 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
             if (((lanes >> l) & 1u) && is_wall[(size_t)(base + x0 + l)]) lanes &= ~(1u << l);
         ch.y = (int)((uint32_t)x0 | (lanes << CHUNK_LANES_SHIFT));
     }
+    mark_plain_warps(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
     const std::vector<int32_t> tiles =
         wn.empty() ? std::vector<int32_t>()
                    : build_tiles(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
@@ -1133,7 +1126,7 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
             ++c->stats_samples;
         }
         int launched = 0;
-        CK(DISPATCH(c->desc.precision, launch_step, a, step_mode(c), c->stream, &launched, &c->side), "step kernel");
+        CK(DISPATCH(c->desc.precision, launch_step, a, c->mode, c->stream, &launched, &c->side), "step kernel");
         c->kernel_launches += launched;
         if (check) {
             CK(launch_finalize(c->d_partials, step_partials(c), c->d_health, c->d_status, c->stream), "finalize");

@@ -324,11 +324,31 @@ std::string build_index(const uint8_t *box_flags, int nx, int ny, int nz, int pe
             }
         }
     if ((int64_t)out.chunks.size() > (int64_t)INT32_MAX / CHUNK) return "too many chunks";
+    mark_plain_warps(out.chunks, out.row_nb, out.mask, F.np, F.pp);
     out.tiles = build_tiles(out.chunks, out.row_nb, out.mask, F.np, F.pp);
     out.units = build_units(out.chunks, out.row_nb, out.mask, F.np, F.pp);
     out.pair_items = build_pair_items(out.tiles);
     out.rest_chunks = build_rest_chunks(out.chunks, out.tiles, out.pair_items);
     return "";
+}
+
+void mark_plain_warps(std::vector<int2> &chunks, const std::vector<int32_t> &row_nb, const std::vector<uint32_t> &mask,
+                      int n_row, bool periodic_row) {
+    constexpr size_t WARP = 32 / CHUNK;
+    for (size_t k = 0; k < chunks.size(); k += WARP) {
+        bool plain = k + WARP <= chunks.size();
+        for (size_t j = k; plain && j < k + WARP; ++j) {
+            const uint32_t w = (uint32_t)chunks[j].y;
+            const int x0 = (int)(w & CHUNK_X0_MASK);
+            const uint32_t *m = &mask[(size_t)(row_nb[(size_t)chunks[j].x * ROW_RECORD_INTS + 4] + x0)];
+            plain = ((w >> CHUNK_LANES_SHIFT) & 0xFFu) == 0xFFu && !(periodic_row && (x0 == 0 || x0 + CHUNK >= n_row));
+            for (int l = 0; plain && l < CHUNK; ++l) plain = (m[l] & LINK_MASK) == 0u;
+        }
+        for (size_t j = k; j < std::min(k + WARP, chunks.size()); ++j) {
+            const uint32_t w = (uint32_t)chunks[j].y & ~CHUNK_PLAIN;
+            chunks[j].y = (int)(w | (plain ? CHUNK_PLAIN : 0u));
+        }
+    }
 }
 
 std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
@@ -339,12 +359,14 @@ std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vec
         const int x = (int)((uint32_t)chunks[k].y & CHUNK_X0_MASK);
         const int p0 = x - (nb[4] + x) % UNIT_ALIGN;  // at most one chunk before the first
         uint64_t fluid = 0, present = 0;
+        uint32_t plain_warps = 0;
         const int row = chunks[k].x;
         for (; k < chunks.size() && chunks[k].x == row; ++k) {
             const int x0 = (int)((uint32_t)chunks[k].y & CHUNK_X0_MASK), l = x0 - p0;
             if (l >= UNIT_CELLS) break;
             fluid |= (uint64_t)(((uint32_t)chunks[k].y >> CHUNK_LANES_SHIFT) & 0xFFu) << l;
             present |= (uint64_t)0xFF << l;
+            if ((uint32_t)chunks[k].y & CHUNK_PLAIN) plain_warps |= 1u << (UNIT_PLAIN_SHIFT + l / CHUNK);
         }
         bool plain = fluid == ~(uint64_t)0;
         for (int l = 0; plain && l < UNIT_CELLS; ++l) plain = (mask[(size_t)(nb[4] + p0 + l)] & LINK_MASK) == 0u;
@@ -352,7 +374,8 @@ std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vec
         const uint32_t lo = (uint32_t)__builtin_ctzll(present) / CHUNK, hi = (63u - (uint32_t)__builtin_clzll(present)) / CHUNK;
         const int32_t head[UNIT_NB] = {p0, (int32_t)(uint32_t)fluid, (int32_t)(uint32_t)(fluid >> 32),
                                        (int32_t)(uint32_t)present, (int32_t)(uint32_t)(present >> 32),
-                                       (int32_t)(lo | hi << UNIT_HI_SHIFT), (plain ? UNIT_PLAIN : 0) | (wrap ? UNIT_WRAP : 0)};
+                                       (int32_t)(lo | hi << UNIT_HI_SHIFT),
+                                       (int32_t)((plain ? UNIT_PLAIN : 0) | (wrap ? UNIT_WRAP : 0) | plain_warps)};
         units.insert(units.end(), head, head + UNIT_NB);
         units.insert(units.end(), nb, nb + 9);
     }
@@ -393,14 +416,14 @@ std::vector<int32_t> build_tiles(const std::vector<int2> &chunks, const std::vec
                                  const std::vector<uint32_t> &mask, int n_row, bool periodic_row) {
     std::vector<int32_t> tiles;
     int row = -1, p0 = 0, n = 0;  // the open tile
-    uint32_t fluid = 0, present = 0;
+    uint32_t fluid = 0, present = 0, plain_warps = 0;
     auto flush = [&]() {
         if (n == 0) return;
         // fast: 32 fluid cells without wall links, none writing a wrap-around copy
         bool fast = fluid == 0xFFFFFFFFu && !(periodic_row && (p0 == 0 || p0 + 31 >= n_row - 1));
         const int32_t base = row_nb[(size_t)row * ROW_RECORD_INTS + 4];
         for (int l = 0; fast && l < 32; ++l) fast = (mask[(size_t)(base + p0 + l)] & LINK_MASK) == 0u;
-        tiles.push_back((int32_t)((uint32_t)p0 | (fast ? TILE_FAST : 0u)));
+        tiles.push_back((int32_t)((uint32_t)p0 | (fast ? TILE_FAST : 0u) | plain_warps));
         tiles.push_back((int32_t)fluid);
         tiles.push_back((int32_t)present);
         for (int j = 0; j < 9; ++j) tiles.push_back(row_nb[(size_t)row * ROW_RECORD_INTS + j]);
@@ -413,10 +436,11 @@ std::vector<int32_t> build_tiles(const std::vector<int2> &chunks, const std::vec
             flush();
             row = c.x;
             p0 = x0;
-            fluid = present = 0;
+            fluid = present = plain_warps = 0;
         }
         fluid |= lanes << (CHUNK * n);
         present |= 0xFFu << (CHUNK * n);
+        if ((uint32_t)c.y & CHUNK_PLAIN) plain_warps |= 1u << (TILE_PLAIN_SHIFT + n);
         ++n;
     }
     flush();
@@ -550,6 +574,22 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
     for (const int4 &n : ix.bnodes)
         if (n.z < 0 || n.z >= ns || ix.row_nb[(size_t)n.y * ROW_RECORD_INTS + 4] + n.x != n.z) return "boundary node";
 
+    // Warps of the chunk kernel: the plain bit on all four chunks of a full
+    // group of fluid cells without wall links or wrap-around copies, else on none
+    std::vector<uint8_t> plain_slot((size_t)ns, 0);
+    for (size_t k = 0; k < ix.chunks.size(); ++k) {
+        const size_t first = k / 4 * 4;
+        bool plain = first + 4 <= ix.chunks.size();
+        for (size_t j = first; plain && j < first + 4; ++j)
+            for (int l = 0; l < CHUNK; ++l) {
+                const int p = (int)((uint32_t)ix.chunks[j].y & CHUNK_X0_MASK) + l;
+                const uint32_t m = ix.mask[(size_t)(ix.row_nb[(size_t)ix.chunks[j].x * ROW_RECORD_INTS + 4] + p)];
+                plain = plain && m == ((uint32_t)TYPE_FLUID << TYPE_SHIFT) && !(pp && (p == 0 || p == np - 1));
+            }
+        if (plain != (((uint32_t)ix.chunks[k].y & CHUNK_PLAIN) != 0u)) return "plain bit of a chunk";
+        if (plain) plain_slot[(size_t)(ix.row_nb[(size_t)ix.chunks[k].x * ROW_RECORD_INTS + 4] + ((uint32_t)ix.chunks[k].y & CHUNK_X0_MASK))] = 1;
+    }
+
     // Tiles of the tile kernel: every fluid cell in exactly one fluid lane, at
     // its own slot, with the bases of its own row; every lane's pulls (p0 - 1
     // .. p0 + 32 of each neighbour row, checked with a margin of 8) and link
@@ -563,7 +603,7 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
     for (int64_t t = 0; t < nt; ++t) {
         const int32_t *rec = &ix.tiles[(size_t)t * TILE_INTS];
         const bool fast = ((uint32_t)rec[0] & TILE_FAST) != 0u;
-        const int p0 = (int)((uint32_t)rec[0] & ~TILE_FAST);
+        const int p0 = (int)((uint32_t)rec[0] & CHUNK_X0_MASK);
         const uint32_t fl = (uint32_t)rec[1], pr = (uint32_t)rec[2];
         const int32_t *tb = rec + 3;
         if (p0 % CHUNK || (fl & ~pr)) return "tile start or lanes";
@@ -581,6 +621,8 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
             if (!((pr >> l) & 1u)) continue;
             const int64_t s = (int64_t)tb[4] + p0 + l;
             if (s < 0 || s >= ns) return "tile lane outside the buffer";
+            if (l % CHUNK == 0 && plain_slot[(size_t)s] != (((uint32_t)rec[0] >> (TILE_PLAIN_SHIFT + l / CHUNK)) & 1u))
+                return "plain bit of a tile";
             if (!((fl >> l) & 1u)) continue;
             const int64_t bx = box_of_slot[(size_t)s];
             if (bx < 0 || flags[bx] != LBM_FLUID || in_tile[(size_t)bx]++) return "tile lane is not a unique fluid cell";
@@ -615,6 +657,8 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
             const bool fluid = ((uint32_t)rec[1 + l / 32] >> (l % 32)) & 1u, there = ((uint32_t)rec[3 + l / 32] >> (l % 32)) & 1u;
             const int64_t s = (int64_t)ub[4] + rec[0] + l;
             if (there && (l / CHUNK < lo || l / CHUNK > hi || s < 0 || s >= ns)) return "unit lane outside its pieces or the buffer";
+            if (there && l % CHUNK == 0 && plain_slot[(size_t)s] != (((uint32_t)rec[6] >> (UNIT_PLAIN_SHIFT + l / CHUNK)) & 1u))
+                return "plain bit of a unit";
             plain = plain && fluid;
             if (!fluid) continue;
             if (!there) return "fluid lane of an absent chunk";
@@ -645,13 +689,13 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
         for (const int t : {it.x, it.y}) {
             const int32_t *rec = &ix.tiles[(size_t)t * TILE_INTS];
             if (!((uint32_t)rec[0] & TILE_FAST)) return "pair item of a tile that is not fast";
-            const uint32_t p0 = (uint32_t)rec[0] & ~TILE_FAST;
+            const uint32_t p0 = (uint32_t)rec[0] & CHUNK_X0_MASK;
             for (uint32_t k = 0; k < 4; ++k)
                 split.emplace_back(rec[3 + 4], (p0 + CHUNK * k) | (0xFFu << CHUNK_LANES_SHIFT));
         }
     }
     auto key = [&](const int2 &c) -> ChunkKey {
-        return {ix.row_nb[(size_t)c.x * ROW_RECORD_INTS + 4], (uint32_t)c.y};
+        return {ix.row_nb[(size_t)c.x * ROW_RECORD_INTS + 4], (uint32_t)c.y & ~CHUNK_PLAIN};
     };
     for (const int2 &c : ix.rest_chunks) {
         if (c.x < 0 || (int64_t)c.x >= nrows) return "rest chunk row";

@@ -12,8 +12,8 @@
 // GB300 design: pull scheme over a fluid-only slot layout (rows of cells
 // contiguous along the lattice's longer axis), structure-of-arrays
 // populations stored as deviations from the lattice weights; one warp per
-// tile of up to 32 cells of a row (FP32) or one thread per cell (FP16S,
-// FP64), with the inlet/outlet nodes and the interpolated-wall cells in
+// tile of up to 32 cells of a row (FP32), one thread per two cells over staged
+// copies (FP16S, larger lattices) or one thread per cell (smaller FP16S, FP64), with the inlet/outlet nodes and the interpolated-wall cells in
 // kernels of their own on a second stream.  Every pull source has a
 // slot (wall links read a ghost slot the cell filled with its reflected
 // population in the previous step), so the gather is 27 unconditional
@@ -187,7 +187,7 @@ __device__ __forceinline__ R cst(int a, int b) {
 template <class R>
 struct Axis {
     R d[3], g0[3], g1[3];
-    // lo, hi: u^2 - u and u^2 + u in one rounding each
+    // lo, hi: u^2 - u and u^2 + u in one rounding each, else the square is rounded first
     __device__ __forceinline__ Axis(R u, bool lo, bool hi);
 };
 
@@ -247,7 +247,7 @@ struct F2 {
 };
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(__fadd2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(__ffma2_rn(b.v, bc2(-1.0f), a.v)); }
-__device__ __forceinline__ F2 operator-(F2 a) { return F2(make_float2(-a.v.x, -a.v.y)); }
+__device__ __forceinline__ F2 operator-(F2 a) { return F2(__fmul2_rn(a.v, bc2(-1.0f))); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 &operator+=(F2 &a, F2 b) { return a = a + b; }
 __device__ __forceinline__ F2 &operator*=(F2 &a, F2 b) { return a = a * b; }
@@ -258,11 +258,21 @@ __device__ __forceinline__ F2 fma_(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 __device__ __forceinline__ F2 add_(F2 a, F2 b) { return a + b; }
 __device__ __forceinline__ F2 sub_(F2 a, F2 b) { return a - b; }
 __device__ __forceinline__ F2 mul_(F2 a, F2 b) { return a * b; }
+// Sums with a product that was rounded on its own: cell by cell, since the
+// compiler takes a packed product and a packed sum together (and a packed
+// multiply-add by one as a sum).
+__device__ __forceinline__ F2 add_apart(F2 a, F2 b) { return F2(make_float2(__fadd_rn(a.v.x, b.v.x), __fadd_rn(a.v.y, b.v.y))); }
+__device__ __forceinline__ float add_apart(float a, float b) { return __fadd_rn(a, b); }
+
+template <class R>
+__device__ __forceinline__ R pick(bool a, R x, R y) { return a ? x : y; }
+template <>
+__device__ __forceinline__ F2 pick(bool a, F2 x, F2 y) { return F2(make_float2(a ? x.v.x : y.v.x, a ? x.v.y : y.v.y)); }
 
 template <class R>
 __device__ __forceinline__ Axis<R>::Axis(R u, bool lo, bool hi) {
     const R h = R(0.5), u2 = mul_(u, u);
-    const R m = lo ? fma_(u, u, -u) : sub_(u2, u), p = hi ? fma_(u, u, u) : add_(u2, u);
+    const R m = pick(lo, fma_(u, u, -u), add_apart(u2, -u)), p = pick(hi, fma_(u, u, u), add_apart(u2, u));
     d[0] = mul_(h, m);
     d[1] = -u2;
     d[2] = mul_(h, p);
@@ -275,26 +285,27 @@ __device__ __forceinline__ Axis<R>::Axis(R u, bool lo, bool hi) {
 }
 
 // Shared inputs of the per-line inverse (see collide_ghost1).
+template <class R>
 struct PairCoef {
-    float Axx, Ayy, Azz, Axy, Axz, Ayz, rho_o, drho_o, ux, ux2h, uxh;
+    R Axx, Ayy, Azz, Axy, Axz, Ayz, rho_o, drho_o, ux, ux2h, uxh;
 };
 
 // Line (cy, cz) = (0, 0) of the inverse: f*_i - w_i for cx = -1, 0, +1.
-template <class Out>
-__device__ __forceinline__ void inverse_centre(const PairCoef &c, const Axis<float> &Y, const Axis<float> &Z,
+template <class R, class Out>
+__device__ __forceinline__ void inverse_centre(const PairCoef<R> &c, const Axis<R> &Y, const Axis<R> &Z,
                                                const Out &sink) {
-    const float h = 0.5f, w0 = cst<float>(2, 3), w1_ = cst<float>(1, 6);
-    const float gy0 = Y.g0[1], gz0 = Z.g0[1], gy1 = Y.g1[1], gz1 = Z.g1[1];
-    const float E = mul_(gy0, gz0);
-    const float D = fma_(w0, Z.d[1], mul_(Y.d[1], gz0));
-    const float C0 = fma_(mul_(c.Ayz, gy1), gz1, fma_(-c.Azz, gy0, mul_(-c.Ayy, gz0)));
-    const float B1 = fma_(mul_(c.Axy, gy1), gz0, mul_(mul_(c.Axz, gy0), gz1));
-    const float B2 = mul_(c.Axx, E);
-    const float Bw = add_(fma_(c.drho_o, w0 * w0, mul_(c.rho_o, D)), C0);
-    const float Bd = fma_(c.rho_o, E, C0), xBd = mul_(c.ux2h, Bd);
-    const float v0 = sub_(fma_(w0, Bw, mul_(-2.0f, fma_(c.ux, B1, xBd))), B2);
-    const float S = fma_(h, B2, fma_(c.ux, B1, fma_(w1_, Bw, xBd)));
-    const float A = fma_(h, B1, mul_(c.uxh, Bd));
+    const R h = R(0.5f), w0 = cst<R>(2, 3), w1_ = cst<R>(1, 6), w00 = R(cst<float>(2, 3) * cst<float>(2, 3));
+    const R gy0 = Y.g0[1], gz0 = Z.g0[1], gy1 = Y.g1[1], gz1 = Z.g1[1];
+    const R E = mul_(gy0, gz0);
+    const R D = fma_(w0, Z.d[1], mul_(Y.d[1], gz0));
+    const R C0 = fma_(mul_(c.Ayz, gy1), gz1, fma_(-c.Azz, gy0, mul_(-c.Ayy, gz0)));
+    const R B1 = fma_(mul_(c.Axy, gy1), gz0, mul_(mul_(c.Axz, gy0), gz1));
+    const R B2 = mul_(c.Axx, E);
+    const R Bw = add_(fma_(c.drho_o, w00, mul_(c.rho_o, D)), C0);
+    const R Bd = fma_(c.rho_o, E, C0), xBd = mul_(c.ux2h, Bd);
+    const R v0 = sub_(fma_(w0, Bw, mul_(R(-2.0f), fma_(c.ux, B1, xBd))), B2);
+    const R S = fma_(h, B2, fma_(c.ux, B1, fma_(w1_, Bw, xBd)));
+    const R A = fma_(h, B1, mul_(c.uxh, Bd));
     sink(4, sub_(S, A), v0, add_(S, A));
 }
 
@@ -307,7 +318,7 @@ __device__ __forceinline__ void inverse_centre(const PairCoef &c, const Axis<flo
 //   B1 = Axv g0f g1v + Axf g1f g0v,  B2 = Axx E,
 // with the same Bw, Bd, v0, S, A as the scalar line.
 template <int JA, int JB, class Out>
-__device__ __forceinline__ void inverse_pair(const PairCoef &c, const Axis<float> &Y, const Axis<float> &Z,
+__device__ __forceinline__ void inverse_pair(const PairCoef<float> &c, const Axis<float> &Y, const Axis<float> &Z,
                                              const Out &sink) {
     constexpr bool YV = (JA / 3) == (JB / 3);  // same cz: y varies
     constexpr int cf = YV ? JA / 3 - 1 : JA % 3 - 1;  // fixed axis velocity
@@ -334,6 +345,33 @@ __device__ __forceinline__ void inverse_pair(const PairCoef &c, const Axis<float
     sink(JB, om.y, o0.y, op.y);
 }
 
+// inverse_pair for two cells, a cell to a packed lane: one line after the
+// other, each value in the same order of operations.
+template <int JA, int JB, class Out>
+__device__ __forceinline__ void inverse_pair(const PairCoef<F2> &c, const Axis<F2> &Y, const Axis<F2> &Z,
+                                             const Out &sink) {
+    constexpr bool YV = (JA / 3) == (JB / 3);
+    constexpr int cf = YV ? JA / 3 - 1 : JA % 3 - 1;
+    const Axis<F2> &V = YV ? Y : Z;
+    const Axis<F2> &F = YV ? Z : Y;
+    const F2 Avv = YV ? c.Ayy : c.Azz, Aff = YV ? c.Azz : c.Ayy;
+    const F2 Axv = YV ? c.Axy : c.Axz, Axf = YV ? c.Axz : c.Axy;
+    const F2 h = F2(0.5f), f0 = F.g0[cf + 1], f1 = F.g1[cf + 1], fd = mul_(F.d[cf + 1], F2(1.0f / 6.0f));
+    const F2 P = mul_(c.Ayz, f1), Q = mul_(Aff, g2<F2>(cf)), C = mul_(mul_(h, Avv), f0);
+    const F2 b1 = mul_(mul_(h, Axv), f0), b0 = mul_(mul_(h, Axf), f1), x0 = mul_(mul_(h, c.Axx), f0), n0 = mul_(-c.Axx, f0);
+    const F2 w = mul_(c.drho_o, F2(w1<float>(cf) * (1.0f / 6.0f))), u2 = mul_(F2(2.0f), c.ux);
+#pragma unroll
+    for (int k = 0; k < 3; k += 2) {
+        const F2 v0 = V.g0[k], v1 = V.g1[k];
+        const F2 E = mul_(v0, f0), D = fma_(V.d[k], f0, fd), C0 = fma_(v1, P, fma_(v0, Q, C)), hB1 = fma_(v1, b1, mul_(v0, b0));
+        const F2 Bw = fma_(c.rho_o, D, add_apart(C0, w)), Bd = fma_(c.rho_o, E, C0);
+        const F2 t = fma_(c.ux2h, Bd, mul_(u2, hB1)), A = fma_(c.uxh, Bd, hB1);
+        const F2 o0 = fma_(F2(2.0f / 3.0f), Bw, fma_(F2(-2.0f), t, mul_(v0, n0)));
+        const F2 S = fma_(F2(1.0f / 6.0f), Bw, fma_(v0, x0, t));
+        sink(k ? JB : JA, sub_(S, A), o0, add_(S, A));
+    }
+}
+
 // Writes a line of three outputs (cx = -1, 0, +1 of line j) back into d.
 template <class R>
 struct ToArray {
@@ -356,78 +394,93 @@ struct ToArrayStress {
     __device__ __forceinline__ void operator()(int j, R vm, R v0, R vp) const { ToArray<R>{d}(j, vm, v0, vp); }
 };
 
-// Moment sums of the FP32 default-rate collision: m = drho, jx, jy, jz, pxx,
-// pyy, pzz, pxy, pxz, pyz, the sums of (f - w) weighted by 1, c, and c_a c_b.
-// The x-pass sums each (cy, cz) line with weights 1, cx, cx^2; the other axes
-// follow.
-template <class R>
-__device__ __forceinline__ void ghost1_sums(const R (&d)[27], R (&m)[10]) {
+// Moment sums of the FP32 and FP16S collisions: m = drho, jx, jy, jz, pxx,
+// pyy, pzz, pxy, pxz, pyz, the sums of (f - w) weighted by 1, c, and c_a c_b;
+// ld(i) gives f_i - w_i, or a power of two times it, of one cell (R = float)
+// or two (R = F2).  The x-pass sums each (cy, cz) line with weights 1, cx,
+// cx^2; the other axes follow.
+template <class R, class Load>
+__device__ __forceinline__ void ghost1_sums(const Load &ld, R (&m)[10]) {
     R s0[9], s1[9], s2[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
-        const R a = d[3 * j], b = d[3 * j + 1], c = d[3 * j + 2];
+        const R a = ld(3 * j), b = ld(3 * j + 1), c = ld(3 * j + 2);
         s0[j] = (a + b) + c;
         s1[j] = c - a;
         s2[j] = c + a;
     }
-    R drho = 0, jx = 0, jy = 0, jz = 0, pxx = 0, pyy = 0, pzz = 0, pxy = 0, pxz = 0, pyz = 0;
+    R drho = s0[0], jx = s1[0], pxx = s2[0];
 #pragma unroll
-    for (int j = 0; j < 9; ++j) {
-        const int cy = j % 3 - 1, cz = j / 3 - 1;
+    for (int j = 1; j < 9; ++j) {
         drho += s0[j];
         jx += s1[j];
         pxx += s2[j];
-        if (cy != 0) {
-            jy += cy > 0 ? s0[j] : -s0[j];
-            pyy += s0[j];
-            pxy += cy > 0 ? s1[j] : -s1[j];
-        }
-        if (cz != 0) {
-            jz += cz > 0 ? s0[j] : -s0[j];
-            pzz += s0[j];
-            pxz += cz > 0 ? s1[j] : -s1[j];
-        }
-        if (cy != 0 && cz != 0) pyz += (cy * cz) > 0 ? s0[j] : -s0[j];
     }
+    // lines in storage order, each pair of a column's first two at once
+    const R jy = (((((s0[2] - s0[0]) - s0[3]) + s0[5]) - s0[6]) + s0[8]), pyy = ((((s0[0] + s0[2]) + s0[3]) + s0[5]) + s0[6]) + s0[8];
+    const R pxy = ((((s1[2] - s1[0]) - s1[3]) + s1[5]) - s1[6]) + s1[8];
+    // z: lines 0 1 2 against 6 7 8, one after the other
+    const R zn = (s0[0] + s0[1]) + s0[2], xn = (s1[0] + s1[1]) + s1[2];
+    const R jz = ((s0[6] - zn) + s0[7]) + s0[8], pzz = ((zn + s0[6]) + s0[7]) + s0[8], pxz = ((s1[6] - xn) + s1[7]) + s1[8];
+    const R pyz = ((s0[0] - s0[2]) - s0[6]) + s0[8];
     m[0] = drho, m[1] = jx, m[2] = jy, m[3] = jz, m[4] = pxx;
     m[5] = pyy, m[6] = pzz, m[7] = pxy, m[8] = pxz, m[9] = pyz;
 }
 
-// The rest of the FP32 default-rate collision from the moment sums: rho, u, the
-// six second-order central Hermite moments, their relaxation, and the
-// inverse transform, line by line into sink(j, f*_{3j} - w, f*_{3j+1} - w,
-// f*_{3j+2} - w).  With SCALED (RATE_KEPT of FP16S) the sums are of
-// (f - w) / in_scale and the outputs are (f* - w) * out_scale: the scales,
-// powers of two, act on the ten moments and the eight output coefficients.
-// fused: the roundings of the y and z columns, see RATE_KEPT.
-template <bool SCALED, class Out>
-__device__ __forceinline__ void ghost1_finish(const float (&m)[10], float omega, float &rho, float &ux, float &uy,
-                                              float &uz, float in_scale, float out_scale, bool fused, const Out &sink) {
-    const float drho = SCALED ? mul_(m[0], in_scale) : m[0], th = theta0<float>();
-    rho = add_(1.0f, drho);
-    const float inv = recip(rho);
+// Roundings of the rate-1 collision in FP32 arithmetic.  Where a product
+// meets a sum it is rounded before the sum or taken into it (a fused
+// multiply-add), and FP16 storage carries such a difference on: in some 50
+// steps it grows to the size of the storage's own noise, 1e-3 of a velocity.
+// So each FP16S cell keeps one set of roundings whatever kernel updates it and
+// whether statistics are sampled: whole warps of plain cells in the chunk list
+// (CHUNK_PLAIN) and cells with interpolated walls take the default, the other
+// cells lane_rounds, the request server's served_rounds.  y, z: u_y^2 -+ u_y
+// and u_z^2 + u_z in one rounding; late: the second-order moments' scale first.
+struct Rounds {
+    bool y = false, z = false, late = false;
+};
+template <int AX>
+__device__ __forceinline__ Rounds lane_rounds(bool plain) { return {!plain, !plain && AX == 2, false}; }
+__device__ __forceinline__ constexpr Rounds served_rounds() { return {true, true, true}; }
+
+// The rest of the FP32 / FP16S default-rate collision from the moment sums:
+// rho, u, the six second-order central Hermite moments, their relaxation, and
+// the inverse transform, line by line into sink(j, f*_{3j} - w, f*_{3j+1} - w,
+// f*_{3j+2} - w).  With SCALED (FP16S) the sums are of (f - w) / in_scale and
+// the outputs are (f* - w) * out_scale: the scales, powers of two, act on the
+// ten moments and the eight output coefficients.
+template <bool SCALED, class R, class Out>
+__device__ __forceinline__ void ghost1_finish(const R (&m)[10], R omega, R &rho, R &ux, R &uy, R &uz, R in_scale,
+                                              R out_scale, Rounds rounds, const Out &sink) {
+    const R drho = SCALED ? mul_(m[0], in_scale) : m[0], th = theta0<R>();
+    rho = add_(R(1.0f), drho);
+    const R inv = recip(rho);
     ux = mul_(SCALED ? mul_(m[1], in_scale) : m[1], inv);
     uy = mul_(SCALED ? mul_(m[2], in_scale) : m[2], inv);
     uz = mul_(SCALED ? mul_(m[3], in_scale) : m[3], inv);
     // Second-order central Hermite moments sum_i ((c-u)_a (c-u)_b - theta0 delta_ab) f_i,
     // from the deviation moments (sum c_a c_b w = theta0 delta_ab).
-    const float rx = -mul_(rho, ux), ry = -mul_(rho, uy), rz = -mul_(rho, uz);
-    auto less = [&](float p, float r, float u) { return SCALED ? fma_(p, in_scale, mul_(r, u)) : fma_(r, u, p); };
-    const float a2[6] = {fma_(-th, drho, less(m[4], rx, ux)), fma_(-th, drho, less(m[5], ry, uy)),
-                         fma_(-th, drho, less(m[6], rz, uz)), less(m[7], rx, uy),
-                         less(m[8], rx, uz),                  less(m[9], ry, uz)};
+    const R rx = -mul_(rho, ux), ry = -mul_(rho, uy), rz = -mul_(rho, uz);
+    auto less = [&](R p, R r, R u) {
+        if (!SCALED) return fma_(r, u, p);
+        return rounds.late ? fma_(r, u, mul_(p, in_scale)) : fma_(p, in_scale, mul_(r, u));
+    };
+    const R a2[6] = {fma_(-th, drho, less(m[4], rx, ux)), fma_(-th, drho, less(m[5], ry, uy)),
+                     fma_(-th, drho, less(m[6], rz, uz)), less(m[7], rx, uy),
+                     less(m[8], rx, uz),                  less(m[9], ry, uz)};
     sink.moments(omega, a2);
     // Inverse: f* = rho prod g0 + sum over the six relaxed second-order moments
     // of A_m prod_a g_{m_a}; orders 1 and 3..6 are zero after relaxation.
     // Per (cy, cz) line the x-dependence is spanned by {w, d, g1, g2}(cx):
     //   f*_i - w_i = wx Bw + dx Bd + g1x B1 + g2x B2,
-    // and for cx = +-1 this splits into S +- A.  Lines go in pairs on the
-    // packed FP32 pipe (two lanes per instruction): (cy = -1, +1) at each cz,
-    // then (cz = -1, +1) at cy = 0; the centre line alone.
-    const float one_w = sub_(1.0f, omega), k = SCALED ? mul_(one_w, out_scale) : one_w, uxh = mul_(0.5f, ux);
-    const Axis<float> Y(uy, fused, fused), Z(uz, false, fused);
-    const PairCoef c{mul_(k, a2[0]), mul_(k, a2[1]), mul_(k, a2[2]), mul_(k, a2[3]), mul_(k, a2[4]), mul_(k, a2[5]),
-                     SCALED ? mul_(rho, out_scale) : rho, SCALED ? mul_(drho, out_scale) : drho, ux, mul_(uxh, ux), uxh};
+    // and for cx = +-1 this splits into S +- A.  One cell's lines go in pairs
+    // on the packed FP32 pipe (two lanes per instruction): (cy = -1, +1) at
+    // each cz, then (cz = -1, +1) at cy = 0; two cells' lines one by one with a
+    // cell to a lane; the centre line alone.
+    const R one_w = sub_(R(1.0f), omega), k = SCALED ? mul_(one_w, out_scale) : one_w, uxh = mul_(R(0.5f), ux);
+    const Axis<R> Y(uy, rounds.y, rounds.y), Z(uz, false, rounds.z);
+    const PairCoef<R> c{mul_(k, a2[0]), mul_(k, a2[1]), mul_(k, a2[2]), mul_(k, a2[3]), mul_(k, a2[4]), mul_(k, a2[5]),
+                        SCALED ? mul_(rho, out_scale) : rho, SCALED ? mul_(drho, out_scale) : drho, ux, mul_(uxh, ux), uxh};
     inverse_pair<0, 2>(c, Y, Z, sink);
     inverse_pair<3, 5>(c, Y, Z, sink);
     inverse_pair<6, 8>(c, Y, Z, sink);
@@ -435,14 +488,11 @@ __device__ __forceinline__ void ghost1_finish(const float (&m)[10], float omega,
     inverse_centre(c, Y, Z, sink);
 }
 
-// The FP16S form of the two parts above, for one cell (R = float) or two
-// (R = F2).  ld(i) gives the stored value (f_i - w_i) / in_scale (FP64 takes
-// the sums too).
-//
-// The moment sums run axis by axis (x within a line, then y, then z), each
-// +-1 pair summed and differenced once: 67 operations.
+// The same moment sums axis by axis (x within a line, then y, then z), each
+// +-1 pair summed and differenced once: 67 operations.  The form of FP64, the
+// general collision and the FP32 / FP64 inlet/outlet nodes.
 template <class R, class Load>
-__device__ __forceinline__ void scaled_sums(const Load &ld, R (&m)[10]) {
+__device__ __forceinline__ void axis_sums(const Load &ld, R (&m)[10]) {
     R t0[3], e0[3], d0[3], t1[3], d1[3], t2[3];  // per cz: sums over cy of s0, s2-in-y, s1-in-y, ...
 #pragma unroll
     for (int z = 0; z < 3; ++z) {
@@ -475,8 +525,15 @@ __device__ __forceinline__ void scaled_sums(const Load &ld, R (&m)[10]) {
 }
 
 // The lines of ro f^eq/rho + sum k a_ab g_ab at velocity u, less the weights'
-// part (ro - dro) w: the inverse transform described at scaled_finish.  With
-// ro = dro = 0 it gives the part of the relaxed second-order moments alone.
+// part (ro - dro) w.  With ro = dro = 0 it gives the part of the relaxed
+// second-order moments alone.  With the half coefficients
+//   P0 = rho gz0 + Azz g2z, P1 = Ayz gz1, P2 = Ayy gz0   (cz level)
+//   T = uy^2/2 P0 + uy P1 + P2/2,  O = (uy P0 + P1) / 2  (cy = +-1: +-O)
+// a line's coefficients are Bd = gy0 P0 + gy1 P1 + g2y P2 = w P0 + T +- O and
+// Bw = Bd - wy wz in the form w W0 + T +- O, W0 = rho dz + drho wz + Azz g2z,
+// which has no O(1) cancellation; cy = 0 takes -2 T.  Along x, with
+// u = ux^2/2 Bd + ux B1 + B2/2: f*_0 = 2/3 Bw - 2 u and f*_+- = Bw/6 + u
+// +- (ux Bd + B1)/2.
 template <class R, class Out>
 __device__ __forceinline__ void relaxed_lines(R k, const R (&a2)[6], R ro, R dro, R ux, R uy, R uz, const Out &sink) {
     const R h = R(0.5), w0 = cst<R>(2, 3), w1_ = cst<R>(1, 6), m2 = R(-2), hk = mul_(h, k);
@@ -508,36 +565,6 @@ __device__ __forceinline__ void relaxed_lines(R k, const R (&a2)[6], R ro, R dro
             sink(3 * z + y, sub_(S, A), fma_(m2, u, mul_(w0, Bw)), add_(S, A));
         }
     }
-}
-
-// Relaxation and inverse transform.  With the half coefficients
-//   P0 = rho gz0 + Azz g2z, P1 = Ayz gz1, P2 = Ayy gz0   (cz level)
-//   T = uy^2/2 P0 + uy P1 + P2/2,  O = (uy P0 + P1) / 2  (cy = +-1: +-O)
-// a line's coefficients are Bd = gy0 P0 + gy1 P1 + g2y P2 = w P0 + T +- O and
-// Bw = Bd - wy wz in the form w W0 + T +- O, W0 = rho dz + drho wz + Azz g2z,
-// which has no O(1) cancellation; cy = 0 takes -2 T.  Along x, with
-// u = ux^2/2 Bd + ux B1 + B2/2: f*_0 = 2/3 Bw - 2 u and f*_+- = Bw/6 + u
-// +- (ux Bd + B1)/2.  About 180 operations, against 230 line by line.
-template <class R, class Out>
-__device__ __forceinline__ void scaled_finish(const R (&m)[10], R omega, R &rho, R &ux, R &uy, R &uz, R in_scale,
-                                              R out_scale, const Out &sink) {
-    const R drho = mul_(m[0], in_scale), jx = mul_(m[1], in_scale), jy = mul_(m[2], in_scale), jz = mul_(m[3], in_scale);
-    rho = add_(R(1), drho);
-    const R inv = recip(rho);
-    ux = mul_(jx, inv);
-    uy = mul_(jy, inv);
-    uz = mul_(jz, inv);
-    const R mjx = -jx, mjy = -jy, mth = -theta0<R>();
-    // second-order central Hermite moments p_ab - rho u_a u_b - theta0 drho delta_ab
-    const R a2[6] = {fma_(mjx, ux, fma_(mth, drho, mul_(m[4], in_scale))),
-                     fma_(mjy, uy, fma_(mth, drho, mul_(m[5], in_scale))),
-                     fma_(-jz, uz, fma_(mth, drho, mul_(m[6], in_scale))),
-                     fma_(mjx, uy, mul_(m[7], in_scale)),
-                     fma_(mjx, uz, mul_(m[8], in_scale)),
-                     fma_(mjy, uz, mul_(m[9], in_scale))};
-    sink.moments(omega, a2);
-    const R k = mul_(sub_(R(1), omega), out_scale);
-    relaxed_lines<R>(k, a2, mul_(rho, out_scale), mul_(drho, out_scale), ux, uy, uz, sink);
 }
 
 // The FP64 form of the second part.  FP64 is bound by its arithmetic pipe, so
@@ -637,40 +664,21 @@ __device__ __forceinline__ void raw_finish(const R (&m)[10], R omega, R &rho, R 
 }
 
 // Collision with the default ghost rates (all 1).  d holds f_i - w_i on entry;
-// the post-collision f*_i - w_i go to the sink line by line, or back into d
-// without one.  rho, u receive the (conserved) moments.  With SCALED, d holds
-// (f_i - w_i) / in_scale and the outputs are (f*_i - w_i) * out_scale.
-template <class R, bool SCALED = false, class Out = ToArray<R>>
-__device__ __forceinline__ void collide_ghost1(R (&d)[27], R omega, R &rho, R &ux, R &uy, R &uz,
-                                               R in_scale = R(1), R out_scale = R(1), const Out *sink = nullptr) {
+// the post-collision f*_i - w_i go to the sink line by line.  rho, u receive
+// the (conserved) moments.  With SCALED, d holds (f_i - w_i) / in_scale and the
+// outputs are (f*_i - w_i) * out_scale.
+template <class R, bool SCALED = false, class Out>
+__device__ __forceinline__ void collide_ghost1(R (&d)[27], R omega, R &rho, R &ux, R &uy, R &uz, R in_scale, R out_scale,
+                                               const Out &sink, Rounds rounds = Rounds()) {
     R m[10];
-    if constexpr (SCALED) {
-        scaled_sums<R>([&](int i) { return d[i]; }, m);
-        scaled_finish<R>(m, omega, rho, ux, uy, uz, in_scale, out_scale, *sink);
-    } else if constexpr (std::is_same<R, double>::value) {
-        scaled_sums<R>([&](int i) { return d[i]; }, m);
-        if (sink)
-            raw_finish<R>(m, omega, rho, ux, uy, uz, *sink);
-        else
-            raw_finish<R>(m, omega, rho, ux, uy, uz, ToArray<R>{d});
+    auto ld = [&](int i) { return d[i]; };
+    if constexpr (std::is_same<R, double>::value) {
+        axis_sums<R>(ld, m);
+        raw_finish<R>(m, omega, rho, ux, uy, uz, sink);
     } else {
-        ghost1_sums(d, m);
-        if (sink)
-            ghost1_finish<false>(m, omega, rho, ux, uy, uz, 1.0f, 1.0f, false, *sink);
-        else
-            ghost1_finish<false>(m, omega, rho, ux, uy, uz, 1.0f, 1.0f, false, ToArray<R>{d});
+        ghost1_sums<R>(ld, m);
+        ghost1_finish<SCALED, R>(m, omega, rho, ux, uy, uz, in_scale, out_scale, SCALED ? rounds : Rounds(), sink);
     }
-}
-
-// The same with the roundings of RATE_KEPT (FP16S).  fused: of the columns,
-// as in the fluid lanes outside the uniform warps of a lattice with rows
-// along z.
-template <bool SCALED, class Out>
-__device__ __forceinline__ void collide_kept(float (&d)[27], float omega, float &rho, float &ux, float &uy, float &uz,
-                                             float in_scale, float out_scale, bool fused, const Out &sink) {
-    float m[10];
-    ghost1_sums(d, m);
-    ghost1_finish<SCALED>(m, omega, rho, ux, uy, uz, in_scale, out_scale, fused, sink);
 }
 
 // The equilibrium part alone: the lines of ro f^eq(u)/rho less (ro - dro) w,
@@ -708,13 +716,13 @@ struct EqLines {
 // Collision with every ghost rate equal to omega.  T^-1 S T is then omega on
 // all but the conserved moments, on which f^eq - f has no part, so the step
 // is lattice BGK with the full equilibrium (Sec. 2.1): f* = f + omega (f^eq
-// - f), in deviations, with the equilibrium's lines as in scaled_finish.
+// - f), in deviations, with the equilibrium's lines as in relaxed_lines.
 // About 250 operations instead of 600 for the 27-moment cascade, and no 27
 // moments to hold.
 template <class R, class Out>
 __device__ __forceinline__ void collide_bgk(R (&d)[27], R omega, R &rho, R &ux, R &uy, R &uz, const Out &sink) {
     R m[10];
-    ghost1_sums(d, m);
+    ghost1_sums<R>([&](int i) { return d[i]; }, m);
     const R drho = m[0], jx = m[1], jy = m[2], jz = m[3], th = theta0<R>();
     rho = add_(R(1), drho);
     const R inv = recip(rho);
@@ -769,7 +777,7 @@ template <class R, class Sink = ToArray<R>>
 __device__ __forceinline__ void collide_general(R (&d)[27], R omega, const R (&ghost)[4], R &rho, R &ux,
                                                 R &uy, R &uz, const Sink *sink = nullptr) {
     R s[10];
-    scaled_sums<R>([&](int i) { return d[i]; }, s);
+    axis_sums<R>([&](int i) { return d[i]; }, s);
     const R drho = s[0];
     rho = add_(R(1), drho);
     const R inv = recip(rho);
@@ -1002,9 +1010,7 @@ __device__ __forceinline__ void collide(typename Storage<P>::R (&d)[27], const F
     using R = typename Storage<P>::R;
     const ToArrayStress<R> sink{a, stress_slot, d};
     if constexpr (G == RATE_ONE)
-        collide_ghost1<R, false, ToArrayStress<R>>(d, fp.omega, rho, ux, uy, uz, R(1), R(1), &sink);
-    else if constexpr (G == RATE_KEPT)
-        collide_kept<false>(d, fp.omega, rho, ux, uy, uz, 1.0f, 1.0f, false, sink);
+        collide_ghost1<R>(d, fp.omega, rho, ux, uy, uz, R(1), R(1), sink);
     else if constexpr (G == RATE_BGK)
         collide_bgk<R>(d, fp.omega, rho, ux, uy, uz, sink);
     else
@@ -1164,11 +1170,16 @@ struct OwnStore {
 };
 
 template <class R>
+__device__ __forceinline__ void record_axial(const StepArgs &a, int slot, R uz) {
+    const double w = (double)uz;
+    a.stats[slot] += w;
+    a.stats[a.stride + slot] = fma_(w, w, a.stats[a.stride + slot]);
+}
+
+template <class R>
 __device__ __forceinline__ void record_cell(const StepArgs &a, int slot, R rho, R ux, R uy, R uz, double (&hv)[6]) {
     if (a.flags & STEP_STATS) {
-        const double w = (double)uz;
-        a.stats[slot] += w;
-        a.stats[a.stride + slot] = fma_(w, w, a.stats[a.stride + slot]);
+        record_axial(a, slot, uz);
         if (a.flags & STEP_STATS_FULL) {  // time averages of u, u u and rho (Sec. 2.2)
             const double u[3] = {(double)ux, (double)uy, (double)uz};
             double *p = a.stats + 2 * (int64_t)a.stride + slot;
@@ -1195,7 +1206,7 @@ __device__ __forceinline__ void record_cell(const StepArgs &a, int slot, R rho, 
 // at the row ends, which the memory system would otherwise have to read
 // back before writing them, at no extra instructions per warp.
 template <int P, int G, bool WIDE, bool WALLQ, int AX, bool CG = false>
-__device__ __forceinline__ void cell_update(const StepArgs &a, int row, int x, bool fluid, int qk, double (&hv)[6]) {
+__device__ __forceinline__ void cell_update(const StepArgs &a, int row, int x, bool fluid, bool plain, int qk, double (&hv)[6]) {
     using R = typename Storage<P>::R;
     int nb[9];
     load_row(a.row_nb, row, nb);
@@ -1206,16 +1217,14 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int row, int x, b
                                : (((m >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~m & LINK_MASK) : 0u);
     R d[27];
     R rho, ux, uy, uz;
-    constexpr bool RAW = (G == RATE_ONE || G == RATE_KEPT) && Storage<P>::SCALED;  // FP16 scale folded into the collision
+    constexpr bool RAW = G == RATE_ONE && Storage<P>::SCALED;  // FP16 scale folded into the collision
     gather<P, WIDE, AX, RAW, CG>(a, nb, x, d);
     if constexpr (WALLQ) interpolate_walls<P, WIDE, RAW, CG>(a, qk, slot, links, d);
     if constexpr (G != RATE_GENERAL) {
         const LineStore<P, WIDE, RAW, AX> sink{a, nb, x, slot, links, own};
         if constexpr (G == RATE_ONE)
-            collide_ghost1<R, RAW, LineStore<P, WIDE, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
-                                                                R(a.scale), &sink);
-        else if constexpr (G == RATE_KEPT)
-            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, false, sink);
+            collide_ghost1<R, RAW>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale), sink,
+                                   lane_rounds<AX>(plain));
         else
             collide_bgk<R>(d, flow<R>(a).omega, rho, ux, uy, uz, sink);
     } else {
@@ -1231,7 +1240,7 @@ __device__ __forceinline__ void fluid_cell(const StepArgs &a, int chunk, int lan
     const int2 ch = __ldg(a.chunks + chunk);
     const uint32_t cw = (uint32_t)ch.y;
     const bool fluid = (cw >> (CHUNK_LANES_SHIFT + lane)) & 1u;
-    cell_update<P, G, WIDE, false, AX, CG>(a, ch.x, (int)(cw & CHUNK_X0_MASK) + lane, fluid, -1, hv);
+    cell_update<P, G, WIDE, false, AX, CG>(a, ch.x, (int)(cw & CHUNK_X0_MASK) + lane, fluid, cw & CHUNK_PLAIN, -1, hv);
 }
 
 // Fluid lane of the step kernel with a warp-uniform fast path (default ghost
@@ -1251,11 +1260,12 @@ __device__ __forceinline__ void fluid_lane_voted(const StepArgs &a, int chunk, i
     R d[27];
     int x = 0, slot = 0;
     uint32_t m = 0u;
-    bool fluid = false;
+    bool fluid = false, plain = false;
     if (valid) {
         const int2 ch = __ldg(a.chunks + chunk);
         const uint32_t cw = (uint32_t)ch.y;
         fluid = (cw >> (CHUNK_LANES_SHIFT + lane)) & 1u;
+        plain = cw & CHUNK_PLAIN;
         x = (int)(cw & CHUNK_X0_MASK) + lane;
         load_row(a.row_nb, ch.x, nb);
         slot = nb[4] + x;
@@ -1269,21 +1279,13 @@ __device__ __forceinline__ void fluid_lane_voted(const StepArgs &a, int chunk, i
     R rho, ux, uy, uz;
     if (fast) {
         const OwnStore<P, RAW> sink{a, slot};
-        if constexpr (G == RATE_KEPT)
-            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, false, sink);
-        else
-            collide_ghost1<R, RAW, OwnStore<P, RAW>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
-                                                     R(a.scale), &sink);
+        collide_ghost1<R, RAW>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale), sink, lane_rounds<AX>(plain));
     } else {
         const uint32_t links = fluid ? (m & LINK_MASK) : 0u;
         const uint32_t own = fluid ? (LINK_MASK | OWN_FLUID)
                                    : (((m >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~m & LINK_MASK) : 0u);
         const LineStore<P, false, RAW, AX> sink{a, nb, x, slot, links, own};
-        if constexpr (G == RATE_KEPT)
-            collide_kept<true>(d, flow<R>(a).omega, rho, ux, uy, uz, a.inv_scale, a.scale, AX == 2, sink);
-        else
-            collide_ghost1<R, RAW, LineStore<P, false, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz,
-                                                             R(a.inv_scale), R(a.scale), &sink);
+        collide_ghost1<R, RAW>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale), sink, lane_rounds<AX>(plain));
     }
     if (fluid) record_cell(a, slot, rho, ux, uy, uz, hv);
 }
@@ -1295,7 +1297,7 @@ __device__ __forceinline__ void fluid_lane_voted(const StepArgs &a, int chunk, i
 template <int P, int G, bool WIDE, int AX, bool CG = false>
 __device__ __forceinline__ void wall_cell(const StepArgs &a, int k, double (&hv)[6]) {
     const int4 node = __ldg(a.wnodes + k);
-    cell_update<P, G, WIDE, true, AX, CG>(a, node.y, node.x, true, node.w, hv);
+    cell_update<P, G, WIDE, true, AX, CG>(a, node.y, node.x, true, true, node.w, hv);
 }
 
 // Output sink of an inlet/outlet node: f* - f^eq of the partner comes in, the
@@ -1334,8 +1336,8 @@ struct NodeStore {
 };
 
 // One line (cx = -1, 0, 1) of f^eq(rho, u) - w in product form, without O(1)
-// cancellation: (rho - 1) w + rho (dx gy gz + wx (dy gz + wy dz)), with the
-// roundings of RATE_KEPT.
+// cancellation: (rho - 1) w + rho (dx gy gz + wx (dy gz + wy dz)).  The FP16S
+// nodes' form, with one set of roundings as in Rounds.
 struct EqNode {
     Axis<float> X, Y, Z;
     float r, dr;
@@ -1359,7 +1361,8 @@ struct EqNode {
 //   f*_i(x_b) = f^eq_i(rho_b, u_b) + f*_i(x_f) - f^eq_i(rho_f, u_f),
 // inlet: rho_b = rho_f, u_b prescribed; outlet: rho_b = rho_out, u_b = u_f.
 // With the default rates f* - f^eq of the partner is its relaxed
-// second-order part alone, so no equilibrium of the partner is formed.
+// second-order part alone, so no equilibrium of the partner is formed (FP16S
+// forms both, see Rounds).
 // Few nodes run at a time, each a chain of latencies; what counts is the
 // depth of the dependent loads (record, pulls) and the operations after
 // them.
@@ -1407,9 +1410,9 @@ __device__ __forceinline__ void boundary_node(const StepArgs &a, int k, double (
         if (lf) interpolate_walls<P, WIDE, false, CG>(a, __ldg(a.wall_qidx + sf), sf, lf, d);
     }
     R rho;
-    if constexpr (G == RATE_ONE) {
+    if constexpr (G == RATE_ONE && P != 2) {
         R s[10];
-        scaled_sums<R>([&](int i) { return d[i]; }, s);
+        axis_sums<R>([&](int i) { return d[i]; }, s);
         const R drho = s[0], jx = s[1], jy = s[2], jz = s[3], th = theta0<R>();
         rho = add_(R(1), drho);
         const R inv = recip(rho), uxf = mul_(jx, inv), uyf = mul_(jy, inv), uzf = mul_(jz, inv);
@@ -1427,7 +1430,7 @@ __device__ __forceinline__ void boundary_node(const StepArgs &a, int k, double (
         collide<P, G>(d, fp, rf, uxf, uyf, uzf, a, slot);  // the node takes its partner's stress
         if (!inlet) ux = uxf, uy = uyf, uz = uzf;
         rho = inlet ? rf : fp.rho_out;
-        if constexpr (G == RATE_KEPT) {
+        if constexpr (G == RATE_ONE) {
             const EqNode fe(rf, uxf, uyf, uzf), be(rho, ux, uy, uz);
             const NodeStore<P, WIDE, AX> out{a, slot, pos, EqLines<R>(rho, R(0), ux, uy, uz)};
 #pragma unroll
@@ -1500,7 +1503,7 @@ __global__ void __launch_bounds__(STEP_THREADS, P == 0 ? 1 : (G == RATE_GENERAL 
     } else {
         const int gt = blockIdx.x * STEP_THREADS + threadIdx.x;
         const int chunk = gt / CHUNK;
-        if constexpr (LBM_FAST_PATH && (G == RATE_ONE || G == RATE_KEPT) && !WIDE && P != 0)
+        if constexpr (LBM_FAST_PATH && G == RATE_ONE && !WIDE && P != 0)
             fluid_lane_voted<P, G, AX>(a, chunk, gt % CHUNK, hv);  // every lane of the block calls it
         else if (chunk < a.nchunks)
             fluid_cell<P, G, WIDE, AX>(a, chunk, gt % CHUNK, hv);
@@ -1594,8 +1597,9 @@ struct TileRec {
 // One warp's update of a tile (lane = the warp lane, out = the warp's
 // shared-memory slice of TileOut<P>::ELEMS elements).  Without FAST every tile
 // takes the line sink, and out is not used: half the code, for kernels that
-// otherwise wait on the instruction cache.
-template <int P, int AX, bool CG = false, bool FAST = true>
+// otherwise wait on the instruction cache.  SERVED: the request server's
+// roundings.
+template <int P, int AX, bool CG = false, bool FAST = true, bool SERVED = false>
 __device__ __forceinline__ void tile_update(const StepArgs &a, const TileRec &rec, int lane, typename TileOut<P>::T *out,
                                             double (&hv)[6]) {
     using O = TileOut<P>;
@@ -1608,13 +1612,14 @@ __device__ __forceinline__ void tile_update(const StepArgs &a, const TileRec &re
     const int p0 = (int)((uint32_t)r0.x & CHUNK_X0_MASK);
     const int x = p0 + lane, slot = nb[4] + x;
     const bool fluid = ((uint32_t)r0.y >> lane) & 1u;
+    const Rounds rounds =
+        SERVED ? served_rounds() : lane_rounds<AX>(((uint32_t)r0.x >> (TILE_PLAIN_SHIFT + lane / CHUNK)) & 1u);
     R d[27];
     gather<P, false, AX, RAW, CG>(a, nb, x, d);  // every lane's pulls lie inside the buffer margins
     R rho, ux, uy, uz;
     if (FAST && fast) {
         const SharedStore<P, RAW> sink{a, slot, out + lane};
-        collide_ghost1<R, RAW, SharedStore<P, RAW>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
-                                                    R(a.scale), &sink);
+        collide_ghost1<R, RAW>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale), sink, rounds);
         __syncwarp();
         // piece q = 4 i + k (FP16S) / 8 i + k (FP32): elements 16k/S.. of population i,
         // at shared offset 16 q bytes and at own slots nb[4] + p0 + k PIECE
@@ -1636,8 +1641,7 @@ __device__ __forceinline__ void tile_update(const StepArgs &a, const TileRec &re
         const uint32_t own = fluid ? (LINK_MASK | OWN_FLUID)
                                    : (present && ((m >> TYPE_SHIFT) & 3u) == TYPE_PAD ? (~m & LINK_MASK) : 0u);
         const LineStore<P, false, RAW, AX> sink{a, nb, x, slot, links, own};
-        collide_ghost1<R, RAW, LineStore<P, false, RAW, AX>>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale),
-                                                             R(a.scale), &sink);
+        collide_ghost1<R, RAW>(d, flow<R>(a).omega, rho, ux, uy, uz, R(a.inv_scale), R(a.scale), sink, rounds);
     }
     if (fluid) record_cell(a, slot, rho, ux, uy, uz, hv);
 }
@@ -1729,8 +1733,9 @@ __device__ __forceinline__ void pair_update(const StepArgs &a, int t, int k, dou
     __half2 d[27];
     gather_pair<AX>(a, nb, x, d);
     F2 m[10], rho, ux, uy, uz;
-    scaled_sums<F2>([&](int i) { return Half2ToF2{}(d[i]); }, m);
-    scaled_finish<F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale), PairStore{a, slot});
+    ghost1_sums<F2>([&](int i) { return Half2ToF2{}(d[i]); }, m);
+    ghost1_finish<true, F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale),
+                            lane_rounds<AX>(((uint32_t)r0.x >> (TILE_PLAIN_SHIFT + 2 * k / CHUNK)) & 1u), PairStore{a, slot});
     double h0[6] = {0, 0, 0, 0, 0, 0}, h1[6] = {0, 0, 0, 0, 0, 0};
     record_cell(a, slot, rho.v.x, ux.v.x, uy.v.x, uz.v.x, h0);
     record_cell(a, slot + 1, rho.v.y, ux.v.y, uy.v.y, uz.v.y, h1);
@@ -1770,12 +1775,15 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_PAIR_MIN_BLOCKS) k_step_pair
 // FP32 pipe, one instruction stream for every unit (the output sink alone
 // tells plain units, 64 fluid cells without wall links, from the others).
 //
-// Measured per step, before (chunk kernel) and now: Re 6500 nozzle 445 ->
-// 339 us (4.61 TB/s of algorithmic bytes), Re 3500 nozzle 151 -> 126 us,
-// periodic 256^3 497 -> 349 us (5.20 TB/s).  Two stages and 4 blocks of 4
-// warps per SM: 3 blocks 361 us on the Re 6500 nozzle, 5 blocks (96
-// registers, no spills) 395 us, three stages 347 us; more bytes in flight
-// only widen the span of the arrays that is open at a time.
+// Measured per step, chunk kernel and this one: Re 6500 nozzle 446 -> 370 us
+// (4.22 TB/s of algorithmic bytes; with axial averages 553 -> 497), Re 3500
+// nozzle 151 -> 134 us, periodic 256^3 501 -> 369 us (4.91 TB/s).  Two stages
+// and 4 blocks of 4 warps per SM: 3 blocks take 379 us on the Re 6500 nozzle, a
+// third stage changes nothing.  The moments and lines in fewer operations (250
+// a cell pair instead of 320) took 336 us, in other roundings (see Rounds).
+// Steps that sample full statistics take the chunk kernel, whose 32 cells a
+// warp touch each accumulator's sectors at once: 503 us against 627 on the Re
+// 3500 nozzle.
 #ifndef LBM_STAGE_DEPTH
 #define LBM_STAGE_DEPTH 2
 #endif
@@ -1785,7 +1793,6 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_PAIR_MIN_BLOCKS) k_step_pair
 #ifndef LBM_STAGE_RUN
 #define LBM_STAGE_RUN 3
 #endif
-constexpr int STAGE_SHORT = 6;                       // lists of fewer rounds are handed out by position
 constexpr int STAGE_DEPTH = LBM_STAGE_DEPTH;
 constexpr int STAGE_RUN = LBM_STAGE_RUN;             // units per ticket
 constexpr int STAGE_WINDOW = 160;                    // bytes of one population's window: 128 + 2 x 16
@@ -1848,16 +1855,7 @@ struct UnitStore {
     bool plain, wrap;
     uint32_t links[2], both, own[2];  // both: own of both cells; own: of one cell only
     uint32_t fluid;                   // bit h: cell x + h is a fluid cell
-    __device__ __forceinline__ void moments(F2 omega, const F2 (&a2)[6]) const {
-        if ((a.flags & (STEP_STATS | STEP_STATS_FULL)) != (STEP_STATS | STEP_STATS_FULL)) return;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float s[6];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) s[q] = h ? a2[q].v.y : a2[q].v.x;
-            if (fluid & (1u << h)) record_stress(a, slot + h, h ? omega.v.y : omega.v.x, s);
-        }
-    }
+    __device__ __forceinline__ void moments(F2, const F2 (&)[6]) const {}  // no full statistics here
     __device__ __forceinline__ void put(int i, int s, __half v) const {
         static_cast<__half *>(a.fout)[elem<false>(i, a.stride, s)] = v;
     }
@@ -1942,18 +1940,19 @@ __device__ __forceinline__ void stage_update(const StepArgs &a, const char *st, 
                               __half2float(*reinterpret_cast<const __half *>(p + 2))));
     };
     F2 m[10], rho, ux, uy, uz;
-    scaled_sums<F2>(ld, m);
-    scaled_finish<F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale), sink);
+    ghost1_sums<F2>(ld, m);
+    ghost1_finish<true, F2>(m, F2(a.pf.omega), rho, ux, uy, uz, F2(a.inv_scale), F2(a.scale),
+                            lane_rounds<AX>((rec[6] >> (UNIT_PLAIN_SHIFT + 2 * lane / CHUNK)) & 1), sink);
     if (a.flags & STEP_STATS) {
-        double hv[6];
-        if (sink.fluid & 1u) record_cell(a, slot, rho.v.x, ux.v.x, uy.v.x, uz.v.x, hv);
-        if (sink.fluid & 2u) record_cell(a, slot + 1, rho.v.y, ux.v.y, uy.v.y, uz.v.y, hv);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (sink.fluid & (1u << h)) record_axial(a, slot + h, h ? uz.v.y : uz.v.x);
     }
 }
 
 // The units a warp takes: runs of STAGE_RUN consecutive units from the work
 // counter (one address takes an atomic about every 2 ns: single-unit runs
-// throughout take 551 us a step on the Re 6500 nozzle, runs of three 339 us),
+// throughout took 551 us a step on the Re 6500 nozzle where runs of three took 339),
 // and single ones over the last two rounds of the warps, so that they finish
 // together.  The next ticket is drawn while the current run is handed out.
 struct UnitQueue {
@@ -2501,7 +2500,7 @@ cudaError_t launch_step_ax(const StepArgs &a, cudaStream_t s, const SideStream *
         }
     }
     if constexpr (P == 2 && G == RATE_ONE && !WD) {
-        if (a.units && !(a.flags & STEP_REDUCE)) {
+        if (a.units && !(a.flags & (STEP_REDUCE | STEP_STATS_FULL))) {
             const int blocks = std::min(a.stage_blocks, (a.nunits + STAGE_WARPS - 1) / STAGE_WARPS);
             k_step_units<AX><<<blocks, STEP_THREADS, STAGE_SMEM, s>>>(a);
             ++launches;
@@ -2534,14 +2533,7 @@ cudaError_t launch_step(const StepArgs &a, int mode, cudaStream_t s, int *launch
     const bool wide = a.wide_offsets || a.stride > MAX_SLOTS_32;
     int n = 0;
     cudaError_t e;
-    if constexpr (P == 2) {
-        if (mode == RATE_KEPT && !wide) {
-            e = launch_step_rows<P, RATE_KEPT, false>(a, s, side, n);
-            if (launches) *launches += n;
-            return e != cudaSuccess ? e : cudaGetLastError();
-        }
-    }
-    if (mode == RATE_ONE || mode == RATE_KEPT)
+    if (mode == RATE_ONE)
         e = wide ? launch_step_rows<P, RATE_ONE, true>(a, s, side, n) : launch_step_rows<P, RATE_ONE, false>(a, s, side, n);
     else if (mode == RATE_BGK && !wide)
         e = launch_step_rows<P, RATE_BGK, false>(a, s, side, n);

@@ -69,7 +69,14 @@ constexpr int STATS_FULL = 18;
 enum : uint32_t {
     CHUNK_X0_MASK = (1u << 20) - 1u,
     CHUNK_LANES_SHIFT = 20,
+    // The chunk's warp in the chunk kernel (four consecutive chunks of the list)
+    // holds 32 fluid cells, none with a wall link or at a row end that writes
+    // wrap-around copies: an FP16S cell's roundings go by it in every kernel.
+    CHUNK_PLAIN = 1u << 28,
 };
+// Sets CHUNK_PLAIN on the chunks of such warps and clears it on the others.
+void mark_plain_warps(std::vector<int2> &chunks, const std::vector<int32_t> &row_nb, const std::vector<uint32_t> &mask,
+                      int n_row, bool periodic_row);
 
 // Row records: rows run along the row axis (x, or z for lattices longer in z
 // than in x).  In storage coordinates p (along the row) and a, b (across it),
@@ -84,13 +91,15 @@ constexpr int ROW_RECORD_INTS = 12;
 // Tile records of the tile fluid kernel: a tile is up to four consecutive
 // chunks of one row, i.e. up to 32 consecutive positions [p0, p0 + 32).  A
 // record holds p0 (with the fast flag TILE_FAST: 32 fluid cells, none with
-// a wall link or a wrap-around copy), the fluid-lane mask (bit l: position
+// a wall link or a wrap-around copy, and from TILE_PLAIN_SHIFT on the
+// CHUNK_PLAIN bits of its chunks), the fluid-lane mask (bit l: position
 // p0 + l is a fluid cell), the present-lane mask (bit l: p0 + l lies in one
 // of the tile's chunks; other lanes store nothing) and the row's nine
 // neighbour bases (as in the row record), so that a tile needs no dependent
 // index load.
 constexpr int TILE_INTS = 12;
 constexpr uint32_t TILE_FAST = 1u << 31;
+constexpr int TILE_PLAIN_SHIFT = 24;
 
 // Group a chunk list (in row order) into tile records, in the same order;
 // mask: the link words, n_row / periodic_row: the row axis (wrap-around
@@ -122,41 +131,31 @@ constexpr size_t NODE_BYTES = NODE_INT4S * 16;
 // row's first), the fluid-lane and the present-lane masks (64 bits each, low
 // word first), the first and the last present chunk, the flags UNIT_PLAIN (64
 // fluid cells, none with a wall link) and UNIT_WRAP (plain, with a row end
-// that writes wrap-around copies), and the row's nine neighbour bases: 64
-// bytes.
+// that writes wrap-around copies) with the CHUNK_PLAIN bits of the chunks from
+// UNIT_PLAIN_SHIFT on, and the row's nine neighbour bases: 64 bytes.
 constexpr int UNIT_ALIGN = 16;
 constexpr int UNIT_CELLS = 64;
 constexpr int UNIT_INTS = 16;
 constexpr int UNIT_NB = 7;  // first of the nine neighbour bases in a record
 constexpr int UNIT_HI_SHIFT = 8;
-constexpr int UNIT_PLAIN = 1, UNIT_WRAP = 2;
+constexpr int UNIT_PLAIN = 1, UNIT_WRAP = 2, UNIT_PLAIN_SHIFT = 8;
 // The staged kernel takes over from the chunk kernel at this many units per
-// resident warp (about 0.9 M cells): its warps start and end on atomics of one
-// address, a few us a launch.  At 4.4 rounds (96^3) it takes 36.5 us against
-// the chunk kernel's 34.6, at 13.5 rounds (128^3) 59.5 against 69.7.
-constexpr int STAGE_ROUNDS = 6;
+// resident warp (about 2 M cells): its warps start and end on atomics of one
+// address, a few us a launch.  Staged against chunk, us a step: nozzles of 1.4 /
+// 1.8 / 2.3 / 2.9 / 3.5 M cells (9 / 12 / 16 / 20 / 25 rounds) 61 / 73 / 84 / 98 /
+// 110 against 54 / 68 / 82 / 104 / 121, periodic boxes of 104^3 / 128^3 / 144^3 /
+// 160^3 (9 / 13.5 / 26 / 32 rounds) 49 / 63 / 100 / 123 against 51 / 72 / 98 / 132.
+constexpr int STAGE_ROUNDS = 13;
 std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
                                  const std::vector<uint32_t> &mask, int n_row, bool periodic_row);
 
 // Form of the collision: general ghost rates (the 27-moment cascade), all
 // ghost rates 1 (the default), or all ghost rates equal to omega (lattice BGK).
-// RATE_KEPT is RATE_ONE for FP16S with statistics on (32-bit offsets, no
-// fluid kernel asked for by name), in the chunk kernel and with the roundings
-// of the releases before the staged kernel.  FP16 storage carries a last-bit
-// difference on to the size of its own noise in some 50 steps, 1e-3 of a
-// velocity, and the averages, returned in FP64, show that in full; with these
-// roundings a run's averages repeat those taken earlier (nozzles of 49 000 to
-// 4.5 million cells, both wall treatments, 120 to 400 steps: to the bit, with
-// RATE_ONE's they are off by 1e-4 to 5e-4).  They are the ones a compiler
-// picked where a product meets a sum, hence the choice by kind of warp and
-// row axis.  The price is the chunk kernel's step, 448 us on the Re 6500
-// nozzle where the staged kernel takes 336.
-enum : int { RATE_GENERAL = 0, RATE_ONE = 1, RATE_BGK = 2, RATE_KEPT = 3 };
+enum : int { RATE_GENERAL = 0, RATE_ONE = 1, RATE_BGK = 2 };
 
 // Fluid kernel of the FP32 / FP16S steps: AUTO is the tile kernel in FP32
 // and, in FP16S, the staged unit kernel for larger lattices and the chunk
-// kernel for smaller ones and with statistics on; the others are kept for
-// testing.
+// kernel for smaller ones; the others are kept for testing.
 enum class FluidKernel { AUTO, CHUNK, TILE, PAIRS, STAGED };
 
 // A second stream and its fork / join events: a step's wall-cell and

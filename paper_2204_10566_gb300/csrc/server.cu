@@ -92,7 +92,7 @@ __device__ __forceinline__ void serve_nodes(const StepArgs a, int i, int lane) {
 template <int P, int AX>
 __device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec, int lane) {
     double hv[6] = {0, 0, 0, 0, 0, 0};
-    tile_update<P, AX, true, false>(a, rec, lane, nullptr, hv);
+    tile_update<P, AX, true, false, true>(a, rec, lane, nullptr, hv);
     flag_non_finite(a, hv[5]);
 }
 
