@@ -56,7 +56,7 @@ typedef enum {
     LBM_ERR_CUDA = 3,     /* a CUDA runtime call failed */
     LBM_ERR_STATE = 4,    /* call out of order (e.g. lbm_step before lbm_set_geometry) */
     LBM_ERR_UNSTABLE = 5, /* a health check found non-finite populations */
-    LBM_ERR_TIMEOUT = 6   /* a bounded device-side wait gave up */
+    LBM_ERR_TIMEOUT = 6   /* a bounded device-side wait gave up: the state is lost (set it anew; lbm_step) */
 } lbm_status;
 
 typedef enum {
@@ -267,11 +267,18 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int32_t layout);
  * stream beside it; they read the same input and write disjoint outputs, so
  * their order changes no result.  The health check and the statistics
  * sampling ride on these kernels when due.
- * Errors: LBM_ERR_STATE (no geometry / params / init), LBM_ERR_CUDA. */
+ * Runs of steps that go in one launch (see lbm_kernel_launches) wait at a
+ * barrier over the device between steps, for some seconds at most.  If a wait
+ * gives up, the state is lost: lbm_sync, the next call that reads the state or
+ * the averages back, and every later one that needs the state return
+ * LBM_ERR_TIMEOUT until it is set anew (lbm_init_*, lbm_set_populations,
+ * lbm_restore, lbm_set_geometry).
+ * Errors: LBM_ERR_STATE (no geometry / params / init), LBM_ERR_CUDA,
+ * LBM_ERR_TIMEOUT. */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t n);
 
 /* Wait for the stream; report a deferred LBM_ERR_UNSTABLE (a health check saw
- * a non-finite value) or LBM_ERR_CUDA.  The unstable flag stays set until the
+ * a non-finite value), LBM_ERR_TIMEOUT or LBM_ERR_CUDA.  The unstable flag stays set until the
  * next init call. */
 lbm_status lbm_sync(lbm_ctx *ctx);
 
@@ -457,7 +464,9 @@ lbm_status lbm_server_check_request(const lbm_request *req, int64_t budget_bytes
  * in a tick is its health check: a lattice with a non-finite density or
  * velocity is evicted (its memory freed) and ends FAILED with
  * LBM_ERR_UNSTABLE; the others are not affected.  Blocks until the tick's
- * work is done.  Outputs (may be NULL): resident lattices, queued requests. */
+ * work is done.  If a device-side wait of the tick gives up, every lattice in
+ * it ends FAILED with LBM_ERR_TIMEOUT, which the call returns too; queued
+ * requests are not affected.  Outputs (may be NULL): resident lattices, queued requests. */
 lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued);
 
 /* State (LBM_REQ_*) and steps done of a request. */

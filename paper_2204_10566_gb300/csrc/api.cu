@@ -53,6 +53,11 @@ struct lbm_ctx {
     int32_t *d_units_wall = nullptr; // the same without the cells with interpolated walls
     int64_t n_units_wall = 0;
     int stage_blocks = 0;            // grid of the staged kernel
+    int polls = 0;                   // of its barrier waits
+    uint32_t *h_status = nullptr;    // the host's copy of the status word, page-locked (see queue_status)
+    uint32_t status_word = 0;        // or, without page-locked memory, here
+    bool run_unread = false;         // a several-step launch whose status the host has not seen
+    bool torn = false;               // one gave up: the state is partly a step ahead
     int run_blocks = 0, run_mode = -1;  // largest grid of the several-step kernel, and for which collision form
     double *d_partials = nullptr;
     double *d_health = nullptr;
@@ -216,11 +221,19 @@ void for_active(const lbm_ctx *c, int32_t layout, F fn) {  // fn(active k, host 
     for (int64_t k = 0; k < c->idx.n_active; ++k) fn(k, layout == LBM_LAYOUT_BOX ? c->idx.box_of_active[k] : k);
 }
 
+// A several-step launch that gave up at its barrier leaves some cells a step
+// ahead of others.  The state cannot be used until it is set anew; every call
+// that would read or advance it says so.
+lbm_status torn(lbm_ctx *c) {
+    return fail(c, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (several-step kernel): set the state anew");
+}
+
 lbm_status need(lbm_ctx *c, bool geom, bool params, bool state) {
     if (!c) return LBM_ERR_ARG;
     if (geom && !c->has_geom) return fail(c, LBM_ERR_STATE, "no geometry: call lbm_set_geometry first");
     if (params && !c->has_params) return fail(c, LBM_ERR_STATE, "no parameters: call lbm_set_params first");
     if (state && !c->has_state) return fail(c, LBM_ERR_STATE, "no state: call an init function first");
+    if (state && c->torn) return torn(c);
     c->err.clear();
     return LBM_OK;
 }
@@ -370,6 +383,23 @@ cudaError_t in_parts(lbm_ctx *c, int64_t n, cudaStream_t first_on, cudaStream_t 
     return e != cudaSuccess ? e : (e1 != cudaSuccess ? e1 : e2);
 }
 
+// Status of the several-step launches so far, for a call that reads the state
+// back: queue_status before its own work on c->stream, settle once the stream
+// is idle.  No cost when the last look was after the last such launch.
+cudaError_t queue_status(lbm_ctx *c) {
+    if (!c->run_unread) return cudaSuccess;
+    if (!c->h_status && cudaMallocHost(&c->h_status, sizeof *c->h_status) != cudaSuccess) {
+        c->h_status = nullptr;
+        cudaGetLastError();
+    }
+    return cudaMemcpyAsync(c->h_status ? c->h_status : &c->status_word, c->d_status, 4, cudaMemcpyDeviceToHost, c->stream);
+}
+lbm_status settle(lbm_ctx *c) {
+    if (c->run_unread && ((c->h_status ? *c->h_status : c->status_word) & 2u)) c->torn = true;
+    c->run_unread = false;
+    return c->torn ? torn(c) : LBM_OK;
+}
+
 // Grid of the several-step kernel for the next n steps, 0 when they run one
 // by one: FP64 (bound by its arithmetic, not by launches), 64-bit offsets, a
 // fluid kernel asked for by name, a stream that is being captured (one
@@ -406,6 +436,7 @@ lbm_status reset_state(lbm_ctx *c) {
     c->t = 0;
     c->stats_samples = 0;
     c->stats_on = false;
+    c->run_unread = c->torn = false;
     CK(cudaMemsetAsync(c->d_status, 0, 4, c->stream), "reset status");
     if (c->d_stats) CK(cudaMemsetAsync(c->d_stats, 0, stats_bytes(c), c->stream), "reset stats");
     c->has_state = true;
@@ -580,6 +611,7 @@ lbm_status lbm_create(const lbm_desc *desc, lbm_ctx **out) {
     // without allocating tens of gigabytes.
     const char *wide = std::getenv("LBM_WIDE_OFFSETS");
     c->wide_offsets = wide && wide[0] == '1';
+    c->polls = barrier_polls();
     // LBM_FLUID_KERNEL selects another fluid kernel than the default (FP32:
     // tile kernel, FP16S: staged or chunk kernel by size, FP64: chunk kernel),
     // for testing every variant on the same lattices: "chunk", "tile", "pairs"
@@ -624,6 +656,7 @@ lbm_status lbm_destroy(lbm_ctx *c) {
     }
     if (c->side.fork) cudaEventDestroy(c->side.fork);
     if (c->side.join) cudaEventDestroy(c->side.join);
+    if (c->h_status) cudaFreeHost(c->h_status);
     delete c;
     return LBM_OK;
 }
@@ -790,6 +823,7 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->fluid_blocks = DISPATCH(c->desc.precision, step_fluid_blocks, (int32_t)c->idx.chunks.size());
     c->nblocks = partial_capacity(c, 0);
     c->run_mode = -1;
+    c->run_unread = c->torn = false;
     c->stage_blocks = DISPATCH(c->desc.precision, step_stage_blocks, c->desc.device);
     for (int k = 0; k < 2; ++k) {
         c->f_raw[k] = dev_alloc(c, raw_pop_bytes(c));
@@ -1061,8 +1095,10 @@ lbm_status lbm_get_populations(lbm_ctx *c, double *f, int32_t layout) {
     const size_t bytes = (size_t)n * 27 * 8;
     double *d = (double *)dev_alloc(c, bytes);
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-    cudaError_t e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_act, c->idx.nslots,
-                             1.0f / fp16_scale(c), d, c->stream);
+    cudaError_t e = queue_status(c);
+    if (e == cudaSuccess)
+        e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_act, c->idx.nslots,
+                     1.0f / fp16_scale(c), d, c->stream);
     if (layout == LBM_LAYOUT_ACTIVE) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, bytes, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1070,14 +1106,14 @@ lbm_status lbm_get_populations(lbm_ctx *c, double *f, int32_t layout) {
         std::vector<double> h((size_t)n * 27);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, bytes, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e == cudaSuccess) {
+        if (e == cudaSuccess && (st = settle(c)) == LBM_OK) {
             memset(f, 0, (size_t)layout_count(c, layout) * 27 * 8);
             for_active(c, layout, [&](int64_t k, int64_t r) { memcpy(f + 27 * r, &h[27 * (size_t)k], 27 * 8); });
         }
     }
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "get populations");
-    return LBM_OK;
+    return settle(c);
 }
 
 lbm_status lbm_step(lbm_ctx *c, int64_t n) {
@@ -1102,9 +1138,11 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
             r.t_new = t_new;
             r.tiles = c->d_tiles_wall ? c->d_tiles_wall : c->d_tiles;  // whatever the per-step kernel takes
             r.ntiles = (int32_t)tile_count(c);
-            RunArgs run{m, 0, c->stats_start, c->stats_stride, reinterpret_cast<int32_t *>(c->d_status) + BARRIER_WORD};
+            RunArgs run{m, 0, c->stats_start, c->stats_stride, reinterpret_cast<int32_t *>(c->d_status) + BARRIER_WORD,
+                        c->polls};
             if (c->stats_on) run.stats_flags = STEP_STATS | (c->stats_ncomp == STATS_FULL ? STEP_STATS_FULL : 0);
             CK(DISPATCH(c->desc.precision, launch_run, r, run, c->mode, run_grid, c->stream), "steps kernel");
+            c->run_unread = true;
             ++c->kernel_launches;
             if (c->stats_on) {  // sampled steps among t_new .. t_new + m - 1
                 const int64_t lo = std::max(t_new, c->stats_start) - c->stats_start, hi = t_new + m - 1 - c->stats_start;
@@ -1151,7 +1189,9 @@ lbm_status lbm_sync(lbm_ctx *c) {
         CK(cudaMemcpyAsync(c->health, c->d_health, 6 * 8, cudaMemcpyDeviceToHost, c->stream), "read health");
         CK(cudaStreamSynchronize(c->stream), "sync health");
     }
-    if (status & 2u) return fail(c, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (step kernel)");
+    c->run_unread = false;
+    if (status & 2u) c->torn = true;
+    if (c->torn) return torn(c);
     if (status & 1u) return fail(c, LBM_ERR_UNSTABLE, "a health check found non-finite populations");
     return LBM_OK;
 }
@@ -1186,7 +1226,8 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
         hr = h.data();
         hu = h.data() + n;
     }
-    const cudaError_t e = in_parts(
+    const cudaError_t queued = queue_status(c);
+    const cudaError_t e = queued != cudaSuccess ? queued : in_parts(
         c, n, c->stream, c->side.stream,
         [&](int64_t k0, int64_t k1, cudaStream_t s) {
             return DISPATCH(c->desc.precision, launch_moments, c->f[c->cur], c->d_act, k0, k1, c->idx.nslots,
@@ -1201,6 +1242,8 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
         });
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "get moments");
+    st = settle(c);
+    if (st) return st;
     if (layout == LBM_LAYOUT_ACTIVE) return LBM_OK;
     const int64_t total = layout_count(c, layout);
     if (rho) memset(rho, 0, (size_t)total * 8);
@@ -1218,12 +1261,15 @@ lbm_status lbm_get_totals(lbm_ctx *c, double *mass, double mom[3]) {
     lbm_status st = need(c, true, false, true);
     if (st) return st;
     DeviceGuard g(c->desc.device);
+    CK(queue_status(c), "read status");
     CK(DISPATCH(c->desc.precision, launch_reduce, c->f[c->cur], c->d_act, c->idx.nslots, 1.0f / fp16_scale(c),
                 c->d_partials, c->stream),
        "reduce");
     CK(launch_finalize(c->d_partials, reduce_blocks(c->idx.nslots), c->d_health, c->d_status, c->stream), "finalize");
     CK(cudaMemcpyAsync(c->health, c->d_health, 6 * 8, cudaMemcpyDeviceToHost, c->stream), "read totals");
     CK(cudaStreamSynchronize(c->stream), "sync totals");
+    st = settle(c);
+    if (st) return st;
     if (mass) *mass = c->health[0];
     if (mom)
         for (int a = 0; a < 3; ++a) mom[a] = c->health[1 + a];
@@ -1295,6 +1341,7 @@ lbm_status lbm_stats_get(lbm_ctx *c, double *mean_uz, double *mean_uzuz, int64_t
     if (layout != LBM_LAYOUT_ACTIVE && layout != LBM_LAYOUT_BOX) return fail(c, LBM_ERR_ARG, "bad layout");
     if (n_samples) *n_samples = c->stats_samples;
     if (!mean_uz && !mean_uzuz) return LBM_OK;
+    if (c->torn) return torn(c);
     const int64_t n = c->idx.n_active;
     const size_t total = (size_t)layout_count(c, layout) * 8, bytes = (size_t)n * 2 * 8;
     double *out[2] = {mean_uz, mean_uzuz};
@@ -1306,20 +1353,23 @@ lbm_status lbm_stats_get(lbm_ctx *c, double *mean_uz, double *mean_uzuz, int64_t
     double *d = (double *)dev_alloc(c, bytes);  // <u_z>[n], then <u_z^2>[n]
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n : 0);
-    cudaError_t e = launch_stats_mean(c->d_stats, STATS_AXIAL, c->d_act, c->idx.nslots, 1.0 / (double)c->stats_samples,
-                                      d, d + n, c->stream);
+    cudaError_t e = queue_status(c);
+    if (e == cudaSuccess)
+        e = launch_stats_mean(c->d_stats, STATS_AXIAL, c->d_act, c->idx.nslots, 1.0 / (double)c->stats_samples, d, d + n,
+                              c->stream);
     for (int q = 0; q < 2; ++q) {
         if (e != cudaSuccess || !out[q]) continue;
         double *to = layout == LBM_LAYOUT_BOX ? h.data() : out[q];  // the active order goes straight to the caller
         if (layout == LBM_LAYOUT_ACTIVE) fault_in(to, total);
         e = cudaMemcpyAsync(to, d + q * n, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e == cudaSuccess && (st = settle(c)) != LBM_OK) break;
         if (e == cudaSuccess && layout == LBM_LAYOUT_BOX)
             for_active(c, layout, [&](int64_t k, int64_t r) { out[q][r] = h[(size_t)k]; });
     }
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
-    return LBM_OK;
+    return st;
 }
 
 lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int32_t layout) {
@@ -1328,6 +1378,7 @@ lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int3
     if (layout != LBM_LAYOUT_ACTIVE && layout != LBM_LAYOUT_BOX) return fail(c, LBM_ERR_ARG, "bad layout");
     if (n_samples) *n_samples = c->stats_samples;
     if (!mean) return LBM_OK;
+    if (c->torn) return torn(c);
     if (c->stats_ncomp != STATS_FULL && c->stats_samples > 0)
         return fail(c, LBM_ERR_STATE, "the accumulators hold axial statistics only");
     constexpr int Q = LBM_STATS_FULL_COMPONENTS;  // the rows after the axial ones
@@ -1341,13 +1392,17 @@ lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int3
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n * Q : 0);
     double *to = layout == LBM_LAYOUT_BOX ? h.data() : mean;
-    cudaError_t e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act,
-                                      c->idx.nslots, 1.0 / (double)c->stats_samples, d, nullptr, c->stream);
+    cudaError_t e = queue_status(c);
+    if (e == cudaSuccess)
+        e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act, c->idx.nslots,
+                              1.0 / (double)c->stats_samples, d, nullptr, c->stream);
     if (layout == LBM_LAYOUT_ACTIVE) fault_in(to, bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(to, d, bytes, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
+    st = settle(c);
+    if (st) return st;
     if (layout == LBM_LAYOUT_BOX)
         for_active(c, layout, [&](int64_t k, int64_t r) { memcpy(mean + r * Q, &h[(size_t)k * Q], Q * 8); });
     return LBM_OK;
@@ -1401,12 +1456,13 @@ lbm_status lbm_checkpoint(lbm_ctx *c, void *buf, size_t bytes) {
     char *p = static_cast<char *>(buf);
     memcpy(p, &h, sizeof h);
     p += sizeof h;
+    CK(queue_status(c), "read status");
     CK(cudaMemcpyAsync(p, c->f[c->cur], pop_bytes(c), cudaMemcpyDeviceToHost, c->stream), "checkpoint f");
     p += pop_bytes(c);
     if (c->d_stats)
         CK(cudaMemcpyAsync(p, c->d_stats, stats_bytes(c), cudaMemcpyDeviceToHost, c->stream), "checkpoint stats");
     CK(cudaStreamSynchronize(c->stream), "sync checkpoint");
-    return LBM_OK;
+    return settle(c);
 }
 
 lbm_status lbm_restore(lbm_ctx *c, const void *buf, size_t bytes) {
@@ -1436,6 +1492,7 @@ lbm_status lbm_restore(lbm_ctx *c, const void *buf, size_t bytes) {
         if (st) return st;
         CK(cudaMemcpyAsync(c->d_stats, p, stats_bytes(c), cudaMemcpyHostToDevice, c->stream), "restore stats");
     }
+    c->run_unread = c->torn = false;
     CK(cudaMemsetAsync(c->d_status, 0, 4, c->stream), "reset status");
     CK(cudaStreamSynchronize(c->stream), "sync restore");
     c->t = h.t;

@@ -1,10 +1,16 @@
 // Precision-independent kernels: the fixed-order final pass of the FP64
 // health reduction and the time-average readback.
 #include <algorithm>
+#include <cstdlib>
 
 #include "lbm_internal.h"
 
 namespace lbm {
+
+int barrier_polls() {
+    const char *s = std::getenv("LBM_BARRIER_POLLS");
+    return s ? std::max(0, std::atoi(s)) : 1 << 22;
+}
 
 int fluid_blocks(int32_t nchunks) {
     const int64_t threads = (int64_t)nchunks * CHUNK;

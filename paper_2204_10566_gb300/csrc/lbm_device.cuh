@@ -2051,17 +2051,17 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STAGE_BLOCKS) k_step_units(c
 #define LBM_RUN_BLOCKS 4
 #endif
 
-// Wait until all blocks have arrived `rounds` times at the barrier word, at
-// most a few seconds: then bit 1 of the status word tells the host, and every
-// block leaves.  The result is uniform over the block.
-__device__ __forceinline__ bool grid_barrier(int32_t *word, int rounds, uint32_t *status) {
+// Wait until all blocks have arrived `rounds` times at the barrier word, for
+// at most `polls` looks (some seconds): then bit 1 of the status word tells the
+// host, and every block leaves.  The result is uniform over the block.
+__device__ __forceinline__ bool grid_barrier(int32_t *word, int rounds, uint32_t *status, int polls) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         const int target = rounds * (int)gridDim.x;
         int seen = 0;
         asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(word) : "memory");
-        for (int k = 0; k < RUN_SPIN_LIMIT; ++k) {
+        for (int k = 0; k < polls; ++k) {
             asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(word) : "memory");
             if (seen >= target || (*(volatile uint32_t *)status & 2u)) break;
         }
@@ -2111,7 +2111,7 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_RUN_BLOCKS) k_run(const Step
                 if (chunk < a.nchunks) fluid_cell<P, G, false, AX, true>(a, chunk, lane % CHUNK, hv);
             }
         }
-        if (s + 1 < run.steps && !grid_barrier(run.barrier, s + 1, a.status)) break;
+        if (s + 1 < run.steps && !grid_barrier(run.barrier, s + 1, a.status, run.polls)) break;
     }
     // the last block to leave clears the words for the next launch
     __syncthreads();

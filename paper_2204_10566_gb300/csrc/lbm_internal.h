@@ -184,7 +184,7 @@ struct alignas(16) StepArgs {
     const int4 *bnodes;     // [nbnodes][NODE_INT4S] inlet/outlet node records
     int32_t nbnodes;
     int32_t fluid_blocks;   // blocks of the fluid kernel (offset of the boundary kernel's partials)
-    uint32_t *status;       // bit 1: a bounded device wait gave up
+    uint32_t *status;       // bit 1: a bounded device wait gave up (the state is torn)
     int32_t nx, ny, nz;     // box (physical x, y, z)
     int32_t n_row;          // cells along the row axis
     int32_t row_axis;       // 0: rows along x, 2: rows along z
@@ -224,9 +224,11 @@ struct RunArgs {
     int32_t stats_flags;  // STEP_STATS (| STEP_STATS_FULL), or 0
     int64_t stats_start, stats_stride;
     int32_t *barrier;
+    int32_t polls;        // of a barrier wait before it gives up
 };
-// Polls of a barrier wait before it gives up (some seconds).
-constexpr int RUN_SPIN_LIMIT = 1 << 22;
+// Polls of a barrier wait before it gives up: some seconds, or the value of
+// LBM_BARRIER_POLLS (0: every wait gives up at once, for tests).
+int barrier_polls();
 
 // Launchers, one set per storage precision (P = 0 FP64, 1 FP32, 2 FP16S).
 // Offsets into a population buffer fit in 32 bits (unsigned) when

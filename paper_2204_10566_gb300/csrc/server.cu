@@ -122,7 +122,7 @@ __device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec,
 #define LBM_SERVE_BLOCKS 5
 #endif
 __global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const TickTable *tab, int32_t *barrier,
-                                                                        uint32_t *status) {
+                                                                        uint32_t *status, int polls) {
     extern __shared__ __align__(16) char serve_smem[];
     DomainEntry *dom = reinterpret_cast<DomainEntry *>(serve_smem);
     const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const 
             }
             if (k < e.steps) SERVE_DISPATCH(e, serve_tile, rec, lane);
         }
-        if (k + 1 < steps && !grid_barrier(barrier, k + 1, status)) break;
+        if (k + 1 < steps && !grid_barrier(barrier, k + 1, status, polls)) break;
     }
     // the last block to leave clears the words for the next tick
     __syncthreads();
@@ -229,7 +229,7 @@ struct lbm_server {
     // and the kernel's barrier words
     uint32_t *d_flags = nullptr, *h_flags = nullptr;
     cudaGraphExec_t exec = nullptr;
-    int grid = 0, smem = 0;  // of the tick's kernel
+    int grid = 0, smem = 0, polls = 0;  // of the tick's kernel
 };
 
 namespace {
@@ -335,7 +335,7 @@ lbm_status capture_tick(lbm_server *s) {
     const TickTable *tab = s->d_tab;
     int32_t *barrier = reinterpret_cast<int32_t *>(s->d_flags) + BARRIER_WORDS;
     uint32_t *status = s->d_flags + STATUS_WORD;
-    void *params[3] = {&tab, &barrier, &status};
+    void *params[4] = {&tab, &barrier, &status, &s->polls};
     const cudaError_t launch = cudaLaunchCooperativeKernel((const void *)k_serve, dim3((unsigned)s->grid),
                                                            dim3(STEP_THREADS), params, (size_t)s->smem, s->stream);
     cudaMemcpyAsync(s->h_flags, s->d_flags, (STATUS_WORD + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream);
@@ -418,6 +418,7 @@ lbm_status lbm_server_create(const lbm_server_desc *desc, lbm_server **out) {
     if (desc->device < 0 || desc->device >= ndev) return LBM_ERR_ARG;
     std::unique_ptr<lbm_server> s(new lbm_server());
     s->desc = *desc;
+    s->polls = barrier_polls();
     cudaSetDevice(desc->device);
     // on a failure below, free what was made so far (no worker runs yet)
     auto undo = [&](lbm_status st) {
@@ -606,7 +607,18 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     }
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("tick: ") + cudaGetErrorString(e));
-    if (s->h_flags[STATUS_WORD] & 2u) return sfail(s, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (tick kernel)");
+    if (s->h_flags[STATUS_WORD] & 2u) {  // torn lattices: no request that took part can go on
+        for (const int64_t id : s->resident) {
+            Request *r = s->reqs[id].get();
+            r->state = LBM_REQ_FAILED;
+            r->fail_status = LBM_ERR_TIMEOUT;
+            r->index_error = "a bounded device-side wait gave up in a tick";
+            release(s, r);
+        }
+        s->resident.clear();
+        if (running) *running = 0;
+        return sfail(s, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (tick kernel): its requests failed");
+    }
     s->graph_launches += 1;
     s->ticks += 1;
     // account, retire finished lattices
