@@ -58,6 +58,7 @@ struct lbm_ctx {
     uint32_t status_word = 0;        // or, without page-locked memory, here
     bool run_unread = false;         // a several-step launch whose status the host has not seen
     bool torn = false;               // one gave up: the state is partly a step ahead
+    bool run_refused = false;        // the device would not take it: steps run one by one
     int run_blocks = 0, run_mode = -1;  // largest grid of the several-step kernel, and for which collision form
     double *d_partials = nullptr;
     double *d_health = nullptr;
@@ -403,9 +404,10 @@ lbm_status settle(lbm_ctx *c) {
 // Grid of the several-step kernel for the next n steps, 0 when they run one
 // by one: FP64 (bound by its arithmetic, not by launches), 64-bit offsets, a
 // fluid kernel asked for by name, a stream that is being captured (one
-// recorded step is then the same kernels as ever), or a larger lattice.
+// recorded step is then the same kernels as ever), a launch that was refused
+// before, or a larger lattice.
 int run_blocks(lbm_ctx *c, int64_t n) {
-    if (n < RUN_MIN_STEPS || c->desc.precision == LBM_FP64 || wide_offsets(c) || c->fluid_kernel != FluidKernel::AUTO)
+    if (n < RUN_MIN_STEPS || c->run_refused || c->desc.precision == LBM_FP64 || wide_offsets(c) || c->fluid_kernel != FluidKernel::AUTO)
         return 0;
     if (c->run_mode != c->mode) {
         c->run_blocks = DISPATCH(c->desc.precision, step_run_blocks, c->mode, c->idx.row_axis, c->desc.device);
@@ -421,7 +423,7 @@ int run_blocks(lbm_ctx *c, int64_t n) {
         return 0;
     }
     if (cs != cudaStreamCaptureStatusNone) return 0;
-    return (int)std::min<int64_t>(c->run_blocks, (items + warps - 1) / warps);
+    return cooperative_blocks((int)std::min<int64_t>(c->run_blocks, (items + warps - 1) / warps));
 }
 
 // Ghost slots and periodic copies of the current buffer from its active cells.
@@ -1124,7 +1126,7 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
     DeviceGuard g(c->desc.device);
     StepArgs a{};
     lbm::ctx_step_args(c, &a);
-    const int run_grid = run_blocks(c, n);
+    int run_grid = run_blocks(c, n);
     for (int64_t k = 0; k < n; ++k) {
         const int64_t t_new = c->t + 1;
         // steps up to the next health check in one launch
@@ -1141,7 +1143,15 @@ lbm_status lbm_step(lbm_ctx *c, int64_t n) {
             RunArgs run{m, 0, c->stats_start, c->stats_stride, reinterpret_cast<int32_t *>(c->d_status) + BARRIER_WORD,
                         c->polls};
             if (c->stats_on) run.stats_flags = STEP_STATS | (c->stats_ncomp == STATS_FULL ? STEP_STATS_FULL : 0);
-            CK(DISPATCH(c->desc.precision, launch_run, r, run, c->mode, run_grid, c->stream), "steps kernel");
+            const cudaError_t e = DISPATCH(c->desc.precision, launch_run, r, run, c->mode, run_grid, c->stream);
+            if (launch_refused(e)) {
+                cudaGetLastError();
+                c->run_refused = true;
+                run_grid = 0;
+                --k;  // the same step again
+                continue;
+            }
+            CK(e, "steps kernel");
             c->run_unread = true;
             ++c->kernel_launches;
             if (c->stats_on) {  // sampled steps among t_new .. t_new + m - 1

@@ -12,6 +12,15 @@ int barrier_polls() {
     return s ? std::max(0, std::atoi(s)) : 1 << 22;
 }
 
+int cooperative_blocks(int blocks) {
+    const char *s = std::getenv("LBM_COOPERATIVE_BLOCKS");
+    return s && blocks > 0 ? std::max(1, std::atoi(s)) : blocks;
+}
+
+bool launch_refused(cudaError_t e) {
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources;
+}
+
 int fluid_blocks(int32_t nchunks) {
     const int64_t threads = (int64_t)nchunks * CHUNK;
     return (int)((threads + STEP_THREADS - 1) / STEP_THREADS);

@@ -229,6 +229,13 @@ struct RunArgs {
 // Polls of a barrier wait before it gives up: some seconds, or the value of
 // LBM_BARRIER_POLLS (0: every wait gives up at once, for tests).
 int barrier_polls();
+// Blocks of a cooperative launch: as computed, or LBM_COOPERATIVE_BLOCKS (a
+// number the device cannot hold at once gets the launch refused, for tests).
+int cooperative_blocks(int blocks);
+// Whether a cooperative launch failed because the device does not hold its
+// blocks at once (fewer multiprocessors for the process than the device has,
+// for one): its steps then run one by one.
+bool launch_refused(cudaError_t e);
 
 // Launchers, one set per storage precision (P = 0 FP64, 1 FP32, 2 FP16S).
 // Offsets into a population buffer fit in 32 bits (unsigned) when

@@ -12,7 +12,8 @@
 // a per-tick table that the graph copies to the device first.  The table
 // changes every tick, the graph never does.  Each cell is updated by the same
 // device code as lbm_step, so a lattice's result does not depend on what else
-// is resident.
+// is resident.  A device that refuses the cooperative launch takes the steps in
+// a launch each.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -108,7 +109,9 @@ __device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec,
         }                                                                                  \
     } while (0)
 
-// All steps of a tick.  Before, a step was four launches in turn (fluid and
+// Steps k0 .. k0 + count - 1 of a tick, as far as its lattices go: all of them
+// in one cooperative launch, or one (no barrier then) in an ordinary launch.
+// Before, a step was four launches in turn (fluid and
 // nodes of each precision) whose blocks copied a lattice's arguments to
 // shared memory for every 128 cells; here the table stays in shared memory,
 // and a warp looks up the lattice and the record of its next tile while it
@@ -121,20 +124,20 @@ __device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec,
 #ifndef LBM_SERVE_BLOCKS
 #define LBM_SERVE_BLOCKS 5
 #endif
-__global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const TickTable *tab, int32_t *barrier,
-                                                                        uint32_t *status, int polls) {
+__global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const TickTable *tab, int k0, int count,
+                                                                        int32_t *barrier, uint32_t *status, int polls) {
     extern __shared__ __align__(16) char serve_smem[];
     DomainEntry *dom = reinterpret_cast<DomainEntry *>(serve_smem);
     const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
-    const int n = tab->n_domains, tiles = tab->n_tiles, nodes = tab->n_nodes, steps = tab->steps;
+    const int n = tab->n_domains, tiles = tab->n_tiles, nodes = tab->n_nodes, end = min(k0 + count, tab->steps);
     for (int w = threadIdx.x; w < n * (int)(sizeof(DomainEntry) / 16); w += STEP_THREADS)
         reinterpret_cast<int4 *>(dom)[w] = reinterpret_cast<const int4 *>(tab->d)[w];
     const int first = warp * (int)gridDim.x + (int)blockIdx.x, stride = (int)gridDim.x * (STEP_THREADS / 32);
-    for (int k = 0; k < steps; ++k) {
+    for (int k = k0; k < end; ++k) {
         __syncthreads();
         if ((int)threadIdx.x < n) {  // the step's buffers, number and check flag
             DomainEntry &e = dom[threadIdx.x];
-            if (k > 0) {
+            if (k > k0 || (k0 & 1)) {
                 const void *t = e.a.fin;
                 e.a.fin = e.a.fout;
                 e.a.fout = const_cast<void *>(t);
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_SERVE_BLOCKS) k_serve(const 
             }
             if (k < e.steps) SERVE_DISPATCH(e, serve_tile, rec, lane);
         }
-        if (k + 1 < steps && !grid_barrier(barrier, k + 1, status, polls)) break;
+        if (k + 1 < end && !grid_barrier(barrier, k - k0 + 1, status, polls)) break;
     }
     // the last block to leave clears the words for the next tick
     __syncthreads();
@@ -229,7 +232,8 @@ struct lbm_server {
     // and the kernel's barrier words
     uint32_t *d_flags = nullptr, *h_flags = nullptr;
     cudaGraphExec_t exec = nullptr;
-    int grid = 0, smem = 0, polls = 0;  // of the tick's kernel
+    int grid = 0, resident_blocks = 0, smem = 0, polls = 0;  // of the tick's kernel
+    bool together = false;              // all steps in one cooperative launch; else a launch each
 };
 
 namespace {
@@ -311,7 +315,7 @@ void worker_loop(lbm_server *s) {
     }
 }
 
-// Grid and shared memory of the tick's kernel: every block resident at once.
+// Grid and shared memory of the tick's kernel: the blocks resident at once.
 cudaError_t serve_grid(lbm_server *s) {
     s->smem = s->desc.max_slots * (int)sizeof(DomainEntry);
     int per_sm = 0, sms = 0, coop = 0;
@@ -320,36 +324,69 @@ cudaError_t serve_grid(lbm_server *s) {
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve, STEP_THREADS, s->smem);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->desc.device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, s->desc.device);
-    if (e == cudaSuccess && (!coop || per_sm < 1)) e = cudaErrorNotSupported;
-    s->grid = per_sm * sms;
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorNotSupported;
+    s->together = coop != 0;
+    s->resident_blocks = per_sm * sms;
+    s->grid = cooperative_blocks(s->resident_blocks);
     return e;
 }
 
-// Capture the tick: table copy, cleared health flags, the kernel, flags back.
-lbm_status capture_tick(lbm_server *s) {
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("begin capture: ") + cudaGetErrorString(e));
-    cudaMemcpyAsync(s->d_tab, s->h_tab, sizeof(TickTable), cudaMemcpyHostToDevice, s->stream);
-    cudaMemsetAsync(s->d_flags, 0, (STATUS_WORD + 1) * sizeof(uint32_t), s->stream);
+// The tick's work on the stream: table copy, cleared health flags, the kernel,
+// flags back.
+cudaError_t enqueue_tick(lbm_server *s) {
     const TickTable *tab = s->d_tab;
     int32_t *barrier = reinterpret_cast<int32_t *>(s->d_flags) + BARRIER_WORDS;
     uint32_t *status = s->d_flags + STATUS_WORD;
-    void *params[4] = {&tab, &barrier, &status, &s->polls};
-    const cudaError_t launch = cudaLaunchCooperativeKernel((const void *)k_serve, dim3((unsigned)s->grid),
-                                                           dim3(STEP_THREADS), params, (size_t)s->smem, s->stream);
-    cudaMemcpyAsync(s->h_flags, s->d_flags, (STATUS_WORD + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream);
-    e = cudaStreamEndCapture(s->stream, &g);
-    if (e == cudaSuccess && launch != cudaSuccess) {
-        cudaGraphDestroy(g);
-        e = launch;
+    cudaError_t e = cudaMemcpyAsync(s->d_tab, s->h_tab, sizeof(TickTable), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_flags, 0, (STATUS_WORD + 1) * sizeof(uint32_t), s->stream);
+    if (s->together) {
+        int k0 = 0, count = s->desc.steps_per_tick;
+        void *params[6] = {&tab, &k0, &count, &barrier, &status, &s->polls};
+        if (e == cudaSuccess)
+            e = cudaLaunchCooperativeKernel((const void *)k_serve, dim3((unsigned)s->grid), dim3(STEP_THREADS), params,
+                                            (size_t)s->smem, s->stream);
+    } else {
+        for (int k = 0; k < s->h_tab->steps && e == cudaSuccess; ++k) {
+            k_serve<<<(unsigned)s->grid, STEP_THREADS, (size_t)s->smem, s->stream>>>(tab, k, 1, barrier, status, s->polls);
+            e = cudaGetLastError();
+        }
     }
-    if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("end capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&s->exec, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->h_flags, s->d_flags, (STATUS_WORD + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream);
+    return e;
+}
+
+// Capture the tick in a graph.
+cudaError_t capture_tick(lbm_server *s) {
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    const cudaError_t work = enqueue_tick(s);
+    e = cudaStreamEndCapture(s->stream, &g);
+    if (work != cudaSuccess) e = work;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&s->exec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        s->exec = nullptr;
+        return e;
+    }
     s->graph_captures += 1;
-    return LBM_OK;
+    return e;
+}
+
+// One tick: the captured graph, or, where the device does not take the
+// cooperative launch, its steps one by one.
+cudaError_t run_tick(lbm_server *s) {
+    if (s->together) {
+        cudaError_t e = s->exec ? cudaSuccess : capture_tick(s);
+        if (e == cudaSuccess) e = cudaGraphLaunch(s->exec, s->stream);
+        if (e == cudaSuccess) s->graph_launches += 1;
+        if (!launch_refused(e)) return e;
+        cudaGetLastError();
+        s->together = false;
+        s->grid = s->resident_blocks;
+    }
+    return enqueue_tick(s);
 }
 
 // The copied flags and the host index are needed only until admission.
@@ -596,14 +633,10 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
             tab->n_nodes += (e.a.nbnodes + 31) / 32;
             tab->steps = std::max(tab->steps, e.steps);
         }
-    if (!s->exec) {
-        lbm_status st = capture_tick(s);
-        if (st != LBM_OK) return st;
-    }
     cudaError_t e;
     {
         const TraceRange run("lbm_server_tick: graph");
-        e = cudaGraphLaunch(s->exec, s->stream);
+        e = run_tick(s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     }
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("tick: ") + cudaGetErrorString(e));
@@ -619,7 +652,6 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
         if (running) *running = 0;
         return sfail(s, LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (tick kernel): its requests failed");
     }
-    s->graph_launches += 1;
     s->ticks += 1;
     // account, retire finished lattices
     std::vector<int64_t> still;
