@@ -12,12 +12,13 @@
 // a per-tick table that the graph copies to the device first.  The table
 // changes every tick, the graph never does.  Each cell is updated by the same
 // device code as lbm_step, so a lattice's result does not depend on what else
-// is resident.  A device that refuses the cooperative launch takes the steps in
-// a launch each.
+// is resident.  A tick of very many cell updates goes in several launches, and
+// a device that refuses the cooperative launch takes the steps in a launch each.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <condition_variable>
+#include <cstdlib>
 #include <cstring>
 #include <deque>
 #include <map>
@@ -40,6 +41,11 @@ float resolve_fp16_scale(float s);
 void ctx_tile_step_args(lbm_ctx *c, StepArgs *out);
 
 constexpr int MAX_SLOTS = LBM_SERVER_MAX_SLOTS;
+// Cell updates one launch takes at most, about a quarter of a second at the
+// 18.6 G a second of twelve lattices of 2.2 M cells: a tick of more (large
+// lattices, many steps) goes in several launches, so that the GPU is not one
+// kernel's for long.  LBM_LAUNCH_UPDATES sets another number, for tests.
+constexpr int64_t LAUNCH_UPDATES = (int64_t)1 << 32;
 
 struct alignas(16) DomainEntry {
     StepArgs a;        // state at the start of the tick: fin is the current buffer
@@ -109,8 +115,8 @@ __device__ __forceinline__ void serve_tile(const StepArgs a, const TileRec &rec,
         }                                                                                  \
     } while (0)
 
-// Steps k0 .. k0 + count - 1 of a tick, as far as its lattices go: all of them
-// in one cooperative launch, or one (no barrier then) in an ordinary launch.
+// Steps k0 .. k0 + count - 1 of a tick, as far as its lattices go: several in a
+// cooperative launch, or one (no barrier then) in an ordinary launch.
 // Before, a step was four launches in turn (fluid and
 // nodes of each precision) whose blocks copied a lattice's arguments to
 // shared memory for every 128 cells; here the table stays in shared memory,
@@ -233,7 +239,8 @@ struct lbm_server {
     uint32_t *d_flags = nullptr, *h_flags = nullptr;
     cudaGraphExec_t exec = nullptr;
     int grid = 0, resident_blocks = 0, smem = 0, polls = 0;  // of the tick's kernel
-    bool together = false;              // all steps in one cooperative launch; else a launch each
+    int64_t launch_updates = LAUNCH_UPDATES;
+    bool together = false;              // several steps in a cooperative launch; else a launch each
 };
 
 namespace {
@@ -331,23 +338,22 @@ cudaError_t serve_grid(lbm_server *s) {
     return e;
 }
 
-// The tick's work on the stream: table copy, cleared health flags, the kernel,
-// flags back.
-cudaError_t enqueue_tick(lbm_server *s) {
+// The tick's work on the stream: table copy, cleared health flags, the kernel
+// for `steps` steps, at most `each` of them in a launch, flags back.
+cudaError_t enqueue_tick(lbm_server *s, int steps, int each) {
     const TickTable *tab = s->d_tab;
     int32_t *barrier = reinterpret_cast<int32_t *>(s->d_flags) + BARRIER_WORDS;
     uint32_t *status = s->d_flags + STATUS_WORD;
     cudaError_t e = cudaMemcpyAsync(s->d_tab, s->h_tab, sizeof(TickTable), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->d_flags, 0, (STATUS_WORD + 1) * sizeof(uint32_t), s->stream);
-    if (s->together) {
-        int k0 = 0, count = s->desc.steps_per_tick;
-        void *params[6] = {&tab, &k0, &count, &barrier, &status, &s->polls};
-        if (e == cudaSuccess)
+    for (int k0 = 0; k0 < steps && e == cudaSuccess; k0 += each) {
+        if (each > 1) {
+            void *params[6] = {&tab, &k0, &each, &barrier, &status, &s->polls};
             e = cudaLaunchCooperativeKernel((const void *)k_serve, dim3((unsigned)s->grid), dim3(STEP_THREADS), params,
                                             (size_t)s->smem, s->stream);
-    } else {
-        for (int k = 0; k < s->h_tab->steps && e == cudaSuccess; ++k) {
-            k_serve<<<(unsigned)s->grid, STEP_THREADS, (size_t)s->smem, s->stream>>>(tab, k, 1, barrier, status, s->polls);
+            if (k0 > 0 && launch_refused(e)) e = cudaErrorLaunchFailure;  // not to be begun again
+        } else {  // no barrier
+            k_serve<<<(unsigned)s->grid, STEP_THREADS, (size_t)s->smem, s->stream>>>(tab, k0, 1, barrier, status, s->polls);
             e = cudaGetLastError();
         }
     }
@@ -361,7 +367,7 @@ cudaError_t capture_tick(lbm_server *s) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    const cudaError_t work = enqueue_tick(s);
+    const cudaError_t work = enqueue_tick(s, s->desc.steps_per_tick, s->desc.steps_per_tick);
     e = cudaStreamEndCapture(s->stream, &g);
     if (work != cudaSuccess) e = work;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&s->exec, g, 0);
@@ -374,19 +380,27 @@ cudaError_t capture_tick(lbm_server *s) {
     return e;
 }
 
-// One tick: the captured graph, or, where the device does not take the
-// cooperative launch, its steps one by one.
-cudaError_t run_tick(lbm_server *s) {
+// One tick of `cells` cells: the captured graph (all steps in one launch), or,
+// past LAUNCH_UPDATES or where the device does not take the cooperative
+// launch, its steps in several launches.
+cudaError_t run_tick(lbm_server *s, int64_t cells) {
+    const int steps = s->h_tab->steps;
     if (s->together) {
-        cudaError_t e = s->exec ? cudaSuccess : capture_tick(s);
-        if (e == cudaSuccess) e = cudaGraphLaunch(s->exec, s->stream);
-        if (e == cudaSuccess) s->graph_launches += 1;
+        const int64_t each = std::max<int64_t>(1, s->launch_updates / std::max<int64_t>(1, cells));
+        cudaError_t e = cudaSuccess;
+        if (each < steps) {
+            e = enqueue_tick(s, steps, (int)each);
+        } else {
+            if (!s->exec) e = capture_tick(s);
+            if (e == cudaSuccess) e = cudaGraphLaunch(s->exec, s->stream);
+            if (e == cudaSuccess) s->graph_launches += 1;
+        }
         if (!launch_refused(e)) return e;
         cudaGetLastError();
         s->together = false;
         s->grid = s->resident_blocks;
     }
-    return enqueue_tick(s);
+    return enqueue_tick(s, steps, 1);
 }
 
 // The copied flags and the host index are needed only until admission.
@@ -456,6 +470,7 @@ lbm_status lbm_server_create(const lbm_server_desc *desc, lbm_server **out) {
     std::unique_ptr<lbm_server> s(new lbm_server());
     s->desc = *desc;
     s->polls = barrier_polls();
+    if (const char *updates = std::getenv("LBM_LAUNCH_UPDATES")) s->launch_updates = std::max(1ll, std::atoll(updates));
     cudaSetDevice(desc->device);
     // on a failure below, free what was made so far (no worker runs yet)
     auto undo = [&](lbm_status st) {
@@ -612,6 +627,7 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
     TickTable *tab = s->h_tab;
     tab->n_domains = tab->n_tiles = tab->n_nodes = tab->steps = 0;
     const int K = s->desc.steps_per_tick;
+    int64_t cells = 0;
     std::vector<int> steps_now(s->resident.size()), flag_of(s->resident.size());
     // FP32 lattices first, then FP16S: the warps, which walk the list together,
     // then change from one collision's code to the other's once a step
@@ -632,11 +648,12 @@ lbm_status lbm_server_tick(lbm_server *s, int32_t *running, int32_t *queued) {
             tab->n_tiles += e.a.ntiles;
             tab->n_nodes += (e.a.nbnodes + 31) / 32;
             tab->steps = std::max(tab->steps, e.steps);
+            cells += r->n_active;
         }
     cudaError_t e;
     {
         const TraceRange run("lbm_server_tick: graph");
-        e = run_tick(s);
+        e = run_tick(s, cells);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     }
     if (e != cudaSuccess) return sfail(s, LBM_ERR_CUDA, std::string("tick: ") + cudaGetErrorString(e));

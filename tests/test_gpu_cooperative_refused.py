@@ -67,3 +67,16 @@ def test_server_ticks_run_step_by_step(lbm, monkeypatch):
     b = served(lbm)
     for (r, u), (q, v) in zip(a, b):
         assert np.isfinite(r).all() and np.array_equal(r, q) and np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("updates", [1, 200000, 700000])
+def test_long_ticks_go_in_several_launches(lbm, monkeypatch, updates):
+    """Past a number of cell updates (LBM_LAUNCH_UPDATES) a tick's steps go in
+    several launches of one, a few, or, once a lattice has finished, all steps:
+    the same results."""
+    monkeypatch.delenv("LBM_LAUNCH_UPDATES", raising=False)
+    a = served(lbm)
+    monkeypatch.setenv("LBM_LAUNCH_UPDATES", str(updates))
+    b = served(lbm)
+    for (r, u), (q, v) in zip(a, b):
+        assert np.isfinite(r).all() and np.array_equal(r, q) and np.array_equal(u, v)
