@@ -243,7 +243,17 @@ lbm_status need(lbm_ctx *c, bool geom, bool params, bool state) {
 // whose warp items are at most RUN_ROUNDS for each resident warp (about 310 000
 // cells; measured at k_run).  A launch takes RUN_MAX_STEPS at most, so that it
 // stays well under a second.
-constexpr int RUN_MIN_STEPS = 8, RUN_MAX_STEPS = 4096, RUN_ROUNDS = 4;
+// Up to RUN_HALF_ROUNDS items for each warp of half the grid (about 100 000
+// cells) the launch takes that half, two blocks per SM, so that lattices
+// stepped on streams of their own run side by side, as their per-step launches
+// do; a grid that fills the device has the others wait.  Half grid / full grid /
+// per step, us a step of one lattice alone and of four on four streams, FP32
+// nozzles of 49 000, 85 000 and 105 000 cells: 6.6 / 7.7 / 10.6 and 4.2 / 7.6 /
+// 5.2; 7.1 / 8.0 / 8.6 and 4.9 / 8.0 / 5.5; 8.5 / 8.4 / 9.7 and 5.8 / 8.4 / 6.1.
+// Beyond, the full grid is the faster one alone (48^3 box 7.2 against 8.8) and
+// the slower one of four (nozzles of 130 000 to 250 000 cells 10.3 to 13.1,
+// per step 7.6 to 12.0).
+constexpr int RUN_MIN_STEPS = 8, RUN_MAX_STEPS = 4096, RUN_ROUNDS = 4, RUN_HALF_ROUNDS = 3;
 
 // Device records of the inlet/outlet nodes (NODE_INT4S) from the index's list.
 std::vector<int32_t> node_records(const lbm_ctx *c) {
@@ -423,7 +433,9 @@ int run_blocks(lbm_ctx *c, int64_t n) {
         return 0;
     }
     if (cs != cudaStreamCaptureStatusNone) return 0;
-    return cooperative_blocks((int)std::min<int64_t>(c->run_blocks, (items + warps - 1) / warps));
+    const int half = std::max(1, c->run_blocks / 2);
+    const int most = items <= (int64_t)RUN_HALF_ROUNDS * warps * half ? half : c->run_blocks;
+    return cooperative_blocks((int)std::min<int64_t>(most, (items + warps - 1) / warps));
 }
 
 // Ghost slots and periodic copies of the current buffer from its active cells.

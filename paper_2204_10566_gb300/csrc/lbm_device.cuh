@@ -2040,10 +2040,10 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STAGE_BLOCKS) k_step_units(c
 // in the per-step kernels, to the same bits.
 //
 // Measured per step, one launch each and in one: laminar nozzle 24x24x160 FP32
-// 10.7 -> 7.6 us, FP16S 12.0 -> 8.4; pipe of 237 000 cells FP32 14.0 -> 11.4;
-// 64^3 lattice BGK 14.4 -> 11.1 (FP32 per step 17.4 with the cascade); smooth
-// nozzle of 226 000 cells 24.1 -> 15.8; 32^3 box 6.2 -> 3.9, of which about
-// 1.5 us is the barrier.  At 80^3 (6.6 rounds) both take 29 us.  4 blocks per
+// 10.6 -> 6.6 us, FP16S 11.2 -> 7.1; pipe of 237 000 cells FP32 14.4 -> 11.2,
+// FP16S 12.5 -> 12.9; 64^3 lattice BGK 14.4 -> 11.1 (FP32 per step 17.4 with the
+// cascade); smooth nozzle of 226 000 cells 24.1 -> 15.8; 32^3 box 7.4 -> 3.7, of
+// which about 1.5 us is the barrier.  At 80^3 (6.6 rounds) both take 29 us.  4 blocks per
 // SM (128 registers, no spills); 5 and 8 spill and take 10 to 40 % longer.  The
 // line sink for every tile: with the fast tiles' path as well the nozzle takes
 // 8.3 us.
