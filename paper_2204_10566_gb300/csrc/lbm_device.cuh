@@ -225,15 +225,7 @@ __device__ __forceinline__ void record_stress(const StepArgs &a, int slot, R ome
 // --------------------------------------------------------------- collision
 
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-// 1/x from the hardware's approximation x0 (about 20 bits) and one
-// third-order step, x0 (1 + e + e^2) with e = 1 - x x0, whose remainder e^3 is
-// below rounding: four FP64 operations.
-__device__ __forceinline__ double recip(double x) {
-    double x0;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(x));
-    const double e = __fma_rn(-x, x0, 1.0);
-    return __fma_rn(x0, __fma_rn(e, e, e), x0);
-}
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
 
@@ -581,9 +573,10 @@ __device__ __forceinline__ void relaxed_lines(R k, const R (&a2)[6], R ro, R dro
 //   M(xxyy) = p*_xx E_y + A_yy E_x + 4 u_x u_y A_xy + theta u_y^2, E = u^2 + theta;
 //   M(xxyz) = u_z M(xxy) + 2 u_x u_y A_xz + A_yz E_x;
 //   M(xxyyz) = u_z (M(xxyy) + theta^2) + 2 u_x A_xz E_y + 2 u_y A_yz E_x; ...
-// 254 FP64 instructions a cell with the moment sums, against about 390 for
-// the line-by-line inverse; at the pipe's 86-87 % either way, the Re 3500
-// nozzle's step takes 2.09 ms instead of 3.12 ms (1 372 -> 2 050 MLUPS).
+// About 260 FP64 instructions a cell with the moment sums and the division,
+// against about 390 for the line-by-line inverse; at the pipe's 86-87 % either
+// way, the Re 3500 nozzle's step takes 2.12 ms instead of 3.12 ms (1 372 ->
+// 2 030 MLUPS).
 template <class R, class Out>
 __device__ __forceinline__ void raw_finish(const R (&m)[10], R omega, R &rho, R &ux, R &uy, R &uz, const Out &sink) {
     const R drho = m[0], jx = m[1], jy = m[2], jz = m[3], th = theta0<R>(), h = R(0.5), q = R(0.25), m2 = R(-2);
@@ -2154,9 +2147,15 @@ __device__ __forceinline__ void load_cell(const void *f, int64_t stride, int slo
 __device__ __forceinline__ bool normal(double x) {
     return ((unsigned)__double2hiint(x) & 0x7ff00000u) - 0x00100000u < 0x7fe00000u;
 }
+// The same for x and 1 / x: |x| < 2^1022 too.
+__device__ __forceinline__ bool invertible(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7ff00000u) - 0x00100000u < 0x7fc00000u;
+}
 
-// j / rho for a normal rho from its reciprocal inv, corrected once: the last
-// bit of the division at three operations.  An infinite j stays infinite.
+// j / rho, for an invertible rho, from its correctly rounded reciprocal inv:
+// the residual of j inv corrects it once, to the correctly rounded quotient
+// (Markstein, IBM J. Res. Dev. 34, 1990; the residual must not underflow: |j|
+// above 2^-968), at three operations.  An infinite j stays infinite.
 __device__ __forceinline__ double quotient(double j, double rho, double inv) {
     const double q = __dmul_rn(j, inv);
     return normal(q) ? __fma_rn(__fma_rn(-rho, q, j), inv, q) : q;
@@ -2181,7 +2180,7 @@ __device__ __forceinline__ void moments_of(const double (&d)[27], double inv_sca
     double jy = hi - lo, jz = ((s[6] - s[0]) + (s[8] - s[2])) + (s[7] - s[1]), drho = (lo + hi) + mid;
     if constexpr (Storage<P>::SCALED) drho *= sc, jx *= sc, jy *= sc, jz *= sc;
     rho = 1.0 + drho;
-    if (normal(rho)) {
+    if (invertible(rho)) {
         const double inv = recip(rho);
         ux = quotient(jx, rho, inv);
         uy = quotient(jy, rho, inv);
