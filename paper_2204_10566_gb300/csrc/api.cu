@@ -344,17 +344,6 @@ int partial_capacity(const lbm_ctx *c, int64_t n_wnodes) {
     return std::max({c->fluid_blocks + nodes, tiles + nodes, split + nodes, reduce_blocks(c->idx.nslots)});
 }
 
-// Faults in the pages of a host array that a device copy is about to fill,
-// one write per page.  A caller's fresh array has none, and a copy engine that
-// meets the missing ones one by one waits for the host each time: 25-48 ms for
-// the axial averages of 3.1 million cells (50 MB), 1.6-2.3 ms with the pages
-// faulted in here while the kernel runs (7.4 ms through a host copy).
-void fault_in(void *p, size_t bytes) {
-    volatile char *c = static_cast<volatile char *>(p);
-    for (size_t k = 0; k < bytes; k += 4096) c[k] = 0;
-    if (bytes) c[bytes - 1] = 0;
-}
-
 // Transfers of per-cell arrays in the active order run in TRANSFER_PARTS parts
 // beside the kernel that reads or writes them, from this many cells on: the
 // copies go on the context's second stream, each part's kernel after (or
@@ -1418,7 +1407,7 @@ lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int3
     if (e == cudaSuccess)
         e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act, c->idx.nslots,
                               1.0 / (double)c->stats_samples, d, nullptr, c->stream);
-    if (layout == LBM_LAYOUT_ACTIVE) fault_in(to, bytes);
+    if (e == cudaSuccess && layout == LBM_LAYOUT_ACTIVE) fault_in(to, bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(to, d, bytes, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dev_free(c, d, bytes);

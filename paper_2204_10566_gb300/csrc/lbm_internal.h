@@ -329,6 +329,19 @@ struct HostIndex {
     std::vector<int64_t> box_of_active;   // [n_active]
 };
 
+// Faults in the pages of a host array that a device copy is about to fill, one
+// write per page, of the byte that is there: should the copy fail, the caller
+// still has what was in the array.  A caller's fresh array has no pages, and a
+// copy engine that meets the missing ones one by one waits for the host each
+// time: 25-48 ms for the axial averages of 3.1 million cells (50 MB), 1.6-2.3 ms
+// with the pages faulted in here while the kernel runs (7.4 ms through a host
+// copy).
+inline void fault_in(void *p, size_t bytes) {
+    volatile char *c = static_cast<volatile char *>(p);
+    for (size_t k = 0; k < bytes; k += 4096) c[k] = c[k];
+    if (bytes) c[bytes - 1] = c[bytes - 1];
+}
+
 // Slack (elements) allocated before and after every population buffer and
 // around the link-word array (keeps 256-byte alignment of the buffers).
 inline int64_t buffer_margin(int nx) { return ((int64_t)nx + 128 + 63) & ~(int64_t)63; }
