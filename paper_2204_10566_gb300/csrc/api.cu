@@ -20,6 +20,7 @@ struct lbm_ctx {
     cudaStream_t stream = nullptr;
     std::string err;
     bool has_geom = false, has_params = false, has_state = false;
+    bool served = false;             // of a request server: read back once, at its end
     HostIndex idx;
     // device buffers
     void *f[2] = {nullptr, nullptr};      // population buffers (inside the raw allocations)
@@ -137,7 +138,10 @@ void dev_free(lbm_ctx *c, void *p, size_t bytes) {
 }
 
 size_t pop_bytes(const lbm_ctx *c) { return (size_t)27 * (size_t)c->idx.nslots * storage_bytes(c->desc.precision); }
-size_t margin_bytes(const lbm_ctx *c) { return (size_t)buffer_margin(c->idx.n_row) * storage_bytes(c->desc.precision); }
+size_t margin_bytes(const lbm_ctx *c) {
+    const int64_t margin = c->idx.units.empty() ? buffer_margin(c->idx.n_row) : stage_margin(c->idx.n_row);
+    return (size_t)margin * storage_bytes(c->desc.precision);
+}
 size_t raw_pop_bytes(const lbm_ctx *c) { return pop_bytes(c) + 2 * margin_bytes(c); }
 size_t raw_mask_bytes(const lbm_ctx *c) { return ((size_t)c->idx.nslots + 2 * MASK_MARGIN) * 4; }
 
@@ -307,13 +311,13 @@ bool tiled(const lbm_ctx *c) {
 int64_t unit_count(const lbm_ctx *c) {
     return c->d_units_wall ? c->n_units_wall : (int64_t)c->idx.units.size() / UNIT_INTS;
 }
-bool staged(const lbm_ctx *c) {
+bool stageable(const lbm_ctx *c) {  // at the default ghost rates
     const int64_t least = c->fluid_kernel == FluidKernel::STAGED ? 1
                           : c->fluid_kernel == FluidKernel::AUTO ? (int64_t)STAGE_ROUNDS * c->stage_blocks * (STEP_THREADS / 32)
                                                                  : INT64_MAX;
-    return c->desc.precision == LBM_FP16S && c->mode == RATE_ONE && !wide_offsets(c) && c->stage_blocks > 0 &&
-           unit_count(c) >= least;
+    return c->desc.precision == LBM_FP16S && !wide_offsets(c) && c->stage_blocks > 0 && unit_count(c) >= least;
 }
+bool staged(const lbm_ctx *c) { return c->mode == RATE_ONE && stageable(c); }
 // Words of the status allocation (256 bytes): 0 the status, TICKET_WORD and
 // the next the staged kernel's counters, BARRIER_WORD and the next those of
 // the several-step kernel, each pair in a sector of its own.
@@ -729,10 +733,11 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
         wn.empty() ? std::vector<int32_t>()
                    : build_tiles(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
     const std::vector<int32_t> units =
-        wn.empty() ? std::vector<int32_t>()
-                   : build_units(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
-    const std::vector<int2> items = build_pair_items(tiles);
-    const std::vector<int2> rest = build_rest_chunks(chunks, tiles, items);
+        wn.empty() || c->idx.units.empty()
+            ? std::vector<int32_t>()
+            : build_units(chunks, c->idx.row_nb, c->idx.mask, c->idx.n_row, periodic_rows(c) != 0);
+    const std::vector<int2> items = pairs(c) ? build_pair_items(tiles) : std::vector<int2>();
+    const std::vector<int2> rest = pairs(c) ? build_rest_chunks(chunks, tiles, items) : std::vector<int2>();
     c->d_wall_qidx = (int32_t *)dev_alloc(c, qidx.size() * 4);
     c->d_wall_q = (uint8_t *)dev_alloc(c, rec.size());
     c->n_wall_q = n;
@@ -743,11 +748,11 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
         c->n_tiles_wall = (int64_t)tiles.size() / TILE_INTS;
         c->d_tiles_wall = (int32_t *)dev_alloc(c, tiles.size() * 4);
         c->n_units_wall = (int64_t)units.size() / UNIT_INTS;
-        c->d_units_wall = (int32_t *)dev_alloc(c, units.size() * 4);
+        c->d_units_wall = units.empty() ? nullptr : (int32_t *)dev_alloc(c, units.size() * 4);
         c->n_items_wall = (int64_t)items.size();
-        c->d_items_wall = (int2 *)dev_alloc(c, items.size() * 8);
+        c->d_items_wall = items.empty() ? nullptr : (int2 *)dev_alloc(c, items.size() * 8);
         c->n_rest_wall = (int64_t)rest.size();
-        c->d_rest_wall = (int2 *)dev_alloc(c, rest.size() * 8);
+        c->d_rest_wall = rest.empty() ? nullptr : (int2 *)dev_alloc(c, rest.size() * 8);
     }
     const int capacity = partial_capacity(c, c->n_wnodes);
     double *partials = c->d_partials;
@@ -760,8 +765,9 @@ lbm_status lbm_set_wall_q(lbm_ctx *c, const int64_t *cells, const uint8_t *q, in
         }
     }
     if (!c->d_wall_qidx || !c->d_wall_q ||
-        (!wn.empty() && (!c->d_wnodes || !c->d_chunks_wall || !c->d_tiles_wall || !c->d_units_wall ||
-                         !c->d_items_wall || !c->d_rest_wall)) ||
+        (!wn.empty() && (!c->d_wnodes || !c->d_chunks_wall || !c->d_tiles_wall)) ||
+        (!units.empty() && !c->d_units_wall) || (!items.empty() && !c->d_items_wall) ||
+        (!rest.empty() && !c->d_rest_wall) ||
         !partials) {
         release_wall_q(c);
         return fail(c, LBM_ERR_OOM, "wall-distance allocation failed");
@@ -799,7 +805,7 @@ lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *flags) {
     std::string msg = build_index(flags, c->desc.nx, c->desc.ny, c->desc.nz, c->desc.periodic, idx, 0,
                                   c->desc.row_axis);
     if (!msg.empty()) return fail(c, LBM_ERR_ARG, msg);
-    return lbm::ctx_install_index(c, std::move(idx));
+    return lbm::ctx_install_index(c, std::move(idx), false);
 }
 
 }  // extern "C"
@@ -808,26 +814,33 @@ namespace lbm {
 
 int64_t ctx_footprint(const lbm_desc &d, const HostIndex &ix) {
     const int S = storage_bytes(d.precision);
-    const int64_t pop = 27 * ix.nslots * S + 2 * buffer_margin(ix.n_row) * S;
+    const int64_t pop = 27 * ix.nslots * S + 2 * buffer_margin(ix.n_row) * S;  // a served context has no unit records
     const int64_t blocks = std::max<int64_t>(fluid_blocks((int32_t)ix.chunks.size()) + node_blocks((int64_t)ix.bnodes.size()),
                                              reduce_blocks(ix.nslots));
     return 2 * pop + (ix.nslots + 2 * MASK_MARGIN) * 4 + (int64_t)ix.row_nb.size() * 4 + (int64_t)ix.chunks.size() * 8 +
            (int64_t)(ix.bnodes.size() * NODE_BYTES) + ix.nslots * 4 + (int64_t)ix.tiles.size() * 4 +
-           (int64_t)ix.units.size() * 4 + (int64_t)ix.pair_items.size() * 8 + (int64_t)ix.rest_chunks.size() * 8 +
            blocks * REDUCE_SLOTS * 8 + 64 + 256;
 }
 
-lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
+lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx, bool served) {
     DeviceGuard g(c->desc.device);
     CK(cudaStreamSynchronize(c->stream), "sync before geometry change");
     release_geometry(c);
     c->idx = std::move(idx);
     const size_t ns = (size_t)c->idx.nslots;
+    // only the records that this context's kernels read take device memory (the
+    // server's kernel walks the tiles)
+    c->stage_blocks = DISPATCH(c->desc.precision, step_stage_blocks, c->desc.device);
+    c->served = served;
+    if (served || !stageable(c)) std::vector<int32_t>().swap(c->idx.units);
+    if (served || !pairs(c)) {
+        std::vector<int2>().swap(c->idx.pair_items);
+        std::vector<int2>().swap(c->idx.rest_chunks);
+    }
     c->fluid_blocks = DISPATCH(c->desc.precision, step_fluid_blocks, (int32_t)c->idx.chunks.size());
     c->nblocks = partial_capacity(c, 0);
     c->run_mode = -1;
     c->run_unread = c->torn = false;
-    c->stage_blocks = DISPATCH(c->desc.precision, step_stage_blocks, c->desc.device);
     for (int k = 0; k < 2; ++k) {
         c->f_raw[k] = dev_alloc(c, raw_pop_bytes(c));
         c->f[k] = c->f_raw[k] ? static_cast<char *>(c->f_raw[k]) + margin_bytes(c) : nullptr;
@@ -839,14 +852,15 @@ lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx) {
     c->d_bnodes = (int4 *)dev_alloc(c, c->idx.bnodes.size() * NODE_BYTES);
     c->d_act = (int32_t *)dev_alloc(c, ns * 4);
     c->d_tiles = (int32_t *)dev_alloc(c, c->idx.tiles.size() * 4);
-    c->d_units = (int32_t *)dev_alloc(c, c->idx.units.size() * 4);
-    c->d_items = (int2 *)dev_alloc(c, c->idx.pair_items.size() * 8);
-    c->d_rest = (int2 *)dev_alloc(c, c->idx.rest_chunks.size() * 8);
+    if (!c->idx.units.empty()) c->d_units = (int32_t *)dev_alloc(c, c->idx.units.size() * 4);
+    if (!c->idx.pair_items.empty()) c->d_items = (int2 *)dev_alloc(c, c->idx.pair_items.size() * 8);
+    if (!c->idx.rest_chunks.empty()) c->d_rest = (int2 *)dev_alloc(c, c->idx.rest_chunks.size() * 8);
     c->d_partials = (double *)dev_alloc(c, (size_t)c->nblocks * REDUCE_SLOTS * 8);
     c->d_health = (double *)dev_alloc(c, 8 * 8);
     c->d_status = (uint32_t *)dev_alloc(c, 256);
     if (!c->f[0] || !c->f[1] || !c->d_mask || !c->d_row_nb || !c->d_chunks || !c->d_bnodes || !c->d_act ||
-        !c->d_tiles || !c->d_units || !c->d_items || !c->d_rest || !c->d_partials || !c->d_health || !c->d_status) {
+        !c->d_tiles || (!c->idx.units.empty() && !c->d_units) || (!c->idx.pair_items.empty() && !c->d_items) ||
+        (!c->idx.rest_chunks.empty() && !c->d_rest) || !c->d_partials || !c->d_health || !c->d_status) {
         release_geometry(c);
         return fail(c, LBM_ERR_OOM, "device allocation failed in lbm_set_geometry");
     }
@@ -1229,7 +1243,9 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
     DeviceGuard g(c->desc.device);
     const int64_t n = c->idx.n_active;
     const size_t bytes = (size_t)n * 4 * 8;
-    double *d = (double *)dev_alloc(c, bytes);  // rho[n], then u[n][3]
+    // rho[n], then u[n][3]; a served lattice, done with its steps, has the other
+    // population buffer for them (54 bytes a cell or more)
+    double *d = (double *)(c->served ? c->f_raw[1 - c->cur] : dev_alloc(c, bytes));
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n * 4 : 0);
     double *hr = rho, *hu = u;  // in the active order each part goes straight into the caller's arrays
@@ -1251,7 +1267,7 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
                 r = cudaMemcpyAsync(hu + 3 * k0, d + n + 3 * k0, (size_t)(k1 - k0) * 24, cudaMemcpyDeviceToHost, s);
             return r;
         });
-    dev_free(c, d, bytes);
+    if (!c->served) dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "get moments");
     st = settle(c);
     if (st) return st;

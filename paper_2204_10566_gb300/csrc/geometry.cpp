@@ -650,7 +650,7 @@ std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, in
         if (lo < 0 || hi < lo || hi > 7 || ((int64_t)ub[4] + rec[0]) % UNIT_ALIGN || rec[0] % CHUNK) return "unit start or pieces";
         for (int j = 0; j < 9; ++j) {
             const int64_t first = (int64_t)ub[j] + rec[0] + CHUNK * (lo - 1), end = (int64_t)ub[j] + rec[0] + CHUNK * (hi + 2);
-            if (first < -margin || end > ns + margin) return "unit window outside the buffer";
+            if (first < -stage_margin(np) || end > ns + stage_margin(np)) return "unit window outside the buffer";
         }
         bool plain = true, ends = false;
         for (int l = 0; l < UNIT_CELLS; ++l) {

@@ -344,7 +344,9 @@ inline void fault_in(void *p, size_t bytes) {
 
 // Slack (elements) allocated before and after every population buffer and
 // around the link-word array (keeps 256-byte alignment of the buffers).
-inline int64_t buffer_margin(int nx) { return ((int64_t)nx + 128 + 63) & ~(int64_t)63; }
+inline int64_t buffer_margin(int nx) { return ((int64_t)nx + 64 + 63) & ~(int64_t)63; }
+// The same for a context with unit records, whose windows reach further.
+inline int64_t stage_margin(int nx) { return ((int64_t)nx + 128 + 63) & ~(int64_t)63; }
 constexpr int64_t MASK_MARGIN = 64;
 
 // Returns "" on success, else a description of the inconsistency.  With
@@ -359,8 +361,8 @@ int choose_row_axis(int nx, int ny, int nz, int requested);
 std::string validate_index(const HostIndex &ix, const uint8_t *flags, int nx, int ny, int nz, int periodic);
 
 // Hooks into a context for the request server (implemented in api.cu).
-int64_t ctx_footprint(const lbm_desc &desc, const HostIndex &ix);  // device bytes lbm_set_geometry allocates
-lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx);        // allocate + upload a built index
+int64_t ctx_footprint(const lbm_desc &desc, const HostIndex &ix);  // device bytes of a served context
+lbm_status ctx_install_index(lbm_ctx *c, HostIndex &&idx, bool served);  // allocate + upload a built index
 void ctx_step_args(lbm_ctx *c, StepArgs *out);                      // arguments of the next step
 void ctx_advance(lbm_ctx *c, int64_t steps);                        // account for steps run elsewhere
 int64_t ctx_steps(const lbm_ctx *c);

@@ -250,8 +250,8 @@ lbm_status sfail(lbm_server *s, lbm_status st, const std::string &m) {
     return st;
 }
 
-// Device bytes a request holds while resident: the context's buffers plus
-// the readback staging of its moments.
+// Device bytes a request holds while resident: the context's buffers (the
+// readback of its moments is staged in one of them).
 int64_t request_footprint(const lbm_request &q, const HostIndex &idx) {
     lbm_desc d{};
     d.nx = q.nx;
@@ -259,7 +259,7 @@ int64_t request_footprint(const lbm_request &q, const HostIndex &idx) {
     d.nz = q.nz;
     d.periodic = q.periodic;
     d.precision = q.precision;
-    return ctx_footprint(d, idx) + idx.n_active * 32;
+    return ctx_footprint(d, idx);
 }
 
 // The checks of lbm_server_submit that need no index (host only).  *active
@@ -431,7 +431,7 @@ lbm_status admit(lbm_server *s, Request *r) {
     d.allocator = s->desc.allocator;
     lbm_ctx *c = nullptr;
     lbm_status st = lbm_create(&d, &c);
-    if (st == LBM_OK) st = ctx_install_index(c, std::move(r->idx));
+    if (st == LBM_OK) st = ctx_install_index(c, std::move(r->idx), true);
     if (st == LBM_OK) st = lbm_set_params(c, &r->req.params);
     const double u0[3] = {0.0, 0.0, 0.0};
     if (st == LBM_OK) st = lbm_init_equilibrium(c, 1.0, u0);
