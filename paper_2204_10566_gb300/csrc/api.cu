@@ -388,15 +388,17 @@ cudaError_t in_parts(lbm_ctx *c, int64_t n, cudaStream_t first_on, cudaStream_t 
 }
 
 // Status of the several-step launches so far, for a call that reads the state
-// back: queue_status before its own work on c->stream, settle once the stream
-// is idle.  No cost when the last look was after the last such launch.
-cudaError_t queue_status(lbm_ctx *c) {
+// back: queue_status behind its own copies to the host, on their stream (before
+// the kernels, the copy would have them wait for the copy engine and back: 20
+// us), settle once they are done.  No cost when the last look was after the last
+// such launch.
+cudaError_t queue_status(lbm_ctx *c, cudaStream_t s) {
     if (!c->run_unread) return cudaSuccess;
     if (!c->h_status && cudaMallocHost(&c->h_status, sizeof *c->h_status) != cudaSuccess) {
         c->h_status = nullptr;
         cudaGetLastError();
     }
-    return cudaMemcpyAsync(c->h_status ? c->h_status : &c->status_word, c->d_status, 4, cudaMemcpyDeviceToHost, c->stream);
+    return cudaMemcpyAsync(c->h_status ? c->h_status : &c->status_word, c->d_status, 4, cudaMemcpyDeviceToHost, s);
 }
 lbm_status settle(lbm_ctx *c) {
     if (c->run_unread && ((c->h_status ? *c->h_status : c->status_word) & 2u)) c->torn = true;
@@ -1112,16 +1114,16 @@ lbm_status lbm_get_populations(lbm_ctx *c, double *f, int32_t layout) {
     const size_t bytes = (size_t)n * 27 * 8;
     double *d = (double *)dev_alloc(c, bytes);
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
-    cudaError_t e = queue_status(c);
-    if (e == cudaSuccess)
-        e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_act, c->idx.nslots,
-                     1.0f / fp16_scale(c), d, c->stream);
+    cudaError_t e = DISPATCH(c->desc.precision, launch_get_populations, c->f[c->cur], c->d_act, c->idx.nslots,
+                             1.0f / fp16_scale(c), d, c->stream);
     if (layout == LBM_LAYOUT_ACTIVE) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, bytes, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = queue_status(c, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     } else {
         std::vector<double> h((size_t)n * 27);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, bytes, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = queue_status(c, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess && (st = settle(c)) == LBM_OK) {
             memset(f, 0, (size_t)layout_count(c, layout) * 27 * 8);
@@ -1253,8 +1255,7 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
         hr = h.data();
         hu = h.data() + n;
     }
-    const cudaError_t queued = queue_status(c);
-    const cudaError_t e = queued != cudaSuccess ? queued : in_parts(
+    const cudaError_t e = in_parts(
         c, n, c->stream, c->side.stream,
         [&](int64_t k0, int64_t k1, cudaStream_t s) {
             return DISPATCH(c->desc.precision, launch_moments, c->f[c->cur], c->d_act, k0, k1, c->idx.nslots,
@@ -1265,6 +1266,7 @@ lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *u, int32_t layout) {
             if (rho) r = cudaMemcpyAsync(hr + k0, d + k0, (size_t)(k1 - k0) * 8, cudaMemcpyDeviceToHost, s);
             if (u && r == cudaSuccess)
                 r = cudaMemcpyAsync(hu + 3 * k0, d + n + 3 * k0, (size_t)(k1 - k0) * 24, cudaMemcpyDeviceToHost, s);
+            if (k1 == n && r == cudaSuccess) r = queue_status(c, s);
             return r;
         });
     if (!c->served) dev_free(c, d, bytes);
@@ -1288,12 +1290,12 @@ lbm_status lbm_get_totals(lbm_ctx *c, double *mass, double mom[3]) {
     lbm_status st = need(c, true, false, true);
     if (st) return st;
     DeviceGuard g(c->desc.device);
-    CK(queue_status(c), "read status");
     CK(DISPATCH(c->desc.precision, launch_reduce, c->f[c->cur], c->d_act, c->idx.nslots, 1.0f / fp16_scale(c),
                 c->d_partials, c->stream),
        "reduce");
     CK(launch_finalize(c->d_partials, reduce_blocks(c->idx.nslots), c->d_health, c->d_status, c->stream), "finalize");
     CK(cudaMemcpyAsync(c->health, c->d_health, 6 * 8, cudaMemcpyDeviceToHost, c->stream), "read totals");
+    CK(queue_status(c, c->stream), "read status");
     CK(cudaStreamSynchronize(c->stream), "sync totals");
     st = settle(c);
     if (st) return st;
@@ -1380,15 +1382,14 @@ lbm_status lbm_stats_get(lbm_ctx *c, double *mean_uz, double *mean_uzuz, int64_t
     double *d = (double *)dev_alloc(c, bytes);  // <u_z>[n], then <u_z^2>[n]
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n : 0);
-    cudaError_t e = queue_status(c);
-    if (e == cudaSuccess)
-        e = launch_stats_mean(c->d_stats, STATS_AXIAL, c->d_act, c->idx.nslots, 1.0 / (double)c->stats_samples, d, d + n,
-                              c->stream);
+    cudaError_t e = launch_stats_mean(c->d_stats, STATS_AXIAL, c->d_act, c->idx.nslots, 1.0 / (double)c->stats_samples,
+                                      d, d + n, c->stream);
     for (int q = 0; q < 2; ++q) {
         if (e != cudaSuccess || !out[q]) continue;
         double *to = layout == LBM_LAYOUT_BOX ? h.data() : out[q];  // the active order goes straight to the caller
         if (layout == LBM_LAYOUT_ACTIVE) fault_in(to, total);
         e = cudaMemcpyAsync(to, d + q * n, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = queue_status(c, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess && (st = settle(c)) != LBM_OK) break;
         if (e == cudaSuccess && layout == LBM_LAYOUT_BOX)
@@ -1419,12 +1420,11 @@ lbm_status lbm_stats_get_full(lbm_ctx *c, double *mean, int64_t *n_samples, int3
     if (!d) return fail(c, LBM_ERR_OOM, "staging allocation failed");
     std::vector<double> h(layout == LBM_LAYOUT_BOX ? (size_t)n * Q : 0);
     double *to = layout == LBM_LAYOUT_BOX ? h.data() : mean;
-    cudaError_t e = queue_status(c);
-    if (e == cudaSuccess)
-        e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act, c->idx.nslots,
-                              1.0 / (double)c->stats_samples, d, nullptr, c->stream);
+    cudaError_t e = launch_stats_mean(c->d_stats + (size_t)STATS_AXIAL * (size_t)c->idx.nslots, Q, c->d_act,
+                                      c->idx.nslots, 1.0 / (double)c->stats_samples, d, nullptr, c->stream);
     if (e == cudaSuccess && layout == LBM_LAYOUT_ACTIVE) fault_in(to, bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(to, d, bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = queue_status(c, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dev_free(c, d, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "stats readback");
@@ -1483,11 +1483,11 @@ lbm_status lbm_checkpoint(lbm_ctx *c, void *buf, size_t bytes) {
     char *p = static_cast<char *>(buf);
     memcpy(p, &h, sizeof h);
     p += sizeof h;
-    CK(queue_status(c), "read status");
     CK(cudaMemcpyAsync(p, c->f[c->cur], pop_bytes(c), cudaMemcpyDeviceToHost, c->stream), "checkpoint f");
     p += pop_bytes(c);
     if (c->d_stats)
         CK(cudaMemcpyAsync(p, c->d_stats, stats_bytes(c), cudaMemcpyDeviceToHost, c->stream), "checkpoint stats");
+    CK(queue_status(c, c->stream), "read status");
     CK(cudaStreamSynchronize(c->stream), "sync checkpoint");
     return settle(c);
 }
