@@ -37,8 +37,6 @@
 #ifndef LBM_STEP_MIN_BLOCKS
 #define LBM_STEP_MIN_BLOCKS 8
 #endif
-// The same for the kernel of the cells with interpolated walls, which keeps
-// the wall record and the own-slot values of a cell in registers as well.
 // When the FP32 chunk kernel runs (LBM_FLUID_KERNEL=chunk), the inlet/outlet
 // nodes ride in its trailing blocks instead of a launch of their own: +2 % on
 // the Re 3500 nozzle, although the node path spills at the fluid path's
@@ -61,6 +59,9 @@
 #ifndef LBM_FAST_PATH
 #define LBM_FAST_PATH 1
 #endif
+// Minimum resident blocks of the kernel of the cells with interpolated walls,
+// which keeps the wall record and the own-slot values of a cell in registers as
+// well.
 #ifndef LBM_STEP_MIN_BLOCKS_WALLQ
 #define LBM_STEP_MIN_BLOCKS_WALLQ 4
 #endif
