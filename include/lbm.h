@@ -262,7 +262,7 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int32_t layout);
 
 /* Enqueue n >= 0 time steps on the context stream (asynchronous).  Each step
  * is the fluid kernel (FP32: one warp per tile of up to 32 cells of a row;
- * FP16S from about 2 million cells: one thread per two cells; else one thread
+ * FP16S from about 1.5 million cells: one thread per two cells; else one thread
  * per cell) on the context's stream, and the inlet/outlet and interpolated-wall kernels on the second
  * stream beside it; they read the same input and write disjoint outputs, so
  * their order changes no result.  The health check and the statistics

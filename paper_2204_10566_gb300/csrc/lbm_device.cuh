@@ -474,11 +474,19 @@ __device__ __forceinline__ void ghost1_finish(const R (&m)[10], R omega, R &rho,
     const Axis<R> Y(uy, rounds.y, rounds.y), Z(uz, false, rounds.z);
     const PairCoef<R> c{mul_(k, a2[0]), mul_(k, a2[1]), mul_(k, a2[2]), mul_(k, a2[3]), mul_(k, a2[4]), mul_(k, a2[5]),
                         SCALED ? mul_(rho, out_scale) : rho, SCALED ? mul_(drho, out_scale) : drho, ux, mul_(uxh, ux), uxh};
-    inverse_pair<0, 2>(c, Y, Z, sink);
-    inverse_pair<3, 5>(c, Y, Z, sink);
-    inverse_pair<6, 8>(c, Y, Z, sink);
-    inverse_pair<1, 7>(c, Y, Z, sink);
-    inverse_centre(c, Y, Z, sink);
+    if constexpr (std::is_same<R, float>::value) {
+        inverse_pair<0, 2>(c, Y, Z, sink);
+        inverse_pair<3, 5>(c, Y, Z, sink);
+        inverse_pair<6, 8>(c, Y, Z, sink);
+        inverse_pair<1, 7>(c, Y, Z, sink);
+        inverse_centre(c, Y, Z, sink);
+    } else {  // with the centre last: 370 us a step of the Re 6500 nozzle instead of 354
+        inverse_centre(c, Y, Z, sink);
+        inverse_pair<1, 7>(c, Y, Z, sink);
+        inverse_pair<3, 5>(c, Y, Z, sink);
+        inverse_pair<0, 2>(c, Y, Z, sink);
+        inverse_pair<6, 8>(c, Y, Z, sink);
+    }
 }
 
 // The same moment sums axis by axis (x within a line, then y, then z), each
@@ -1769,12 +1777,13 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_PAIR_MIN_BLOCKS) k_step_pair
 // FP32 pipe, one instruction stream for every unit (the output sink alone
 // tells plain units, 64 fluid cells without wall links, from the others).
 //
-// Measured per step, chunk kernel and this one: Re 6500 nozzle 446 -> 370 us
-// (4.22 TB/s of algorithmic bytes; with axial averages 553 -> 497), Re 3500
-// nozzle 151 -> 134 us, periodic 256^3 501 -> 369 us (4.91 TB/s).  Two stages
-// and 4 blocks of 4 warps per SM: 3 blocks take 379 us on the Re 6500 nozzle, a
-// third stage changes nothing.  The moments and lines in fewer operations (250
-// a cell pair instead of 320) took 336 us, in other roundings (see Rounds).
+// Measured per step, chunk kernel and this one: Re 6500 nozzle 446 -> 354 us
+// (4.42 TB/s of algorithmic bytes; with axial averages 553 -> 486), Re 3500
+// nozzle 151 -> 127 us, periodic 256^3 501 -> 361 us (5.02 TB/s).  Two stages
+// and 4 blocks of 4 warps per SM: 3 blocks take 6 % longer on the Re 6500
+// nozzle, a third stage changes nothing.  The moments and lines in fewer
+// operations (250 a cell pair instead of 320) took 336 us, in other roundings
+// (see Rounds).
 // Steps that sample full statistics take the chunk kernel, whose 32 cells a
 // warp touch each accumulator's sectors at once: 503 us against 627 on the Re
 // 3500 nozzle.

@@ -142,12 +142,13 @@ constexpr int UNIT_NB = 7;  // first of the nine neighbour bases in a record
 constexpr int UNIT_HI_SHIFT = 8;
 constexpr int UNIT_PLAIN = 1, UNIT_WRAP = 2, UNIT_PLAIN_SHIFT = 8;
 // The staged kernel takes over from the chunk kernel at this many units per
-// resident warp (about 2 M cells): its warps start and end on atomics of one
-// address, a few us a launch.  Staged against chunk, us a step: nozzles of 1.4 /
-// 1.8 / 2.3 / 2.9 / 3.5 M cells (9 / 12 / 16 / 20 / 25 rounds) 61 / 73 / 84 / 98 /
-// 110 against 54 / 68 / 82 / 104 / 121, periodic boxes of 104^3 / 128^3 / 144^3 /
-// 160^3 (9 / 13.5 / 26 / 32 rounds) 49 / 63 / 100 / 123 against 51 / 72 / 98 / 132.
-constexpr int STAGE_ROUNDS = 13;
+// resident warp (about 1.5 M cells): its warps start and end on atomics of one
+// address, a few us a launch.  Staged against chunk, us a step: nozzles of 1.0 /
+// 1.4 / 1.8 / 2.3 / 2.9 / 3.5 M cells (7 / 9 / 12 / 16 / 20 / 25 rounds) 45 / 55 /
+// 65 / 80 / 94 / 105 against 42 / 54 / 68 / 82 / 104 / 121, periodic boxes of 96^3
+// / 104^3 / 112^3 / 128^3 / 160^3 (7.6 / 9 / 10 / 13.5 / 32 rounds) 39 / 48 / 50 /
+// 61 / 119 against 35 / 51 / 51 / 72 / 132.
+constexpr int STAGE_ROUNDS = 10;
 std::vector<int32_t> build_units(const std::vector<int2> &chunks, const std::vector<int32_t> &row_nb,
                                  const std::vector<uint32_t> &mask, int n_row, bool periodic_row);
 
