@@ -263,8 +263,8 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int32_t layout);
 /* Enqueue n >= 0 time steps on the context stream (asynchronous).  Each step
  * is the fluid kernel (FP32: one warp per tile of up to 32 cells of a row;
  * FP16S from about 1.5 million cells: one thread per two cells; else one thread
- * per cell) on the context's stream, and the inlet/outlet and interpolated-wall kernels on the second
- * stream beside it; they read the same input and write disjoint outputs, so
+ * per cell) on the context's stream, and the inlet/outlet and
+ * interpolated-wall kernels on the second stream beside it; they read the same input and write disjoint outputs, so
  * their order changes no result.  The health check and the statistics
  * sampling ride on these kernels when due.
  * Runs of steps that go in one launch (see lbm_kernel_launches) wait at a
@@ -278,8 +278,8 @@ lbm_status lbm_get_populations(lbm_ctx *ctx, double *f, int32_t layout);
 lbm_status lbm_step(lbm_ctx *ctx, int64_t n);
 
 /* Wait for the stream; report a deferred LBM_ERR_UNSTABLE (a health check saw
- * a non-finite value), LBM_ERR_TIMEOUT or LBM_ERR_CUDA.  The unstable flag stays set until the
- * next init call. */
+ * a non-finite value), LBM_ERR_TIMEOUT or LBM_ERR_CUDA.  The unstable flag
+ * stays set until the next init call. */
 lbm_status lbm_sync(lbm_ctx *ctx);
 
 /* Number of steps taken since the last init. */

@@ -351,8 +351,12 @@ int partial_capacity(const lbm_ctx *c, int64_t n_wnodes) {
 // Transfers of per-cell arrays in the active order run in TRANSFER_PARTS parts
 // beside the kernel that reads or writes them, from this many cells on: the
 // copies go on the context's second stream, each part's kernel after (or
-// before) its copy.  On the 256^3 vortex (537 MB each way), moments 5.8 ->
-// 3.8 ms and fields 7.3 -> 5.6 ms; below, the extra launches cost more than the overlap gives.
+// before) its copy.  In one part -> in four, page-locked arrays, FP32 boxes of
+// 64^3 / 80^3 / 96^3 / 104^3 / 128^3 / 160^3 / 224^3: fields 171 -> 205, 290 ->
+// 314, 460 -> 391, 565 -> 468, 998 -> 807, 1 877 -> 1 465 and 4 980 -> 3 821 us,
+// moments 132 -> 140, 232 -> 225, 378 -> 319, 474 -> 367, 832 -> 617, 1 579 ->
+// 1 103 and 4 172 -> 2 851 us.  The sides meet near 0.6 million cells; the line
+// lies above, where both transfers gain clearly.
 constexpr int TRANSFER_PARTS = 4;
 constexpr int64_t TRANSFER_SPLIT = 1 << 20;
 

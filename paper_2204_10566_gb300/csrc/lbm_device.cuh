@@ -13,7 +13,8 @@
 // contiguous along the lattice's longer axis), structure-of-arrays
 // populations stored as deviations from the lattice weights; one warp per
 // tile of up to 32 cells of a row (FP32), one thread per two cells over staged
-// copies (FP16S, larger lattices) or one thread per cell (smaller FP16S, FP64), with the inlet/outlet nodes and the interpolated-wall cells in
+// copies (FP16S, larger lattices) or one thread per cell (smaller FP16S,
+// FP64), with the inlet/outlet nodes and the interpolated-wall cells in
 // kernels of their own on a second stream.  Every pull source has a
 // slot (wall links read a ghost slot the cell filled with its reflected
 // population in the previous step), so the gather is 27 unconditional
