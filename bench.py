@@ -39,9 +39,9 @@ LINK_WORD_BYTES = 4
 
 
 # FP64 flops per fluid-cell update of the step kernel (130 additions, 44
-# products, 80 fused pairs: 254 instructions).  The FP64 kernel keeps the FP64
-# pipe ~87 % busy, so its roofline is that pipe, not HBM.
-FP64_FLOPS_PER_CELL = 334
+# products, 82 fused pairs: 256 instructions).  The FP64 kernel keeps the FP64
+# pipe ~86 % busy, so its roofline is that pipe, not HBM.
+FP64_FLOPS_PER_CELL = 338
 FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 rate
 
 
